@@ -34,6 +34,30 @@ vpp_status fail(vpp_status s, const char* fmt, ...) {
 
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
+// The status word of a call that launches nothing.
+vpp_status zero_status(int32_t* status, cudaStream_t stream) {
+    if (status && cudaMemsetAsync(status, 0, sizeof(int32_t), stream) != cudaSuccess)
+        return fail(VPP_ERR_CUDA, "memset status: %s", cudaGetErrorString(cudaGetLastError()));
+    return VPP_OK;
+}
+
+// Launch with programmatic stream serialization: the kernel may start (and set itself up) while its predecessor in the
+// stream still runs, and waits for it (griddepcontrol.wait) before it touches memory.
+template <typename... Params, typename... Args>
+cudaError_t launch(void (*kernel)(Params...), unsigned blocks, unsigned threads, size_t smem, cudaStream_t stream, Args... args) {
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
+}
+
 // ---- device facts, cached per device -------------------------------------------------------------
 struct DeviceInfo {
     bool ready = false;
@@ -316,7 +340,8 @@ int heads_per_item(const vpp_chunk_attn_args* a, Family fam) {
     return pairs_two_heads(a) ? 2 : 1;
 }
 
-using MergeKernel = void (*)(const float*, const float*, int, long long, int, int, const int32_t*, __nv_bfloat16*, float*);
+using MergeKernel = void (*)(const float*, const float*, int, long long, int, int, const int32_t*, const vpp::WorkHeader*, __nv_bfloat16*,
+                             float*);
 // The kernel and the grid for a merge of `splits` partials of total_q x num_q_heads rows of head_dim_v features.
 MergeKernel pick_merge_kernel(int splits, long long total_q, int num_q_heads, int head_dim_v, int sms, unsigned* blocks) {
     const long long pairs = total_q * num_q_heads;
@@ -435,11 +460,8 @@ vpp_status run_chunk_attn(const vpp_chunk_attn_args* a, vpp_stream_t stream_, co
 
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);
     g_launches = 0;
-    if (a->status) {
-        if (cudaMemsetAsync(a->status, 0, sizeof(int32_t), stream) != cudaSuccess)
-            return fail(VPP_ERR_CUDA, "memset status: %s", cudaGetErrorString(cudaGetLastError()));
-    }
-    if (a->total_q == 0 || a->num_reqs == 0) return VPP_OK;
+    if (a->total_q == 0 || a->num_reqs == 0) return zero_status(a->status, stream);
+    // (otherwise the attention kernel writes the status word: a memset node and its gap cost a short launch 4 us)
     if (fam == Family::kMla576 && !mla_kernel_available())
         return fail(VPP_ERR_UNSUPPORTED, "the absorbed-MLA kernel needs clusters of two SMs");
 
@@ -555,14 +577,21 @@ vpp_status run_chunk_attn(const vpp_chunk_attn_args* a, vpp_stream_t stream_, co
     pp.row_splits = row_splits;
     pp.q_start = row_splits + a->total_q;
     pp.tile_start = pp.q_start + a->num_reqs + 1;
-    pp.status = a->status;
     {
         // small launches (a short chunk, a small decode batch) take the one-warp decomposition
         const long long tiles_ub = (a->total_q + pp.tile_m - 1) / pp.tile_m + a->num_reqs;
-        if (a->num_reqs <= vpp::kPrepSmallMax && tiles_ub <= vpp::kPrepSmallMax)
-            vpp::prep_small_kernel<<<1, 32, 0, stream>>>(pp);
-        else
-            vpp::prep_kernel<<<1, vpp::kPrepThreads, 0, stream>>>(pp);
+        const bool small = a->num_reqs <= vpp::kPrepSmallMax && tiles_ub <= vpp::kPrepSmallMax;
+        const unsigned threads = small ? vpp::kPrepSmallThreads : vpp::kPrepThreads;
+        // blocks that check the block table: one per 4 entries a thread can have in flight, at most kMaxCheckers
+        long long checkers = 0;
+        if (paged) {
+            const long long entries = static_cast<long long>(a->num_reqs) * a->max_blocks_per_req;
+            checkers = (entries + 4 * threads - 1) / (4 * threads);
+            if (checkers > vpp::kMaxCheckers) checkers = vpp::kMaxCheckers;
+        }
+        const cudaError_t pe = launch(small ? vpp::prep_small_kernel : vpp::prep_kernel, static_cast<unsigned>(1 + checkers), threads,
+                                      0, stream, pp);
+        if (pe != cudaSuccess) return fail(VPP_ERR_CUDA, "work decomposition launch: %s", cudaGetErrorString(pe));
     }
     ++g_launches;
 
@@ -591,28 +620,18 @@ vpp_status run_chunk_attn(const vpp_chunk_attn_args* a, vpp_stream_t stream_, co
     if (mla_pair) {
         auto kern = vpp::attn_mla2_kernel;
         ce = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, vpp::kMla2SmemBytes);
-        if (ce == cudaSuccess) kern<<<(sms / 2) * 2, vpp::kMla2Threads, vpp::kMla2SmemBytes, stream>>>(tm_q9, tm_qh9, tm_k93, tm_k92, tm_k, ap, box_rows);
+        if (ce == cudaSuccess)
+            ce = launch(kern, static_cast<unsigned>((sms / 2) * 2), vpp::kMla2Threads, vpp::kMla2SmemBytes, stream, tm_q9, tm_qh9, tm_k93,
+                        tm_k92, tm_k, ap, box_rows);
     } else {
         // a second producer warp for launches bound by the arrival of K/V: pages smaller than a KV tile, batches of decode rows
         const bool v_warp = box_rows < vpp::kTileN || a->total_q <= a->num_reqs;
         auto kern = pairs_two_heads(a) ? (v_warp ? vpp::attn128_ws_kernel<false, true> : vpp::attn128_ws_kernel<false, false>)
                                        : (v_warp ? vpp::attn128_ws_kernel<true, true> : vpp::attn128_ws_kernel<true, false>);
         ce = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, vpp::kWsSmemBytes);
-        if (ce == cudaSuccess) {
-            // programmatic dependent launch: set-up overlaps the work-decomposition kernel (the kernel waits for it
-            // before it reads the work list)
-            cudaLaunchAttribute attr{};
-            attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-            attr.val.programmaticStreamSerializationAllowed = 1;
-            cudaLaunchConfig_t cfg{};
-            cfg.gridDim = dim3(sms);
-            cfg.blockDim = dim3(vpp::kWsThreads);
-            cfg.dynamicSmemBytes = vpp::kWsSmemBytes;
-            cfg.stream = stream;
-            cfg.attrs = &attr;
-            cfg.numAttrs = 1;
-            ce = cudaLaunchKernelEx(&cfg, kern, tm_q, tm_k, tm_v, tm_q2, tm_k2, tm_v2, tm_qh, ap, box_rows);
-        }
+        if (ce == cudaSuccess)
+            ce = launch(kern, static_cast<unsigned>(sms), vpp::kWsThreads, vpp::kWsSmemBytes, stream, tm_q, tm_k, tm_v, tm_q2, tm_k2, tm_v2,
+                        tm_qh, ap, box_rows);
     }
     if (ce != cudaSuccess) return fail(VPP_ERR_CUDA, "attention kernel attributes: %s", cudaGetErrorString(ce));
     ++g_launches;
@@ -621,20 +640,8 @@ vpp_status run_chunk_attn(const vpp_chunk_attn_args* a, vpp_stream_t stream_, co
     if (L.splits > 1) {
         unsigned blocks = 1;
         const MergeKernel mk = pick_merge_kernel(L.splits, a->total_q, a->num_q_heads, a->head_dim_v, sms, &blocks);
-        cudaLaunchAttribute attr{};
-        attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr.val.programmaticStreamSerializationAllowed = 1;
-        cudaLaunchConfig_t cfg{};
-        cfg.gridDim = dim3(blocks);
-        cfg.blockDim = dim3(vpp::kMergeThreads);
-        cfg.stream = stream;
-        cfg.attrs = &attr;
-        cfg.numAttrs = 1;
-        ce = cudaLaunchKernelEx(&cfg, mk, static_cast<const float*>(ap.o_parts),
-                                static_cast<const float*>(ap.lse_parts), static_cast<int>(L.splits),
-                                static_cast<long long>(a->total_q), static_cast<int>(a->num_q_heads),
-                                static_cast<int>(a->head_dim_v), static_cast<const int32_t*>(row_splits),
-                                static_cast<__nv_bfloat16*>(a->out), a->lse);
+        ce = launch(mk, blocks, vpp::kMergeThreads, 0, stream, ap.o_parts, ap.lse_parts, L.splits, a->total_q, a->num_q_heads,
+                    a->head_dim_v, row_splits, pp.header, static_cast<__nv_bfloat16*>(a->out), a->lse);
         if (ce != cudaSuccess) return fail(VPP_ERR_CUDA, "merge launch: %s", cudaGetErrorString(ce));
         ++g_launches;
     }
@@ -658,9 +665,8 @@ vpp_status vpp_lse_merge(const float* o_parts, const float* lse_parts, int32_t n
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);
     unsigned blocks = 1;
     const MergeKernel mk = pick_merge_kernel(num_splits, total_q, num_q_heads, head_dim_v, sm_count_or_default(), &blocks);
-    mk<<<blocks, vpp::kMergeThreads, 0, stream>>>(o_parts, lse_parts, num_splits, total_q, num_q_heads, head_dim_v, nullptr,
-                                                  static_cast<__nv_bfloat16*>(out), lse);
-    cudaError_t ce = cudaGetLastError();
+    const cudaError_t ce = launch(mk, blocks, vpp::kMergeThreads, 0, stream, o_parts, lse_parts, num_splits, total_q, num_q_heads,
+                                  head_dim_v, nullptr, nullptr, static_cast<__nv_bfloat16*>(out), lse);
     if (ce != cudaSuccess) return fail(VPP_ERR_CUDA, "merge launch: %s", cudaGetErrorString(ce));
     return VPP_OK;
 }

@@ -268,13 +268,17 @@ attn_mla2_kernel(const __grid_constant__ CUtensorMap tm_q1, const __grid_constan
     tc_fence_after();
     const uint32_t tmem_base = *s_tmem;
 
-    const int num_units = p.header_ro->num_units;
+    pdl_wait();                  // the work list comes from the work-decomposition kernel launched just before
+    pdl_launch_dependents();
+    const int error = launch_error(p.header_ro);
+    if (blockIdx.x == 0 && tid == 0 && p.status) *p.status = error;
+    const int num_units = error ? 0 : p.header_ro->num_units;
     const int num_pairs = gridDim.x >> 1;
     const int pair = blockIdx.x >> 1;
     // Items: (unit, q-head) for the units of several rows, then one item per single-token unit (the end of the list):
     // those run "packed" -- the q-heads are the rows of the tile (64 per CTA; they all share the one latent kv-head), so
     // the cache is streamed once per token instead of once per head.
-    const int num_packed = p.num_q_heads <= 2 * kMla2Rows ? p.header_ro->num_single : 0;
+    const int num_packed = p.num_q_heads <= 2 * kMla2Rows && !error ? p.header_ro->num_single : 0;
     const int num_normal = num_units - num_packed;
     const int normal_items = num_normal * p.num_q_heads;
     const int total_items = normal_items + num_packed;

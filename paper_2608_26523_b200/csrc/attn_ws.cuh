@@ -211,11 +211,13 @@ attn128_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
 
     pdl_wait();                  // the work list comes from the work-decomposition kernel launched just before
     pdl_launch_dependents();     // (the merge kernel, if any, waits for this grid to finish in the same way)
-    const int num_units = p.header_ro->num_units;
+    const int error = launch_error(p.header_ro);
+    if (blockIdx.x == 0 && tid == 0 && p.status) *p.status = error;
+    const int num_units = error ? 0 : p.header_ro->num_units;
     const int G = p.num_q_heads / p.num_kv_heads;
     // Items: (unit, pair of q-heads) for the units of several rows, then (unit, kv-head) for the single-token units at the
     // end of the list, which run packed when a kv-head's group fits a tile.
-    const int num_packed = G <= kTileM ? p.header_ro->num_single : 0;
+    const int num_packed = G <= kTileM && !error ? p.header_ro->num_single : 0;
     const int num_normal = num_units - num_packed;
     const int heads_per_item = same_head ? 1 : 2;
     const int normal_items = num_normal * (p.num_q_heads / heads_per_item);

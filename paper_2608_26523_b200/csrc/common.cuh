@@ -21,13 +21,25 @@ struct __align__(16) WorkUnit {
     int32_t kv_len;     // prefix_len + chunk_len of the request: keys at or beyond it do not exist
 };
 
+constexpr int kMaxCheckers = 8;   // blocks of the work-decomposition kernel that check the block table
+
 // Head of the workspace; written by the work-decomposition kernel.
 struct WorkHeader {
-    int32_t num_units;  // units in the sorted list
-    int32_t counter;    // persistent-kernel work counter
-    int32_t error;      // VPP_DEV_* (0 = ok); when nonzero num_units is 0
-    int32_t num_single; // the last num_single units of the list are single-token units (rows == 1)
+    int32_t num_units;    // units in the sorted list
+    int32_t counter;      // persistent-kernel work counter
+    int32_t error;        // VPP_DEV_* (0 = ok) of the lengths
+    int32_t num_single;   // the last num_single units of the list are single-token units (rows == 1)
+    int32_t num_checkers; // blocks that checked a part of the block table
+    int32_t bad_table[kMaxCheckers];   // one word each: VPP_DEV_BAD_BLOCK if it found an entry out of range, else 0
 };
+
+// What the checks of the work decomposition found (0 = ok): the kernels after it do nothing when it is not 0.
+__device__ __forceinline__ int launch_error(const WorkHeader* h) {
+    int e = h->error;
+    const int n = h->num_checkers;
+    for (int i = 0; i < n && e == 0; ++i) e = h->bad_table[i];
+    return e;
+}
 
 struct WorkspaceLayout {
     size_t header;      // WorkHeader

@@ -11,6 +11,9 @@
 #include <cstdint>
 #include <cuda_bf16.h>
 
+#include "common.cuh"
+#include "ptx.cuh"
+
 namespace vpp {
 
 constexpr int kMergeThreads = 256;
@@ -19,13 +22,15 @@ constexpr int kMergeSmallMax = 8;   // split counts up to this take the shuffle-
 
 // row_splits: optional int32 per query row = number of partials to merge for that row; rows with
 // fewer than 2 were written in final form by the attention kernel and are skipped.
-// When null, every row merges exactly num_splits partials.
+// When null, every row merges exactly num_splits partials.  header: null, or the launch whose checks must have passed.
 template <int kMergePairs /* pairs per trip */, int kMergeBatch /* partial rows in flight per lane and pair */>
 __global__ void __launch_bounds__(kMergeThreads, 3)
 lse_merge_kernel(const float* __restrict__ o_parts, const float* __restrict__ lse_parts, int num_splits,
                  long long total_q, int num_q_heads, int head_dim_v, const int32_t* __restrict__ row_splits,
-                 __nv_bfloat16* __restrict__ out, float* __restrict__ lse) {
-    asm volatile("griddepcontrol.wait;" ::: "memory");   // partials come from the attention kernel launched just before
+                 const WorkHeader* header, __nv_bfloat16* __restrict__ out, float* __restrict__ lse) {
+    pdl_launch_dependents();
+    pdl_wait();   // partials come from the attention kernel launched just before
+    if (header != nullptr && launch_error(header) != 0) return;   // (nothing was computed and row_splits was not written)
     const long long n_pairs = total_q * num_q_heads;
     const int lane = threadIdx.x & 31;
     const long long warps_total = static_cast<long long>(gridDim.x) * (kMergeThreads / 32);
@@ -124,8 +129,10 @@ template <int kSMax, int kPieces>
 __global__ void __launch_bounds__(kMergeThreads, 3)
 lse_merge_small_kernel(const float* __restrict__ o_parts, const float* __restrict__ lse_parts, int num_splits,
                        long long total_q, int num_q_heads, int head_dim_v, const int32_t* __restrict__ row_splits,
-                       __nv_bfloat16* __restrict__ out, float* __restrict__ lse) {
-    asm volatile("griddepcontrol.wait;" ::: "memory");   // partials come from the attention kernel launched just before
+                       const WorkHeader* header, __nv_bfloat16* __restrict__ out, float* __restrict__ lse) {
+    pdl_launch_dependents();
+    pdl_wait();   // partials come from the attention kernel launched just before
+    if (header != nullptr && launch_error(header) != 0) return;   // (nothing was computed and row_splits was not written)
     const long long n_pairs = total_q * num_q_heads;
     const uint32_t per_row = static_cast<uint32_t>(head_dim_v) >> 2;            // 16-byte pieces per output row
     const uint32_t n_pieces = static_cast<uint32_t>(n_pairs) * per_row;
