@@ -679,9 +679,7 @@ vpp_status vpp_kv_append(const vpp_kv_append_args* a, vpp_stream_t stream_) {
     if (a->head_dim_qk % 8 || a->head_dim_v % 8) return fail(VPP_ERR_UNSUPPORTED, "head dims must be multiples of 8");
     if (a->num_reqs > vpp::kAppendMaxReqs) return fail(VPP_ERR_UNSUPPORTED, "at most %d requests", vpp::kAppendMaxReqs);
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);
-    if (a->status && cudaMemsetAsync(a->status, 0, sizeof(int32_t), stream) != cudaSuccess)
-        return fail(VPP_ERR_CUDA, "memset status: %s", cudaGetErrorString(cudaGetLastError()));
-    if (a->total_q == 0 || a->num_reqs == 0) return VPP_OK;
+    if (a->total_q == 0 || a->num_reqs == 0) return zero_status(a->status, stream);
     if (!a->k_new || !a->k_cache || !a->prefix_len || !a->chunk_len)
         return fail(VPP_ERR_INVALID_ARG, "k_new, k_cache, prefix_len and chunk_len must be non-null");
     if (a->v_new && !a->v_cache) return fail(VPP_ERR_INVALID_ARG, "v_new given without v_cache");
@@ -725,13 +723,15 @@ vpp_status vpp_kv_append(const vpp_kv_append_args* a, vpp_stream_t stream_) {
     p.k_vecs = a->head_dim_qk / 8;
     p.v_vecs = a->v_new ? a->head_dim_v / 8 : 0;
     p.status = a->status;
-    const int rows_per_block = vpp::kAppendThreads / 32;
-    long long blocks = (static_cast<long long>(a->total_q) + rows_per_block - 1) / rows_per_block;
+    const int vecs = p.num_kv_heads * (p.k_vecs + p.v_vecs), warps_per_block = vpp::kAppendThreads / 32;
+    const long long tasks = static_cast<long long>(a->total_q) * ((vecs + vpp::kAppendPiece - 1) / vpp::kAppendPiece);
+    long long blocks = (tasks + warps_per_block - 1) / warps_per_block;
     const long long cap = 16ll * sm_count_or_default();
     if (blocks > cap) blocks = cap;
     const size_t smem = sizeof(int32_t) * (static_cast<size_t>(a->num_reqs) + 1);
-    vpp::kv_append_kernel<<<static_cast<unsigned>(blocks), vpp::kAppendThreads, smem, stream>>>(p);
-    cudaError_t ce = cudaGetLastError();
+    const int copy_blocks = static_cast<int>(blocks);
+    const cudaError_t ce = launch(vpp::kv_append_kernel, static_cast<unsigned>(copy_blocks + (a->status ? 1 : 0)), vpp::kAppendThreads, smem,
+                                  stream, p, copy_blocks);
     if (ce != cudaSuccess) return fail(VPP_ERR_CUDA, "append launch: %s", cudaGetErrorString(ce));
     return VPP_OK;
 }

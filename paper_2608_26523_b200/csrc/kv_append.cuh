@@ -2,16 +2,22 @@
 // of their request (the step that precedes the attention of the same chunk; the paper's chunked-prefill section).
 // Pure data movement, HBM-bound: every byte is read once and written once.
 //
-// One warp per token row.  Lane 0 finds the request of the row (binary search in the exclusive scan of chunk_len that
-// every block builds in shared memory) and its page; then the lanes copy the row's (kv-head, 16-byte vector) units,
-// all loads of a trip issued before the first store (up to kAppendUnroll 16-byte loads in flight per lane).
+// A warp takes one piece of a token row at a time: up to kAppendPiece 16-byte vectors of the row's (kv-head, vector)
+// units, a 4 KB row of eight kv-heads whole.  Its loads are all issued first -- kAppendUnroll in flight per lane -- and the
+// row's destination is looked up while they are in flight: lane 0 finds the request (binary search in the exclusive scan
+// of chunk_len that every block builds in shared memory) and the page.  The block after the copying ones checks the
+// lengths and pages of the whole launch and writes *status, so that the call needs no memset before it.
+// 134 MB (16384 rows of eight kv-heads): 28.0 -> 24.4 us a call, 5.5 TB/s; the rest to the copy rate (20.6 us) is one launch.
 #pragma once
 #include <cstdint>
+
+#include "ptx.cuh"
 
 namespace vpp {
 
 constexpr int kAppendThreads = 256;
-constexpr int kAppendUnroll = 4;
+constexpr int kAppendUnroll = 8;
+constexpr int kAppendPiece = 32 * kAppendUnroll;   // 16-byte vectors a warp moves at a time
 constexpr int kAppendMaxReqs = 8192;   // the scan of chunk_len lives in shared memory (32 KB + 4)
 
 struct AppendParams {
@@ -39,25 +45,29 @@ __device__ __forceinline__ uint4 ld_stream(const uint4* p) {
     return v;
 }
 
-__global__ void __launch_bounds__(kAppendThreads) kv_append_kernel(const AppendParams p) {
-    extern __shared__ int32_t cu[];   // cu[r] = rows before request r; cu[num_reqs] = total
+// Exclusive scan of chunk_len into cu[0 .. num_reqs] (shared memory); true if the lengths describe the launch.
+__device__ __forceinline__ bool append_scan(const AppendParams& p, int32_t* cu) {
     __shared__ int s_bad;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tid = threadIdx.x, lane = tid & 31;
     if (tid == 0) s_bad = 0;
     __syncthreads();
-    if (warp == 0) {
+    bool bad = false;
+    for (int r = tid; r < p.num_reqs; r += kAppendThreads) {   // (all loads at once, then the scan from shared memory)
+        int c = p.chunk_len[r];
+        const int pre = p.prefix_len[r];
+        if (c < 0 || pre < 0 || static_cast<long long>(pre) + c > p.capacity) {
+            bad = true;
+            c = 0;
+        }
+        cu[r] = c;
+    }
+    if (bad) s_bad = 1;
+    __syncthreads();
+    if (tid < 32) {
         int carry = 0;
         for (int base = 0; base < p.num_reqs; base += 32) {
             const int r = base + lane;
-            int c = 0;
-            if (r < p.num_reqs) {
-                c = p.chunk_len[r];
-                const int pre = p.prefix_len[r];
-                if (c < 0 || pre < 0 || static_cast<long long>(pre) + c > p.capacity) {
-                    s_bad = 1;
-                    c = 0;
-                }
-            }
+            const int c = r < p.num_reqs ? cu[r] : 0;
             int x = c;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
@@ -70,14 +80,56 @@ __global__ void __launch_bounds__(kAppendThreads) kv_append_kernel(const AppendP
         if (lane == 0) cu[p.num_reqs] = carry;
     }
     __syncthreads();
-    if (s_bad || cu[p.num_reqs] != p.total_q) {
-        // lengths that do not describe this launch: write nothing
-        if (tid == 0 && blockIdx.x == 0 && p.status) atomicCAS(p.status, 0, 1 /* VPP_DEV_BAD_LENGTHS */);
+    return !s_bad && cu[p.num_reqs] == p.total_q;
+}
+
+// The verdict on the launch (one block): lengths, and the pages of every row.
+__device__ __forceinline__ void append_status(const AppendParams& p, bool lengths_ok) {
+    bool bad = false;
+    if (lengths_ok && p.block_table != nullptr) {
+        const int per_req = p.num_reqs < kAppendThreads ? kAppendThreads / p.num_reqs : 1;   // threads that share a request
+        const int groups = kAppendThreads / per_req, grp = threadIdx.x / per_req, part = threadIdx.x % per_req;
+        for (int r = grp; r < p.num_reqs && grp < groups; r += groups) {
+            const int pre = p.prefix_len[r], c = p.chunk_len[r];
+            if (c == 0) continue;
+            const int32_t* row = p.block_table + static_cast<long long>(r) * p.max_blocks_per_req;
+            const int last = (pre + c - 1) >> p.block_shift;
+            for (int b = (pre >> p.block_shift) + part; b <= last; b += per_req) {
+                const int e = __ldg(row + b);
+                bad |= e < 0 || e >= p.num_blocks;
+            }
+        }
+    }
+    const int any = __syncthreads_or(bad);
+    if (threadIdx.x == 0) *p.status = !lengths_ok ? 1 /* VPP_DEV_BAD_LENGTHS */ : any ? 2 /* VPP_DEV_BAD_BLOCK */ : 0;
+}
+
+// The first copy_blocks blocks copy; the block after them, if there is one, writes the status.
+__global__ void __launch_bounds__(kAppendThreads) kv_append_kernel(const AppendParams p, const int copy_blocks) {
+    extern __shared__ int32_t cu[];   // cu[r] = rows before request r; cu[num_reqs] = total
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    pdl_launch_dependents();
+    pdl_wait();                       // the rows and the lengths may come from the kernel launched just before
+    const bool ok = append_scan(p, cu);
+    if (static_cast<int>(blockIdx.x) >= copy_blocks) {
+        append_status(p, ok);
         return;
     }
+    if (!ok) return;                  // lengths that do not describe this launch: write nothing
     const int units_k = p.num_kv_heads * p.k_vecs, units = units_k + p.num_kv_heads * p.v_vecs;
-    const int warps_total = gridDim.x * (kAppendThreads / 32);
-    for (int row = blockIdx.x * (kAppendThreads / 32) + warp; row < p.total_q; row += warps_total) {
+    const int pieces = (units + kAppendPiece - 1) / kAppendPiece;
+    const long long tasks = static_cast<long long>(p.total_q) * pieces, stride = copy_blocks * (kAppendThreads / 32);
+    for (long long task = blockIdx.x * (kAppendThreads / 32) + warp; task < tasks; task += stride) {
+        const int row = static_cast<int>(task / pieces);
+        const int u0 = static_cast<int>(task - static_cast<long long>(row) * pieces) * kAppendPiece + lane;
+        const uint4* k_src = p.k_new + static_cast<long long>(row) * units_k;
+        const uint4* v_src = p.v_new + static_cast<long long>(row) * (units - units_k);
+        uint4 v[kAppendUnroll];
+#pragma unroll
+        for (int i = 0; i < kAppendUnroll; ++i) {
+            const int u = u0 + 32 * i;
+            if (u < units) v[i] = ld_stream(u < units_k ? k_src + u : v_src + (u - units_k));
+        }
         long long blk = 0;
         int slot = 0;
         if (lane == 0) {
@@ -93,10 +145,7 @@ __global__ void __launch_bounds__(kAppendThreads) kv_append_kernel(const AppendP
             } else {
                 blk = p.block_table[static_cast<long long>(lo) * p.max_blocks_per_req + (pos >> p.block_shift)];
                 slot = pos & ((1 << p.block_shift) - 1);
-                if (blk < 0 || blk >= p.num_blocks) {
-                    if (p.status) atomicCAS(p.status, 0, 2 /* VPP_DEV_BAD_BLOCK */);
-                    blk = -1;
-                }
+                if (blk < 0 || blk >= p.num_blocks) blk = -1;
             }
         }
         blk = __shfl_sync(0xffffffffu, blk, 0);
@@ -104,26 +153,16 @@ __global__ void __launch_bounds__(kAppendThreads) kv_append_kernel(const AppendP
         if (blk < 0) continue;   // the row's page is not valid: skip the row
         uint8_t* k_dst = p.k_cache + blk * p.k_block_stride + slot * p.k_token_stride;
         uint8_t* v_dst = p.v_cache + blk * p.v_block_stride + slot * p.v_token_stride;
-        const uint4* k_src = p.k_new + static_cast<long long>(row) * units_k;
-        const uint4* v_src = p.v_new + static_cast<long long>(row) * (units - units_k);
-        for (int u0 = lane; u0 < units; u0 += 32 * kAppendUnroll) {
-            uint4 v[kAppendUnroll];
 #pragma unroll
-            for (int i = 0; i < kAppendUnroll; ++i) {
-                const int u = u0 + 32 * i;
-                if (u < units) v[i] = ld_stream(u < units_k ? k_src + u : v_src + (u - units_k));
-            }
-#pragma unroll
-            for (int i = 0; i < kAppendUnroll; ++i) {
-                const int u = u0 + 32 * i;
-                if (u >= units) continue;
-                if (u < units_k) {
-                    const int g = u / p.k_vecs, j = u - g * p.k_vecs;
-                    *reinterpret_cast<uint4*>(k_dst + g * p.k_head_stride + j * 16) = v[i];
-                } else {
-                    const int w = u - units_k, g = w / p.v_vecs, j = w - g * p.v_vecs;
-                    *reinterpret_cast<uint4*>(v_dst + g * p.v_head_stride + j * 16) = v[i];
-                }
+        for (int i = 0; i < kAppendUnroll; ++i) {
+            const int u = u0 + 32 * i;
+            if (u >= units) continue;
+            if (u < units_k) {
+                const int g = u / p.k_vecs, j = u - g * p.k_vecs;
+                *reinterpret_cast<uint4*>(k_dst + g * p.k_head_stride + j * 16) = v[i];
+            } else {
+                const int w = u - units_k, g = w / p.v_vecs, j = w - g * p.v_vecs;
+                *reinterpret_cast<uint4*>(v_dst + g * p.v_head_stride + j * 16) = v[i];
             }
         }
     }
