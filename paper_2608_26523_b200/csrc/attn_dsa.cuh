@@ -6,10 +6,12 @@
 // 64 per CTA of a 2-CTA cluster, exactly as in the packed single-token items of the dense pair kernel, from which the
 // MMA, softmax and barrier structure is taken.  What differs is the producer side: a KV tile is 128 listed rows that
 // lie anywhere in the cache, fetched with the gather form of the tensor copy (cp.async.bulk.tensor ... tile::gather4:
-// four rows of 64 columns per instruction, 128-byte swizzle applied on the way in).  A warp issues such copies one lane
-// after the other at ~75-130 clk apiece, but warps issue independently, so the 272 copies of a tile are spread over ten
-// producer warps, two per hand-back group, each issuing one instruction per tile.  (16-byte cp.async copies by the same
-// warps were measured too: 385 TFLOP/s -- a warp keeps too few of them in flight.)
+// four rows of 64 columns per instruction, 128-byte swizzle applied on the way in).  What bounds the kernel is the rate at
+// which these copies are issued: a warp issues them one lane after the other at ~180 clk apiece, warps issue independently,
+// an SM sustains one per ~10 clk.  A tile and CTA takes 272 (K: 64 keys x 9 slabs, V: 128 keys x 4 slabs, four rows each),
+// so they are spread over 17 producer warps of 16 lanes, one slab of 64 keys each, and the register file is split
+// unevenly (setmaxnreg) to make room for them.  2048 tokens with lists of
+// 2048 at prefix 65536: 10 producer warps of 24 and 32 lanes 1458 us, these 1362 us.
 // Entries that do not take part are pointed at the token's own cache row (always present and finite) and masked out
 // of the softmax through a 128-bit validity mask that warp 0 publishes per tile.  The cost per token does not depend on
 // the prefix length: the flat latency curve the paper says weakens its linear-growth assumption.
@@ -20,7 +22,13 @@
 
 namespace vpp {
 
-constexpr int kDsaThreads = 512;   // 16 warps: see the role list in the kernel
+constexpr int kDsaThreads = 768;   // 24 warps: see the role list in the kernel
+// Registers per thread: 80 at launch; after the roles split the five warpgroups of producers and issuers keep kDsaRegsLow
+// and the softmax warpgroup takes kDsaRegsHigh out of what they returned.
+constexpr int kDsaRegsLow = 64, kDsaRegsHigh = 152;
+static_assert(5 * kDsaRegsLow + kDsaRegsHigh <= 6 * 80 && kDsaRegsLow % 8 == 0 && kDsaRegsHigh % 8 == 0, "register budget");
+constexpr int kDsaKWarps = 9, kDsaVWarps = 8;   // one per (hand-back group, slab) of a CTA's 64 keys / (key half, slab)
+static_assert(kDsaKWarps == kMlaSlabs && kDsaVWarps == 2 * kMla2VChunks, "a producer warp per slab");
 constexpr int kDsaMaxReqs = 8192;
 constexpr int kDsaPrepThreads = 256;
 
@@ -107,9 +115,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kDsaThreads, 1)
 dsa_attn_kernel(const __grid_constant__ CUtensorMap tm_qh, const __grid_constant__ CUtensorMap tm_rows, const DsaParams p) {
     // tm_qh:   (64 cols, Hq heads, 9 slabs, T tokens) box (64, 64, 9, 1) -- 64 q-heads of one token, all slabs (heads past Hq read as zero)
     // tm_rows: (576 cols, cache rows) box (64, 1), gather mode: four listed rows of one 64-column slab per copy
-    // Per CTA, 16 warps: warps 0, 6, 8-11 K producers (two per hand-back group; warp 0 also Q and the validity masks),
-    // warps 12-15 V producers (two per group), warp 1 / warp 7 of the leader: one thread each issuing the score and
-    // the P V MMAs of the pair, warps 2-5 softmax.
+    // Per CTA, 24 warps: warp 0 the validity masks (and tensor-memory allocation), warp 1 / warp 2 of the leader: one
+    // thread each issuing the score and the P V MMAs of the pair, warps 4-7 softmax, warps 3 and 8-15 K producers (warp 15 also Q), warps
+    // 16-23 V producers.
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t* gen_base = smem_raw + (smem_base - smem_u32(smem_raw));
@@ -197,97 +205,99 @@ dsa_attn_kernel(const __grid_constant__ CUtensorMap tm_qh, const __grid_constant
 #pragma unroll
         for (int i = 0; i < 4; ++i) e[i] = (k0 + i < p.topk) ? __ldg(src + i) : -1;
     };
-    // rows to fetch for these entries (those that do not take part fetch the token's own row) and which take part
-    auto rows_of = [&](int req, int pos, int self_row, const int (&e)[4], int (&r)[4]) -> uint32_t {
-        uint32_t bits = 0;
+    // rows to fetch for these entries (those that do not take part fetch the token's own row)
+    auto rows_of = [&](int req, int pos, int self_row, const int (&e)[4], int (&r)[4]) {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const bool v = e[i] >= 0 && e[i] <= pos;
-            r[i] = v ? row_of(req, e[i]) : self_row;
-            bits |= (v ? 1u : 0u) << i;
-        }
-        return bits;
+        for (int i = 0; i < 4; ++i) r[i] = e[i] >= 0 && e[i] <= pos ? row_of(req, e[i]) : self_row;
     };
 
     const uint32_t pair_q_full = mapa_u32(bar_q_full, 0), pair_k_full = mapa_u32(bar_k_full, 0),
                    pair_v_full = mapa_u32(bar_v_full, 0);
 
-    if (warp == 0 || warp == 6 || (warp >= 8 && warp <= 11)) {
-        // ===================================== Q / K producers =====================================
-        // A warp issues gather copies one lane after the other, ~75-130 clk apiece, but warps issue independently
-        // (measured: 8 warps x 16 lanes reach one copy per 13-16 clk per SM).  So every hand-back group has warps of its
-        // own and a warp issues ONE instruction per tile as soon as its group is free: K group g (slabs 3 g .. 3 g + 2 of
-        // this CTA's 64 keys = 48 copies) belongs to warps kw = 2 g and 2 g + 1, which take 8 quads of four keys each;
-        // lane = 8 * (slab within the group) + quad: 24 lanes.  Warp 0 also loads Q and publishes the validity mask of
-        // the tile's 128 entries.
-        const int kw = warp == 0 ? 0 : (warp == 6 ? 1 : warp - 6);
-        const int g = kw >> 1;
-        const int quad = 8 * (kw & 1) + (lane & 7), sg = lane >> 3;
-        const int key0 = static_cast<int>(rank) * 64 + 4 * quad;          // first of this lane's four keys in the tile
-        const uint32_t dst = sK + (g * kKG + sg) * 8192 + static_cast<uint32_t>(quad) * 512u;
-        const int col = (g * kKG + sg) * 64;
+    if (warp < 4 || warp > 7) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kDsaRegsLow));
+    if (warp == 0) {
+        // ============================ validity masks ============================
         uint32_t kc = 0;
         bool ok = true;
         for (int t = pair; t < p.total_q && ok; t += num_pairs) {
             const int2 tk = __ldg(p.tok + t);
             if (tk.x < 0) continue;
-            if (warp == 0) {
-                // Q may be replaced once the scores of the previous item's last tile are done
-                if (kc > 0) {
-                    if (lane == 0) ok = mbar_wait(bar_s_full + 8 * ((kc - 1) & 1), ((kc - 1) >> 1) & 1, s_abort, 901);
-                    ok = __shfl_sync(0xffffffffu, ok, 0);
-                    if (!ok) break;
-                }
-                if (lane == 0 && leader) {
-                    mbar_arrive_expect_tx(bar_q_full, 2 * kMla2QBytes);   // both CTAs' boxes, rows outside the tensor included
-                }
-                if (lane == 0) tma2_load_4d(sQ, &tm_qh, pair_q_full, 0, static_cast<int>(rank) * kMla2Rows, 0, t);
-            }
-            const int self_row = row_of(tk.x, tk.y);
-            int e_next[4], m_next[4];
-            load_entries(t, 0, key0, e_next);
-            if (warp == 0) load_entries(t, 0, 4 * lane, m_next);
+            int m_next[4];
+            load_entries(t, 0, 4 * lane, m_next);
             for (int j = 0; j < n_tiles && ok; ++j) {
-                int e[4], r[4];
+                // validity of the tile's 128 entries: word i holds entry 4 l + i of lane l in bit l; a ring of four
+                // slots that the softmax warps hand back after reading
+                uint32_t bits = 0;
 #pragma unroll
-                for (int i = 0; i < 4; ++i) e[i] = e_next[i];
-                if (warp == 0) {
-                    // validity of the tile's 128 entries: word i holds entry 4 l + i of lane l in bit l; a ring of four
-                    // slots that the softmax warps hand back after reading
-                    uint32_t bits = 0;
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) bits |= (m_next[i] >= 0 && m_next[i] <= tk.y ? 1u : 0u) << i;
-                    const uint32_t w0 = __ballot_sync(0xffffffffu, bits & 1u), w1 = __ballot_sync(0xffffffffu, bits & 2u),
-                                   w2 = __ballot_sync(0xffffffffu, bits & 4u), w3 = __ballot_sync(0xffffffffu, bits & 8u);
-                    if (lane == 0) {
-                        if (kc >= 4) ok = mbar_wait(bar_mask_free + 8 * (kc & 3), ((kc - 4) >> 2) & 1, s_abort, 904);
+                for (int i = 0; i < 4; ++i) bits |= (m_next[i] >= 0 && m_next[i] <= tk.y ? 1u : 0u) << i;
+                const uint32_t w0 = __ballot_sync(0xffffffffu, bits & 1u), w1 = __ballot_sync(0xffffffffu, bits & 2u),
+                               w2 = __ballot_sync(0xffffffffu, bits & 4u), w3 = __ballot_sync(0xffffffffu, bits & 8u);
+                if (j + 1 < n_tiles) load_entries(t, j + 1, 4 * lane, m_next);
+                if (lane == 0) {
+                    if (kc >= 4) ok = mbar_wait(bar_mask_free + 8 * (kc & 3), ((kc - 4) >> 2) & 1, s_abort, 904);
+                    if (ok) {
                         volatile uint32_t* m = vmask + (kc & 3) * 4;
                         m[0] = w0; m[1] = w1; m[2] = w2; m[3] = w3;
                         mbar_arrive(bar_mask + 8 * (kc & 3));
                     }
-                    if (j + 1 < n_tiles) load_entries(t, j + 1, 4 * lane, m_next);
-                }
-                if (j + 1 < n_tiles) load_entries(t, j + 1, key0, e_next);
-                rows_of(tk.x, tk.y, self_row, e, r);
-                if (lane == 0 && ok) {
-                    if (g < kKGroups - 1) ok = mbar_wait(bar_k_empty + 8 * g, (kc & 1) ^ 1, s_abort, 902);
-                    else if (kc > 0) ok = mbar_wait(bar_s_full + 8 * ((kc - 1) & 1), ((kc - 1) >> 1) & 1, s_abort, 902);
-                    if (ok && leader && (kw & 1) == 0) mbar_arrive_expect_tx(bar_k_full + 8 * g, 2 * kKG * 8192);
                 }
                 ok = __shfl_sync(0xffffffffu, ok, 0);
-                if (!ok) break;
-                if (sg < kKG) tma2_gather4(dst, &tm_rows, pair_k_full + 8 * g, col, r[0], r[1], r[2], r[3]);
                 ++kc;
             }
         }
-    } else if (warp >= 12) {
-        // ======================================= V producers =======================================
+    } else if (warp == 3 || (warp >= 8 && warp < 8 + kDsaKWarps - 1)) {
+        // ===================================== K producers =====================================
+        // Warp kw brings slab kw of this CTA's 64 keys, a quad of keys per lane, as soon as its hand-back group
+        // (slabs 3 g .. 3 g + 2) is free; the group's first warp announces the bytes of the pair.
+        const int kw = warp == 3 ? 0 : warp - 7;
+        const int g = kw / kKG;
+        const int quad = lane & 15;
+        const int key0 = static_cast<int>(rank) * 64 + 4 * quad;          // first of this lane's four keys in the tile
+        const uint32_t dst = sK + kw * 8192 + static_cast<uint32_t>(quad) * 512u;
+        uint32_t kc = 0;
+        bool ok = true;
+        for (int t = pair; t < p.total_q && ok; t += num_pairs) {
+            const int2 tk = __ldg(p.tok + t);
+            if (tk.x < 0) continue;
+            const int self_row = row_of(tk.x, tk.y);
+            int e_next[4];
+            load_entries(t, 0, key0, e_next);
+            if (kw == kDsaKWarps - 1 && lane == 0) {
+                // This warp loads Q too: it may be replaced once the scores of the previous item's last tile are done, which is
+                // what the last group waits for.  (A warp that runs further ahead, as the one of the masks does, must not wait
+                // on that barrier: two phases ahead its parity reads as done.)
+                if (kc > 0) ok = mbar_wait(bar_s_full + 8 * ((kc - 1) & 1), ((kc - 1) >> 1) & 1, s_abort, 901);
+                if (ok) {
+                    if (leader) mbar_arrive_expect_tx(bar_q_full, 2 * kMla2QBytes);   // both CTAs' boxes, rows outside the tensor included
+                    tma2_load_4d(sQ, &tm_qh, pair_q_full, 0, static_cast<int>(rank) * kMla2Rows, 0, t);
+                }
+            }
+            ok = __shfl_sync(0xffffffffu, ok, 0);
+            for (int j = 0; j < n_tiles && ok; ++j) {
+                int e[4], r[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) e[i] = e_next[i];
+                if (j + 1 < n_tiles) load_entries(t, j + 1, key0, e_next);
+                rows_of(tk.x, tk.y, self_row, e, r);
+                if (lane == 0) {
+                    if (g < kKGroups - 1) ok = mbar_wait(bar_k_empty + 8 * g, (kc & 1) ^ 1, s_abort, 902);
+                    else if (kc > 0) ok = mbar_wait(bar_s_full + 8 * ((kc - 1) & 1), ((kc - 1) >> 1) & 1, s_abort, 902);
+                    if (ok && leader && kw % kKG == 0) mbar_arrive_expect_tx(bar_k_full + 8 * g, 2 * kKG * 8192);
+                }
+                ok = __shfl_sync(0xffffffffu, ok, 0);
+                if (!ok) break;
+                if (lane < 16) tma2_gather4(dst, &tm_rows, pair_k_full + 8 * g, kw * 64, r[0], r[1], r[2], r[3]);
+                ++kc;
+            }
+        }
+    } else if (warp >= 16) {
+        // ===================================== V producers =====================================
         // chunk c = (key half hf, instr i) holds value columns 256 i + 128 rank .. + 127 (two 64-column slabs) of keys
-        // 64 hf .. 64 hf + 63.  Group hf = 64 copies = warps vw = 2 hf and 2 hf + 1 with 8 quads each,
-        // lane = 8 * (2 i + slab) + quad: all 32 lanes, one instruction per tile.
-        const int vw = warp - 12;
-        const int hf = vw >> 1;
-        const int quad = 8 * (vw & 1) + (lane & 7), s4 = lane >> 3;
+        // 64 hf .. 64 hf + 63: four warps per key half (a hand-back group), one slab each, a quad of keys per lane.
+        const int vw = warp - 16;
+        const int hf = vw >> 2, s4 = vw & 3;
+        const int quad = lane & 15;
         const int key0 = hf * 64 + 4 * quad;
         const int slab = 4 * (s4 >> 1) + 2 * static_cast<int>(rank) + (s4 & 1);
         const uint32_t dst = sV + (2 * hf + (s4 >> 1)) * kMla2VChunk + (s4 & 1) * 8192 + static_cast<uint32_t>(quad) * 512u;
@@ -308,11 +318,11 @@ dsa_attn_kernel(const __grid_constant__ CUtensorMap tm_qh, const __grid_constant
                 if (lane == 0) {
                     if (hf < kVGroups - 1) ok = mbar_wait(bar_v_empty + 8 * hf, (vc & 1) ^ 1, s_abort, 903);
                     else if (vc > 0) ok = mbar_wait(bar_pv_done, (vc - 1) & 1, s_abort, 903);
-                    if (ok && leader && (vw & 1) == 0) mbar_arrive_expect_tx(bar_v_full + 8 * hf, 2 * kVG * kMla2VChunk);
+                    if (ok && leader && s4 == 0) mbar_arrive_expect_tx(bar_v_full + 8 * hf, 2 * kVG * kMla2VChunk);
                 }
                 ok = __shfl_sync(0xffffffffu, ok, 0);
                 if (!ok) break;
-                tma2_gather4(dst, &tm_rows, pair_v_full + 8 * hf, slab * 64, r[0], r[1], r[2], r[3]);
+                if (lane < 16) tma2_gather4(dst, &tm_rows, pair_v_full + 8 * hf, slab * 64, r[0], r[1], r[2], r[3]);
                 ++vc;
             }
         }
@@ -361,7 +371,7 @@ dsa_attn_kernel(const __grid_constant__ CUtensorMap tm_qh, const __grid_constant
                 ++kc;
             }
         }
-    } else if (warp == 7 && leader && lane == 0) {
+    } else if (warp == 2 && leader && lane == 0) {
         // ============ P V MMA issuer: one thread for both CTAs of the pair (O += P V) ============
         constexpr uint32_t kIdescPV = idesc_bf16(128, 256, false, true);
         constexpr uint32_t kHi = desc_hi_sw128(1024);
@@ -404,7 +414,9 @@ dsa_attn_kernel(const __grid_constant__ CUtensorMap tm_qh, const __grid_constant
                 ++vc;
             }
         }
-    } else if (warp >= 2 && warp <= 5) {
+    }
+    } else {
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kDsaRegsHigh));
         // ======================================= softmax =======================================
         const int l128 = ((warp & 3) << 5) | lane;     // TMEM lane
         const int row = l128 & 63;                     // row of this CTA's 64 = q-head 64 rank + row
