@@ -342,12 +342,13 @@ const char *vpp_host_last_error(void);
  * block_table, prefix_len, chunk_len, num_reqs (<= 8192), max_blocks_per_req, block_size (power of two), num_blocks,
  * total_q, max_seq_len, softmax_scale: as in vpp_chunk_attn_args.
  * out          bf16 [total_q, num_q_heads, 512]; lse float [total_q, num_q_heads] or NULL.
- * workspace    device memory of at least vpp_sparse_attn_workspace_size(total_q) bytes, 16-byte aligned; owned by the
- *              caller, contents irrelevant on entry.
+ * workspace    device memory of vpp_sparse_attn_workspace_size(total_q) bytes, 16-byte aligned; owned by the
+ *              caller, contents irrelevant on entry.  With few tokens it holds partial results too (their lists are cut into parts, merged by a third kernel); a workspace that holds
+ *              256 + 8 total_q bytes only is accepted and the launch runs uncut.
  * status       optional device int32, zeroed by the call; VPP_DEV_BAD_LENGTHS (nothing is written),
  *              VPP_DEV_BAD_BLOCK (a needed block_table entry outside [0, num_blocks): results undefined but no
  *              access leaves the cache) or VPP_DEV_TIMEOUT as in vpp_chunk_attn_fwd.
- * Returns after enqueueing two kernels on `stream`; no allocation, no synchronisation.
+ * Returns after enqueueing two or three kernels on `stream`; no allocation, no synchronisation.
  */
 typedef struct {
     const void *q;

@@ -736,9 +736,37 @@ vpp_status vpp_kv_append(const vpp_kv_append_args* a, vpp_stream_t stream_) {
     return VPP_OK;
 }
 
-size_t vpp_sparse_attn_workspace_size(int32_t total_q) {
-    return 256 + sizeof(int2) * static_cast<size_t>(total_q > 0 ? total_q : 0);
+namespace {
+// Workspace of a sparse launch: the token table, then -- for launches of so few tokens that their lists are cut into
+// parts -- the number of parts of every token and the partial results.
+struct SparseLayout {
+    size_t row_splits, o_parts, lse_parts, total, base;   // base: without the partials
+    int max_splits;
+};
+constexpr int kSparseMaxSplits = 8;
+SparseLayout sparse_layout(int32_t total_q) {
+    const size_t T = static_cast<size_t>(total_q > 0 ? total_q : 0);
+    SparseLayout L{};
+    L.base = 256 + sizeof(int2) * T;
+    L.total = L.base;
+    // A list is cut only where a whole number of parts, two or more, keeps every item in the one wave of SM pairs: 16 tokens
+    // with 2048-entry lists ran 54 us on 16 of 74 pairs, cut in four they run on 64 pairs.  More tokens fill the pairs
+    // by themselves well enough that a second wave of shorter items costs what it saves.
+    const int pairs = sm_count_or_default() / 2;
+    L.max_splits = T > 0 && pairs >= 2 * static_cast<int>(T) ? pairs / static_cast<int>(T) : 1;
+    if (L.max_splits > kSparseMaxSplits) L.max_splits = kSparseMaxSplits;
+    if (L.max_splits > 1) {
+        const size_t rows = T * L.max_splits * 2 * vpp::kMla2Rows;
+        L.row_splits = align_up(L.base, 256);
+        L.o_parts = align_up(L.row_splits + sizeof(int32_t) * T, 256);
+        L.lse_parts = align_up(L.o_parts + sizeof(float) * rows * vpp::kMlaDv, 256);
+        L.total = L.lse_parts + sizeof(float) * rows;
+    }
+    return L;
 }
+}  // namespace
+
+size_t vpp_sparse_attn_workspace_size(int32_t total_q) { return sparse_layout(total_q).total; }
 
 vpp_status vpp_sparse_mla_fwd(const vpp_sparse_attn_args* a, vpp_stream_t stream_) {
     g_err[0] = 0;
@@ -751,9 +779,7 @@ vpp_status vpp_sparse_mla_fwd(const vpp_sparse_attn_args* a, vpp_stream_t stream
         return fail(VPP_ERR_INVALID_ARG, "softmax_scale must be positive and finite");
     if (a->num_reqs > vpp::kDsaMaxReqs) return fail(VPP_ERR_UNSUPPORTED, "at most %d requests", vpp::kDsaMaxReqs);
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);
-    if (a->status && cudaMemsetAsync(a->status, 0, sizeof(int32_t), stream) != cudaSuccess)
-        return fail(VPP_ERR_CUDA, "memset status: %s", cudaGetErrorString(cudaGetLastError()));
-    if (a->total_q == 0 || a->num_reqs == 0) return VPP_OK;
+    if (a->total_q == 0 || a->num_reqs == 0) return zero_status(a->status, stream);
     if (!a->q || !a->kv_cache || !a->indices || !a->prefix_len || !a->chunk_len || !a->out)
         return fail(VPP_ERR_INVALID_ARG, "q, kv_cache, indices, prefix_len, chunk_len and out must be non-null");
     if ((reinterpret_cast<uintptr_t>(a->q) | reinterpret_cast<uintptr_t>(a->kv_cache) | reinterpret_cast<uintptr_t>(a->out) |
@@ -761,8 +787,14 @@ vpp_status vpp_sparse_mla_fwd(const vpp_sparse_attn_args* a, vpp_stream_t stream
         return fail(VPP_ERR_INVALID_ARG, "q, kv_cache, out and workspace must be 16-byte aligned");
     if (a->kv_row_stride < vpp::kMlaDqk || a->kv_row_stride % 8)
         return fail(VPP_ERR_INVALID_ARG, "kv_row_stride must be a multiple of 8 elements and at least %d", vpp::kMlaDqk);
-    if (!a->workspace || a->workspace_bytes < vpp_sparse_attn_workspace_size(a->total_q))
-        return fail(VPP_ERR_WORKSPACE, "workspace too small: %zu bytes needed", vpp_sparse_attn_workspace_size(a->total_q));
+    const SparseLayout L = sparse_layout(a->total_q);
+    if (!a->workspace || a->workspace_bytes < L.base)
+        return fail(VPP_ERR_WORKSPACE, "workspace too small: %zu bytes needed", L.total);
+    // parts of at least two tiles; a workspace that holds the token table only runs unsplit
+    const int list_tiles = (a->topk + vpp::kTileN - 1) / vpp::kTileN;
+    int splits = a->workspace_bytes < L.total ? 1 : L.max_splits;
+    if (splits > list_tiles / 2) splits = list_tiles / 2;
+    if (splits < 1) splits = 1;
     int shift = 0;
     long long capacity, num_rows;
     if (a->block_table) {
@@ -794,16 +826,17 @@ vpp_status vpp_sparse_mla_fwd(const vpp_sparse_attn_args* a, vpp_stream_t stream
         if (!make_tmap(&tm_qh, a->q, 4, dh, sh, bh) || !make_tmap(&tm_rows, a->kv_cache, 2, dr, sr, br))
             return fail(VPP_ERR_CUDA, "cuTensorMapEncodeTiled(sparse mla) failed");
     }
-    int2* tok = reinterpret_cast<int2*>(static_cast<uint8_t*>(a->workspace));
+    uint8_t* ws = static_cast<uint8_t*>(a->workspace);
+    int2* tok = reinterpret_cast<int2*>(ws);
+    int32_t* row_splits = reinterpret_cast<int32_t*>(ws + L.row_splits);
     const int sms = sm_count_or_default();
     {
         long long blocks = (static_cast<long long>(a->total_q) + vpp::kDsaPrepThreads - 1) / vpp::kDsaPrepThreads;
         if (blocks > 4ll * sms) blocks = 4ll * sms;
         const size_t smem = sizeof(int32_t) * (static_cast<size_t>(a->num_reqs) + 1);
-        vpp::dsa_tokens_kernel<<<static_cast<unsigned>(blocks), vpp::kDsaPrepThreads, smem, stream>>>(
-            a->prefix_len, a->chunk_len, a->num_reqs, a->total_q, capacity, tok, a->status);
-        cudaError_t ce = cudaGetLastError();
-        if (ce != cudaSuccess) return fail(VPP_ERR_CUDA, "token table launch: %s", cudaGetErrorString(ce));
+        const cudaError_t te = launch(vpp::dsa_tokens_kernel, static_cast<unsigned>(blocks), vpp::kDsaPrepThreads, smem, stream, a->prefix_len,
+                                      a->chunk_len, a->num_reqs, a->total_q, capacity, splits, tok, row_splits, a->status);
+        if (te != cudaSuccess) return fail(VPP_ERR_CUDA, "token table launch: %s", cudaGetErrorString(te));
     }
     vpp::DsaParams p{};
     p.indices = a->indices;
@@ -817,19 +850,29 @@ vpp_status vpp_sparse_mla_fwd(const vpp_sparse_attn_args* a, vpp_stream_t stream
     p.num_q_heads = a->num_q_heads;
     p.total_q = a->total_q;
     p.scale_log2e = a->softmax_scale * 1.4426950408889634f;
+    p.splits = splits;
     p.out = a->out;
     p.lse = a->lse;
+    p.o_parts = reinterpret_cast<float*>(ws + L.o_parts);
+    p.lse_parts = reinterpret_cast<float*>(ws + L.lse_parts);
     p.status = a->status;
-    auto kern = vpp::dsa_attn_kernel;
+    auto kern = splits > 1 ? vpp::dsa_attn_kernel<true> : vpp::dsa_attn_kernel<false>;
     cudaError_t ce = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, vpp::kMla2SmemBytes);
     if (ce == cudaSuccess) {
-        int pairs = sms / 2;
-        if (pairs > a->total_q) pairs = a->total_q;
-        kern<<<pairs * 2, vpp::kDsaThreads, vpp::kMla2SmemBytes, stream>>>(tm_qh, tm_rows, p);
-        ce = cudaGetLastError();
+        long long pairs = sms / 2, items = static_cast<long long>(a->total_q) * splits;
+        if (pairs > items) pairs = items;
+        ce = launch(kern, static_cast<unsigned>(pairs * 2), vpp::kDsaThreads, vpp::kMla2SmemBytes, stream, tm_qh, tm_rows, p);
     }
     if (ce != cudaSuccess) return fail(VPP_ERR_CUDA, "sparse attention launch: %s", cudaGetErrorString(ce));
     g_launches = 2;
+    if (splits > 1) {
+        unsigned blocks = 1;
+        const MergeKernel mk = pick_merge_kernel(splits, a->total_q, a->num_q_heads, vpp::kMlaDv, sms, &blocks);
+        ce = launch(mk, blocks, vpp::kMergeThreads, 0, stream, p.o_parts, p.lse_parts, splits, a->total_q, a->num_q_heads, vpp::kMlaDv,
+                    row_splits, nullptr, static_cast<__nv_bfloat16*>(a->out), a->lse);
+        if (ce != cudaSuccess) return fail(VPP_ERR_CUDA, "merge launch: %s", cudaGetErrorString(ce));
+        ++g_launches;
+    }
     return VPP_OK;
 }
 

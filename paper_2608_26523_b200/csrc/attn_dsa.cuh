@@ -12,6 +12,8 @@
 // so they are spread over 17 producer warps of 16 lanes, one slab of 64 keys each, and the register file is split
 // unevenly (setmaxnreg) to make room for them.  2048 tokens with lists of
 // 2048 at prefix 65536: 10 producer warps of 24 and 32 lanes 1458 us, these 1362 us.
+// A launch of few tokens (a decode batch) would leave most pairs idle for the 16 tiles of a 2048-entry list: then a token's
+// list is cut into `splits` parts, an item each, whose partial results lse_merge_small_kernel joins (16 tokens: 62.6 -> 38.2 us for the step).
 // Entries that do not take part are pointed at the token's own cache row (always present and finite) and masked out
 // of the softmax through a 128-bit validity mask that warp 0 publishes per tile.  The cost per token does not depend on
 // the prefix length: the flat latency curve the paper says weakens its linear-growth assumption.
@@ -44,19 +46,24 @@ struct DsaParams {
     int32_t num_q_heads;
     int32_t total_q;
     float scale_log2e;
+    int32_t splits;               // parts a token's list is cut into (1: final results)
     void* out;                    // bf16 [T, Hq, 512]
     float* lse;                   // [T, Hq] or null
+    float* o_parts;               // splits > 1: [splits, T, Hq, 512] and [splits, T, Hq]
+    float* lse_parts;
     int32_t* status;
 };
 
 // (request, position) of every token from the per-request lengths; lengths that do not describe the launch mark every
-// token as skipped and set the status.
+// token as skipped (nothing to merge either) and set the status.
 __global__ void __launch_bounds__(kDsaPrepThreads)
 dsa_tokens_kernel(const int32_t* prefix_len, const int32_t* chunk_len, int num_reqs, int total_q, long long capacity,
-                  int2* tok, int32_t* status) {
+                  int splits, int2* tok, int32_t* row_splits, int32_t* status) {
     extern __shared__ int32_t cu[];   // cu[r] = tokens before request r
     __shared__ int s_bad;
     const int tid = threadIdx.x, lane = tid & 31;
+    pdl_launch_dependents();
+    pdl_wait();
     if (tid == 0) s_bad = 0;
     __syncthreads();
     if (tid < 32) {
@@ -85,8 +92,9 @@ dsa_tokens_kernel(const int32_t* prefix_len, const int32_t* chunk_len, int num_r
     }
     __syncthreads();
     const bool bad = s_bad || cu[num_reqs] != total_q;
-    if (bad && tid == 0 && blockIdx.x == 0 && status) atomicCAS(status, 0, 1 /* VPP_DEV_BAD_LENGTHS */);
+    if (tid == 0 && blockIdx.x == 0 && status) *status = bad ? 1 /* VPP_DEV_BAD_LENGTHS */ : 0;
     for (int t = blockIdx.x * kDsaPrepThreads + tid; t < total_q; t += gridDim.x * kDsaPrepThreads) {
+        if (splits > 1) row_splits[t] = bad ? 0 : splits;
         if (bad) {
             tok[t] = make_int2(-1, -1);
             continue;
@@ -111,6 +119,8 @@ __device__ __forceinline__ void tma2_gather4(uint32_t dst, const CUtensorMap* m,
         : "memory");
 }
 
+// kParts: a token's list is cut into p.splits parts (otherwise p.splits is 1)
+template <bool kParts>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kDsaThreads, 1)
 dsa_attn_kernel(const __grid_constant__ CUtensorMap tm_qh, const __grid_constant__ CUtensorMap tm_rows, const DsaParams p) {
     // tm_qh:   (64 cols, Hq heads, 9 slabs, T tokens) box (64, 64, 9, 1) -- 64 q-heads of one token, all slabs (heads past Hq read as zero)
@@ -183,10 +193,26 @@ dsa_attn_kernel(const __grid_constant__ CUtensorMap tm_qh, const __grid_constant
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *s_tmem;
+    pdl_wait();                  // the token table comes from the kernel launched just before
+    pdl_launch_dependents();
 
     const int num_pairs = gridDim.x >> 1;
     const int pair = blockIdx.x >> 1;
-    const int n_tiles = (p.topk + kTileN - 1) / kTileN;   // the same for every token
+    // Items: (token, part of its list); part s has the tiles first_tile(s) .. first_tile(s + 1) - 1 of the list's.
+    const int list_tiles = (p.topk + kTileN - 1) / kTileN;   // the same for every token
+    const int num_items = kParts ? p.total_q * p.splits : p.total_q;
+    auto part_of = [&](int item, int& t, int& j0, int& j1) {
+        if (!kParts) {
+            t = item;
+            j0 = 0;
+            j1 = list_tiles;
+            return;
+        }
+        t = item / p.splits;
+        const int s = item - t * p.splits;
+        j0 = s * list_tiles / p.splits;
+        j1 = (s + 1) * list_tiles / p.splits;
+    };
 
     // cache row of position e of request req
     auto row_of = [&](int req, int e) -> int {
@@ -220,12 +246,14 @@ dsa_attn_kernel(const __grid_constant__ CUtensorMap tm_qh, const __grid_constant
         // ============================ validity masks ============================
         uint32_t kc = 0;
         bool ok = true;
-        for (int t = pair; t < p.total_q && ok; t += num_pairs) {
+        for (int item = pair; item < num_items && ok; item += num_pairs) {
+            int t, j0, j1;
+            part_of(item, t, j0, j1);
             const int2 tk = __ldg(p.tok + t);
             if (tk.x < 0) continue;
             int m_next[4];
-            load_entries(t, 0, 4 * lane, m_next);
-            for (int j = 0; j < n_tiles && ok; ++j) {
+            load_entries(t, j0, 4 * lane, m_next);
+            for (int j = j0; j < j1 && ok; ++j) {
                 // validity of the tile's 128 entries: word i holds entry 4 l + i of lane l in bit l; a ring of four
                 // slots that the softmax warps hand back after reading
                 uint32_t bits = 0;
@@ -233,7 +261,7 @@ dsa_attn_kernel(const __grid_constant__ CUtensorMap tm_qh, const __grid_constant
                 for (int i = 0; i < 4; ++i) bits |= (m_next[i] >= 0 && m_next[i] <= tk.y ? 1u : 0u) << i;
                 const uint32_t w0 = __ballot_sync(0xffffffffu, bits & 1u), w1 = __ballot_sync(0xffffffffu, bits & 2u),
                                w2 = __ballot_sync(0xffffffffu, bits & 4u), w3 = __ballot_sync(0xffffffffu, bits & 8u);
-                if (j + 1 < n_tiles) load_entries(t, j + 1, 4 * lane, m_next);
+                if (j + 1 < j1) load_entries(t, j + 1, 4 * lane, m_next);
                 if (lane == 0) {
                     if (kc >= 4) ok = mbar_wait(bar_mask_free + 8 * (kc & 3), ((kc - 4) >> 2) & 1, s_abort, 904);
                     if (ok) {
@@ -257,12 +285,14 @@ dsa_attn_kernel(const __grid_constant__ CUtensorMap tm_qh, const __grid_constant
         const uint32_t dst = sK + kw * 8192 + static_cast<uint32_t>(quad) * 512u;
         uint32_t kc = 0;
         bool ok = true;
-        for (int t = pair; t < p.total_q && ok; t += num_pairs) {
+        for (int item = pair; item < num_items && ok; item += num_pairs) {
+            int t, j0, j1;
+            part_of(item, t, j0, j1);
             const int2 tk = __ldg(p.tok + t);
             if (tk.x < 0) continue;
             const int self_row = row_of(tk.x, tk.y);
             int e_next[4];
-            load_entries(t, 0, key0, e_next);
+            load_entries(t, j0, key0, e_next);
             if (kw == kDsaKWarps - 1 && lane == 0) {
                 // This warp loads Q too: it may be replaced once the scores of the previous item's last tile are done, which is
                 // what the last group waits for.  (A warp that runs further ahead, as the one of the masks does, must not wait
@@ -274,11 +304,11 @@ dsa_attn_kernel(const __grid_constant__ CUtensorMap tm_qh, const __grid_constant
                 }
             }
             ok = __shfl_sync(0xffffffffu, ok, 0);
-            for (int j = 0; j < n_tiles && ok; ++j) {
+            for (int j = j0; j < j1 && ok; ++j) {
                 int e[4], r[4];
 #pragma unroll
                 for (int i = 0; i < 4; ++i) e[i] = e_next[i];
-                if (j + 1 < n_tiles) load_entries(t, j + 1, key0, e_next);
+                if (j + 1 < j1) load_entries(t, j + 1, key0, e_next);
                 rows_of(tk.x, tk.y, self_row, e, r);
                 if (lane == 0) {
                     if (g < kKGroups - 1) ok = mbar_wait(bar_k_empty + 8 * g, (kc & 1) ^ 1, s_abort, 902);
@@ -303,17 +333,19 @@ dsa_attn_kernel(const __grid_constant__ CUtensorMap tm_qh, const __grid_constant
         const uint32_t dst = sV + (2 * hf + (s4 >> 1)) * kMla2VChunk + (s4 & 1) * 8192 + static_cast<uint32_t>(quad) * 512u;
         uint32_t vc = 0;
         bool ok = true;
-        for (int t = pair; t < p.total_q && ok; t += num_pairs) {
+        for (int item = pair; item < num_items && ok; item += num_pairs) {
+            int t, j0, j1;
+            part_of(item, t, j0, j1);
             const int2 tk = __ldg(p.tok + t);
             if (tk.x < 0) continue;
             const int self_row = row_of(tk.x, tk.y);
             int e_next[4];
-            load_entries(t, 0, key0, e_next);
-            for (int j = 0; j < n_tiles && ok; ++j) {
+            load_entries(t, j0, key0, e_next);
+            for (int j = j0; j < j1 && ok; ++j) {
                 int e[4], r[4];
 #pragma unroll
                 for (int i = 0; i < 4; ++i) e[i] = e_next[i];
-                if (j + 1 < n_tiles) load_entries(t, j + 1, key0, e_next);
+                if (j + 1 < j1) load_entries(t, j + 1, key0, e_next);
                 rows_of(tk.x, tk.y, self_row, e, r);
                 if (lane == 0) {
                     if (hf < kVGroups - 1) ok = mbar_wait(bar_v_empty + 8 * hf, (vc & 1) ^ 1, s_abort, 903);
@@ -346,11 +378,13 @@ dsa_attn_kernel(const __grid_constant__ CUtensorMap tm_qh, const __grid_constant
             tc_commit2(g < kKGroups - 1 ? bar_k_empty + 8 * g : bar_last, 3);
         };
         static_assert(kKGroups == 3, "one call per K group");
-        for (int t = pair; t < p.total_q && ok; t += num_pairs) {
+        for (int item = pair; item < num_items && ok; item += num_pairs) {
+            int t, j0, j1;
+            part_of(item, t, j0, j1);
             if (__ldg(p.tok + t).x < 0) continue;
             ok = mbar_wait(bar_q_full, q_it & 1, s_abort, 921);
             ++q_it;
-            for (int jj = 0; jj < n_tiles && ok; ++jj) {
+            for (int jj = 0; jj < j1 - j0 && ok; ++jj) {
                 const uint32_t b = kc & 1, kpar = kc & 1;
                 const uint32_t tS = tmem_base + b * 64, bar_s = bar_s_full + 8 * b;
                 // S[b] was last read by the softmax of two tiles ago: its P is ready <=> that read is over
@@ -395,9 +429,11 @@ dsa_attn_kernel(const __grid_constant__ CUtensorMap tm_qh, const __grid_constant
             tc_commit2(g < kVGroups - 1 ? bar_v_empty + 8 * g : bar_pv_done, 3);
         };
         static_assert(kVGroups == 2, "one call per V group");
-        for (int t = pair; t < p.total_q && ok; t += num_pairs) {
+        for (int item = pair; item < num_items && ok; item += num_pairs) {
+            int t, j0, j1;
+            part_of(item, t, j0, j1);
             if (__ldg(p.tok + t).x < 0) continue;
-            for (int jj = 0; jj < n_tiles && ok; ++jj) {
+            for (int jj = 0; jj < j1 - j0 && ok; ++jj) {
                 const uint32_t b = vc & 1, vpar = vc & 1;
                 ok = mbar_wait_cluster(bar_p_full + 8 * b, (vc >> 1) & 1, s_abort, 926);
                 if (!ok) break;
@@ -437,10 +473,12 @@ dsa_attn_kernel(const __grid_constant__ CUtensorMap tm_qh, const __grid_constant
             return true;
         };
         bool ok = true;
-        for (int t = pair; t < p.total_q && ok; t += num_pairs) {
+        for (int item = pair; item < num_items && ok; item += num_pairs) {
+            int t, j0, j1;
+            part_of(item, t, j0, j1);
             if (__ldg(p.tok + t).x < 0) continue;
             float m_ref = -INFINITY, l_run = 0.f;
-            for (int j = 0; j < n_tiles; ++j) {
+            for (int j = j0; j < j1; ++j) {
                 const uint32_t b = tc & 1;
                 const uint32_t tS = tmem_base + b * 64 + lane_off;
                 ok = mbar_wait(bar_s_full + 8 * b, (tc >> 1) & 1, s_abort, 932);
@@ -481,7 +519,7 @@ dsa_attn_kernel(const __grid_constant__ CUtensorMap tm_qh, const __grid_constant
                     const float alpha = grow ? ex2(m_ref - m_new) : 1.f;
                     if (grow) m_ref = m_new;
                     l_run *= alpha;
-                    if (j > 0) {
+                    if (j > j0) {
                         // O is rescaled in place: P V of the previous tile must be done
                         ok = mbar_wait(bar_pv_done, (tc - 1) & 1, s_abort, 935);
                         if (!ok) break;
@@ -541,6 +579,8 @@ dsa_attn_kernel(const __grid_constant__ CUtensorMap tm_qh, const __grid_constant
             tc_fence_after();
             const float inv_l = l_tot > 0.f ? 1.f / l_tot : 0.f;   // no entry took part: the output is zero
             const bool live = h < p.num_q_heads;
+            // row of out / lse, or of the partials (part, token, q-head)
+            const long long out_row = (kParts ? static_cast<long long>(item - t * p.splits) * p.total_q + t : t) * p.num_q_heads + h;
             uint32_t r[32];
 #pragma unroll 1
             for (int c = 0; c < 8; ++c) {
@@ -548,19 +588,29 @@ dsa_attn_kernel(const __grid_constant__ CUtensorMap tm_qh, const __grid_constant
                 tc_wait_ld();
                 if (!live) continue;
                 const int col0 = (c >> 2) * 256 + half * 128 + (c & 3) * 32;
-                uint4* dst = reinterpret_cast<uint4*>(static_cast<uint8_t*>(p.out) +
-                                                      ((static_cast<long long>(t) * p.num_q_heads + h) * kMlaDv + col0) * 2);
+                if (!kParts) {
+                    uint4* dst = reinterpret_cast<uint4*>(static_cast<uint8_t*>(p.out) + (out_row * kMlaDv + col0) * 2);
 #pragma unroll
-                for (int q4 = 0; q4 < 4; ++q4) {
-                    uint32_t w[4];
+                    for (int q4 = 0; q4 < 4; ++q4) {
+                        uint32_t w[4];
 #pragma unroll
-                    for (int e = 0; e < 4; ++e)
-                        w[e] = pack_bf16x2(__uint_as_float(r[q4 * 8 + 2 * e]) * inv_l, __uint_as_float(r[q4 * 8 + 2 * e + 1]) * inv_l);
-                    dst[q4] = make_uint4(w[0], w[1], w[2], w[3]);
+                        for (int e = 0; e < 4; ++e)
+                            w[e] = pack_bf16x2(__uint_as_float(r[q4 * 8 + 2 * e]) * inv_l, __uint_as_float(r[q4 * 8 + 2 * e + 1]) * inv_l);
+                        dst[q4] = make_uint4(w[0], w[1], w[2], w[3]);
+                    }
+                } else {
+                    float4* dst = reinterpret_cast<float4*>(p.o_parts + out_row * kMlaDv + col0);
+#pragma unroll
+                    for (int q4 = 0; q4 < 8; ++q4)
+                        dst[q4] = make_float4(__uint_as_float(r[q4 * 4]) * inv_l, __uint_as_float(r[q4 * 4 + 1]) * inv_l,
+                                              __uint_as_float(r[q4 * 4 + 2]) * inv_l, __uint_as_float(r[q4 * 4 + 3]) * inv_l);
                 }
             }
-            if (live && half == 0 && p.lse)
-                p.lse[static_cast<long long>(t) * p.num_q_heads + h] = (m_ref + log2f(l_tot)) * 0.6931471805599453f;
+            if (live && half == 0) {
+                const float lse = (m_ref + log2f(l_tot)) * 0.6931471805599453f;
+                if (kParts) p.lse_parts[out_row] = lse;
+                else if (p.lse) p.lse[out_row] = lse;
+            }
             tc_fence_before();
         }
     }
