@@ -330,14 +330,36 @@ int choose_splits(const vpp_chunk_attn_args* a, int heads_per_item) {
     return static_cast<int>(s);
 }
 
-// The d = 128 kernel pairs two q-heads of one kv-head per work item; when a kv-head's group is odd (MHA included) an
-// item is two consecutive 128-row query tiles of one q-head instead (work units of 256 rows).
-bool pairs_two_heads(const vpp_chunk_attn_args* a) { return (a->num_q_heads / a->num_kv_heads) % 2 == 0; }
+// How the d = 128 kernel packs (token, q-head) pairs into the rows of a tile (attn_ws.cuh).
+struct RowPacking {
+    int group, tile_tokens;         // items of two tiles: q-heads x tokens of a tile
+    int short_group, short_tokens;  // items of one tile
+    int unit_rows;                  // query rows (tokens) per work unit
+};
+RowPacking row_packing(const vpp_chunk_attn_args* a) {
+    const int G = a->num_q_heads / a->num_kv_heads;
+    RowPacking r{};
+    // the largest part of a kv-head's group that fills at least 125 of the 128 rows (1 always does)
+    r.group = 1;
+    for (int d = 1; d <= vpp::kTileM && d <= G; ++d)
+        if (G % d == 0 && d * (vpp::kTileM / d) >= 125) r.group = d;
+    r.tile_tokens = vpp::kTileM / r.group;
+    // a packed item streams its K/V for these rows alone: the whole group if it fits a tile, however well it fills it
+    r.short_group = G <= vpp::kTileM ? G : r.group;
+    r.short_tokens = vpp::kTileM / r.short_group;
+    r.unit_rows = 2 * r.tile_tokens;
+    return r;
+}
+// Query rows of a work unit.
+int unit_rows_of(const vpp_chunk_attn_args* a, Family fam) { return fam == Family::kGqa128 ? row_packing(a).unit_rows : vpp::kTileM; }
+
+// (the split choice below counts work items of 256 rows: two 128-row tiles)
+bool even_groups(const vpp_chunk_attn_args* a) { return (a->num_q_heads / a->num_kv_heads) % 2 == 0; }
 // The absorbed-MLA kernel runs on pairs of SMs (2-CTA clusters).
 bool mla_kernel_available() { return sm_count_or_default() >= 2; }
 int heads_per_item(const vpp_chunk_attn_args* a, Family fam) {
     if (fam == Family::kMla576) return 1;
-    return pairs_two_heads(a) ? 2 : 1;
+    return even_groups(a) ? 2 : 1;
 }
 
 using MergeKernel = void (*)(const float*, const float*, int, long long, int, int, const int32_t*, const vpp::WorkHeader*, __nv_bfloat16*,
@@ -363,7 +385,8 @@ MergeKernel pick_merge_kernel(int splits, long long total_q, int num_q_heads, in
 vpp::WorkspaceLayout layout_for(const vpp_chunk_attn_args* a, Family fam) {
     vpp::WorkspaceLayout L{};
     const int S = choose_splits(a, heads_per_item(a, fam));
-    const long long tiles = (a->total_q + vpp::kTileM - 1) / vpp::kTileM + a->num_reqs;
+    const int unit_rows = unit_rows_of(a, fam);
+    const long long tiles = (a->total_q + unit_rows - 1) / unit_rows + a->num_reqs;
     L.splits = S;
     L.max_units = static_cast<int32_t>(tiles * S);
     size_t off = 0;
@@ -475,14 +498,6 @@ vpp_status run_chunk_attn(const vpp_chunk_attn_args* a, vpp_stream_t stream_, co
     // ---- tensor maps ----
     CUtensorMap tm_q, tm_k, tm_v;
     {
-        const uint64_t d[3] = {static_cast<uint64_t>(a->head_dim_qk), static_cast<uint64_t>(a->num_q_heads),
-                               static_cast<uint64_t>(a->total_q)};
-        const uint64_t s[2] = {static_cast<uint64_t>(a->head_dim_qk) * 2,
-                               static_cast<uint64_t>(a->head_dim_qk) * a->num_q_heads * 2};
-        const uint32_t b[3] = {64, 1, static_cast<uint32_t>(vpp::kTileM)};
-        if (!make_tmap(&tm_q, a->q, 3, d, s, b)) return fail(VPP_ERR_CUDA, "cuTensorMapEncodeTiled(q) failed");
-    }
-    {
         const uint64_t d[4] = {static_cast<uint64_t>(a->head_dim_qk), static_cast<uint64_t>(B),
                                static_cast<uint64_t>(a->num_kv_heads), static_cast<uint64_t>(n_blocks)};
         const uint64_t s[3] = {static_cast<uint64_t>(a->k_token_stride) * 2, static_cast<uint64_t>(a->k_head_stride) * 2,
@@ -499,22 +514,20 @@ vpp_status run_chunk_attn(const vpp_chunk_attn_args* a, vpp_stream_t stream_, co
         if (!make_tmap(&tm_v, a->v_cache, 4, d, s, b)) return fail(VPP_ERR_CUDA, "cuTensorMapEncodeTiled(v) failed");
     }
 
-    CUtensorMap tm_q2, tm_k2, tm_v2, tm_qh;
+    CUtensorMap tm_k2, tm_v2, tm_qs;
+    const RowPacking rp = row_packing(a);
+    // a batch of decode rows: a packed item's box brings its one token only
+    const int short_box_tokens = a->total_q <= a->num_reqs ? 1 : rp.short_tokens;
     if (fam == Family::kGqa128) {
-        // a single-token ("packed") work item takes the G q-heads of one kv-head as the rows of its Q tile
-        const int G = a->num_q_heads / a->num_kv_heads;
-        const uint64_t dh[3] = {static_cast<uint64_t>(a->head_dim_qk), static_cast<uint64_t>(a->num_q_heads),
+        const uint64_t dq[3] = {static_cast<uint64_t>(a->head_dim_qk), static_cast<uint64_t>(a->num_q_heads),
                                 static_cast<uint64_t>(a->total_q)};
-        const uint64_t sh[2] = {static_cast<uint64_t>(a->head_dim_qk) * 2,
+        const uint64_t sq[2] = {static_cast<uint64_t>(a->head_dim_qk) * 2,
                                 static_cast<uint64_t>(a->head_dim_qk) * a->num_q_heads * 2};
-        const uint32_t bh[3] = {64, static_cast<uint32_t>(G < vpp::kTileM ? G : vpp::kTileM), 1};
-        if (!make_tmap(&tm_qh, a->q, 3, dh, sh, bh)) return fail(VPP_ERR_CUDA, "cuTensorMapEncodeTiled(q heads) failed");
+        const uint32_t bq[3] = {64, static_cast<uint32_t>(rp.group), static_cast<uint32_t>(rp.tile_tokens)};
+        const uint32_t bs[3] = {64, static_cast<uint32_t>(rp.short_group), static_cast<uint32_t>(short_box_tokens)};
+        if (!make_tmap(&tm_q, a->q, 3, dq, sq, bq) || !make_tmap(&tm_qs, a->q, 3, dq, sq, bs))
+            return fail(VPP_ERR_CUDA, "cuTensorMapEncodeTiled(q) failed");
         // the 128 features viewed as (64, 2): a box holds both 64-column slabs of a tile
-        const uint64_t dq[4] = {64, static_cast<uint64_t>(a->total_q), 2, static_cast<uint64_t>(a->num_q_heads)};
-        const uint64_t sq[3] = {static_cast<uint64_t>(a->head_dim_qk) * a->num_q_heads * 2, 128,
-                                static_cast<uint64_t>(a->head_dim_qk) * 2};
-        const uint32_t bq[4] = {64, static_cast<uint32_t>(vpp::kTileM), 2, 1};
-        if (!make_tmap(&tm_q2, a->q, 4, dq, sq, bq)) return fail(VPP_ERR_CUDA, "cuTensorMapEncodeTiled(q tiles) failed");
         const uint64_t d[5] = {64, static_cast<uint64_t>(B), 2, static_cast<uint64_t>(a->num_kv_heads),
                                static_cast<uint64_t>(n_blocks)};
         const uint64_t sk[4] = {static_cast<uint64_t>(a->k_token_stride) * 2, 128, static_cast<uint64_t>(a->k_head_stride) * 2,
@@ -566,9 +579,13 @@ vpp_status run_chunk_attn(const vpp_chunk_attn_args* a, vpp_stream_t stream_, co
     pp.num_blocks = n_blocks;
     pp.splits = L.splits;
     pp.max_units = L.max_units;
-    pp.max_cost = (a->max_seq_len + vpp::kTileN - 1) / vpp::kTileN;
-    if (pp.max_cost < 1) pp.max_cost = 1;
-    pp.tile_m = (fam == Family::kGqa128 && !pairs_two_heads(a)) ? 2 * vpp::kTileM : vpp::kTileM;
+    pp.unit_rows = unit_rows_of(a, fam);
+    pp.short_rows = fam == Family::kGqa128 ? rp.short_tokens : 1;
+    // Item order: kv-head-major inside blocks of so many query rows.  Large blocks keep more CTAs on the same K/V pages, small
+    // ones keep the order longest-first where units differ (no long one is started near the end): a first chunk of 4096 tokens
+    // and 32 heads took 205 us with blocks of 4096 rows, 186 of 512; 8192 tokens at prefix 65536 16.46 ms against 16.58.
+    pp.unit_block = 4096 / pp.unit_rows > 1 ? 4096 / pp.unit_rows : 1;
+    pp.ragged_unit_block = 512 / pp.unit_rows > 1 ? 512 / pp.unit_rows : 1;
     pp.partial = range ? 1 : 0;
     pp.range_begin = range ? range->begin_tile : 0;
     pp.range_end = range ? range->end_tile : 0;
@@ -578,10 +595,10 @@ vpp_status run_chunk_attn(const vpp_chunk_attn_args* a, vpp_stream_t stream_, co
     pp.q_start = row_splits + a->total_q;
     pp.tile_start = pp.q_start + a->num_reqs + 1;
     {
-        // small launches (a short chunk, a small decode batch) take the one-warp decomposition
-        const long long tiles_ub = (a->total_q + pp.tile_m - 1) / pp.tile_m + a->num_reqs;
-        const bool small = a->num_reqs <= vpp::kPrepSmallMax && tiles_ub <= vpp::kPrepSmallMax;
-        const unsigned threads = small ? vpp::kPrepSmallThreads : vpp::kPrepThreads;
+        // a thread per request and per unit of an unsplit launch, as far as a block goes
+        const long long units_ub = (a->total_q + pp.unit_rows - 1) / pp.unit_rows + a->num_reqs;
+        unsigned threads = vpp::kPrepMinThreads;
+        while (threads < vpp::kPrepMaxThreads && threads < units_ub) threads *= 2;
         // blocks that check the block table: one per 4 entries a thread can have in flight, at most kMaxCheckers
         long long checkers = 0;
         if (paged) {
@@ -589,7 +606,7 @@ vpp_status run_chunk_attn(const vpp_chunk_attn_args* a, vpp_stream_t stream_, co
             checkers = (entries + 4 * threads - 1) / (4 * threads);
             if (checkers > vpp::kMaxCheckers) checkers = vpp::kMaxCheckers;
         }
-        const cudaError_t pe = launch(small ? vpp::prep_small_kernel : vpp::prep_kernel, static_cast<unsigned>(1 + checkers), threads,
+        const cudaError_t pe = launch(vpp::prep_kernel, static_cast<unsigned>(1 + checkers), threads,
                                       0, stream, pp);
         if (pe != cudaSuccess) return fail(VPP_ERR_CUDA, "work decomposition launch: %s", cudaGetErrorString(pe));
     }
@@ -604,6 +621,10 @@ vpp_status run_chunk_attn(const vpp_chunk_attn_args* a, vpp_stream_t stream_, co
     ap.num_q_heads = a->num_q_heads;
     ap.num_kv_heads = a->num_kv_heads;
     ap.total_q = a->total_q;
+    ap.group = rp.group;
+    ap.tile_tokens = rp.tile_tokens;
+    ap.short_group = rp.short_group;
+    ap.short_box_tokens = short_box_tokens;
     ap.scale_log2e = a->softmax_scale * 1.4426950408889634f;
     ap.out = a->out;
     ap.lse = a->lse;
@@ -626,12 +647,11 @@ vpp_status run_chunk_attn(const vpp_chunk_attn_args* a, vpp_stream_t stream_, co
     } else {
         // a second producer warp for launches bound by the arrival of K/V: pages smaller than a KV tile, batches of decode rows
         const bool v_warp = box_rows < vpp::kTileN || a->total_q <= a->num_reqs;
-        auto kern = pairs_two_heads(a) ? (v_warp ? vpp::attn128_ws_kernel<false, true> : vpp::attn128_ws_kernel<false, false>)
-                                       : (v_warp ? vpp::attn128_ws_kernel<true, true> : vpp::attn128_ws_kernel<true, false>);
+        auto kern = v_warp ? vpp::attn128_ws_kernel<true> : vpp::attn128_ws_kernel<false>;
         ce = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, vpp::kWsSmemBytes);
         if (ce == cudaSuccess)
-            ce = launch(kern, static_cast<unsigned>(sms), vpp::kWsThreads, vpp::kWsSmemBytes, stream, tm_q, tm_k, tm_v, tm_q2, tm_k2, tm_v2,
-                        tm_qh, ap, box_rows);
+            ce = launch(kern, static_cast<unsigned>(sms), vpp::kWsThreads, vpp::kWsSmemBytes, stream, tm_q, tm_k, tm_v, tm_k2, tm_v2, tm_qs,
+                        ap, box_rows);
     }
     if (ce != cudaSuccess) return fail(VPP_ERR_CUDA, "attention kernel attributes: %s", cudaGetErrorString(ce));
     ++g_launches;

@@ -278,9 +278,9 @@ attn_mla2_kernel(const __grid_constant__ CUtensorMap tm_q1, const __grid_constan
     // Items: (unit, q-head) for the units of several rows, then one item per single-token unit (the end of the list):
     // those run "packed" -- the q-heads are the rows of the tile (64 per CTA; they all share the one latent kv-head), so
     // the cache is streamed once per token instead of once per head.
-    const int num_packed = p.num_q_heads <= 2 * kMla2Rows && !error ? p.header_ro->num_single : 0;
+    const int num_packed = p.num_q_heads <= 2 * kMla2Rows && !error ? p.header_ro->num_short : 0;
     const int num_normal = num_units - num_packed;
-    const int normal_items = num_normal * p.num_q_heads;
+    const int normal_items = num_normal * p.num_q_heads, unit_block = p.header_ro->unit_block;
     const int total_items = normal_items + num_packed;
 
     // KV tiles (128 keys) of a unit: [kv_begin, min(kv_end, ceil((pos0 + rows) / 128)))
@@ -291,7 +291,7 @@ attn_mla2_kernel(const __grid_constant__ CUtensorMap tm_q1, const __grid_constan
     auto get_item = [&](int item, WorkUnit& u, int& h) -> bool {
         if (item < normal_items) {
             int ui;
-            decode_item(item, num_normal, p.num_q_heads, p.num_q_heads, ui, h);
+            decode_item(item, num_normal, unit_block, p.num_q_heads, p.num_q_heads, ui, h);
             u = p.units[ui];
         } else {
             u = p.units[num_normal + (item - normal_items)];

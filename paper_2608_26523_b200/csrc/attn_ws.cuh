@@ -5,17 +5,20 @@
 //               2-deep shared ring, loads the two Q tiles of the item and streams K/V pages through a
 //               ring of 128B-swizzled 32 KB stages (K0 V0 K1 V1 ...), gathered through the block table.
 //   warp 1      MMA issuer: tcgen05.mma  S_t = Q_t K^T  and  O_t += P_t V  for the two query tiles
-//               t = 0, 1 of the item: two q-heads of one kv-head over the same 128 query tokens (even
-//               group sizes) or, when a kv-head's group is odd (MHA included), two consecutive 128-row
-//               tiles of ONE q-head -- either way both tiles use the same K/V stages.
+//               t = 0, 1 of the item, which use the same K/V stages.
 //   warp 2      tensor-memory allocation.
 //   warps 4-7   softmax group for tile 0: one query row per thread, fp32 online softmax on S_0 read
 //               from tensor memory, P_0 written back to tensor memory as bf16 over S_0.
 //   warps 8-11  the same for tile 1.
 // While one group works on its S tile the tensor core runs the other tile's MMAs.
-// A work unit of a single query token (a decode step batched with prefill chunks, or the one-row tail of a chunk) is
-// run "packed": the G q-heads that share a kv-head become the rows of the Q tile, so its K/V is streamed once per
-// kv-head instead of once per pair of q-heads.  Both tiles then use that one Q tile and split the KV tiles between
+//
+// The rows of a tile are (token, q-head) pairs: `group` q-heads of one kv-head over `tile_tokens` consecutive tokens,
+// group * tile_tokens = 125 .. 128 (group = the whole group of a kv-head where that fills a tile; 1 for MHA, which gives
+// tiles of 128 tokens of one head).  A tile of few tokens wastes little on a ragged chunk: a request of 200 tokens with
+// groups of eight takes seven units of 32 tokens where tiles of 128 tokens of one head took 256 (32 ragged chunks of 8192
+// tokens together with 16 decode rows: 4.11 -> 3.50 ms).
+// A work unit whose (token, q-head) rows fill at most one tile -- a decode step, a few tokens, the tail of a chunk -- is
+// run "packed": both tiles of its item use that one Q tile and split the KV tiles between
 // them (even ones to tile 0, odd ones to tile 1) as two independent online softmaxes whose results softmax group 0
 // merges at the end -- one softmax chain per KV tile would leave the memory system idle most of the time.
 // Tensor memory: S_0 | S_1 | O_0 | O_1, 128 fp32 columns each (all 512 columns).
@@ -55,9 +58,9 @@ static_assert(kPartWaitDefer >= 1 && kPartWaitDefer <= 16, "the wait sits inside
 
 struct WsItem {
     WorkUnit u;
-    int32_t h0;      // first of the two q-heads (packed item: first head of the kv-head's group)
+    int32_t h0;      // first q-head of the item's rows
     int32_t valid;   // 0: no more work
-    int32_t packed;  // 1: single-token item, the rows of tile 0 are the G q-heads of one kv-head; tile 1 is unused
+    int32_t packed;  // 1: the rows fill at most tile 0; both tiles use it and split the KV tiles
     int32_t pad;
 };
 
@@ -66,16 +69,15 @@ struct WsItem {
 // registers):  out = (a0 O_0 + a1 O_1) / (a0 l_0 + a1 l_1),  a_t = 2^(m_t - m).  O_1 sits 128 columns after O_0.
 // (every argument by value: a reference to the kernel's parameter block or to the work unit would force them into
 // local memory for the whole kernel)
-__device__ __noinline__ void ws_packed_merge(void* out, float* lse_out, float* o_parts, float* lse_parts, int total_q,
-                                             int num_q_heads, int split, int q_row0, bool second, const float* xm,
-                                             uint32_t tO, int row, int tile_rows, int h, float m_ref, float l_run) {
+__device__ __noinline__ void ws_packed_merge(void* out, float* lse_out, float* o_parts, float* lse_parts, bool final,
+                                             long long out_row, bool second, const float* xm,
+                                             uint32_t tO, int row, int tile_rows, float m_ref, float l_run) {
     const float m1 = xm[row], l1 = xm[128 + row];
     const float m = fmaxf(m_ref, m1);
     const float a0 = m_ref == -INFINITY ? 0.f : ex2(m_ref - m), a1 = m1 == -INFINITY ? 0.f : ex2(m1 - m);
     const float l_tot = a0 * l_run + a1 * l1;
     const float s0 = a0 / l_tot, s1 = a1 / l_tot;
     const bool live = row < tile_rows;
-    const long long grow_idx = q_row0;
     uint32_t r[16], r1[16];
 #pragma unroll 1
     for (int c = 0; c < 8; ++c) {     // 16 output columns at a time (registers)
@@ -89,9 +91,8 @@ __device__ __noinline__ void ws_packed_merge(void* out, float* lse_out, float* o
             if (second) v = fmaf(__uint_as_float(r1[i]), s1, v);
             r[i] = __float_as_uint(v);
         }
-        if (split < 0) {
-            uint4* dst = reinterpret_cast<uint4*>(static_cast<uint8_t*>(out) +
-                                                  ((grow_idx * num_q_heads + h) * 128 + c * 16) * 2);
+        if (final) {
+            uint4* dst = reinterpret_cast<uint4*>(static_cast<uint8_t*>(out) + (out_row * 128 + c * 16) * 2);
 #pragma unroll
             for (int q4 = 0; q4 < 2; ++q4) {
                 uint32_t w[4];
@@ -101,9 +102,7 @@ __device__ __noinline__ void ws_packed_merge(void* out, float* lse_out, float* o
                 dst[q4] = make_uint4(w[0], w[1], w[2], w[3]);
             }
         } else {
-            float4* dst = reinterpret_cast<float4*>(
-                o_parts +
-                ((static_cast<long long>(split) * total_q + grow_idx) * num_q_heads + h) * 128 + c * 16);
+            float4* dst = reinterpret_cast<float4*>(o_parts + out_row * 128 + c * 16);
 #pragma unroll
             for (int q4 = 0; q4 < 4; ++q4)
                 dst[q4] = make_float4(__uint_as_float(r[q4 * 4]), __uint_as_float(r[q4 * 4 + 1]),
@@ -112,27 +111,23 @@ __device__ __noinline__ void ws_packed_merge(void* out, float* lse_out, float* o
     }
     if (live) {
         const float lse = (m + log2f(l_tot)) * 0.6931471805599453f;
-        if (split < 0) {
-            if (lse_out) lse_out[grow_idx * num_q_heads + h] = lse;
+        if (final) {
+            if (lse_out) lse_out[out_row] = lse;
         } else {
-            lse_parts[(static_cast<long long>(split) * total_q + grow_idx) * num_q_heads + h] = lse;
+            lse_parts[out_row] = lse;
         }
     }
 }
 
-template <bool kSameHead, bool kVWarp>
+template <bool kVWarp>
 __global__ void __launch_bounds__(kWsThreads, 1)
 attn128_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
-                  const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_q2,
-                  const __grid_constant__ CUtensorMap tm_k2, const __grid_constant__ CUtensorMap tm_v2,
-                  const __grid_constant__ CUtensorMap tm_qh, const AttnParams p, const int kv_box_rows) {
-    constexpr bool same_head = kSameHead;
-    // same_head: an item is two consecutive 128-row query tiles of one q-head (work units of up to 256 rows) instead of
-    // two q-heads over the same 128 rows -- for odd group sizes, where two q-heads need not share a kv-head.  Tile 1 then
-    // starts 128 rows (and positions) after tile 0; the KV range of the unit covers tile 1, and the causal mask hides
-    // from tile 0 what lies beyond its own rows.
-    // tm_qh: the q tensor with a box of (64 features, G heads, 1 token): the rows of a packed item's Q tile
-    // tm_q2 / tm_k2 / tm_v2 are views of the same tensors with the 128 features split into (64, 2): one box
+                  const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_k2,
+                  const __grid_constant__ CUtensorMap tm_v2, const __grid_constant__ CUtensorMap tm_qs, const AttnParams p,
+                  const int kv_box_rows) {
+    // tm_q:  q with a box of (64 features, group heads, tile_tokens tokens): one 64-column slab of a tile
+    // tm_qs: the same with (64, short_group, short_box_tokens), for packed items
+    // tm_k2 / tm_v2 are views of the caches with the 128 features split into (64, 2): one box
     // of them brings both 64-column slabs of a 128-row tile, i.e. a whole tile per copy instruction.  Issuing a
     // copy costs the producer thread several hundred cycles, so fewer, larger copies matter.  tm_k / tm_v
     // (one slab of kv_box_rows keys per box) serve pages smaller than a KV tile.
@@ -194,10 +189,9 @@ attn128_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
         prefetch_tmap(&tm_q);
         prefetch_tmap(&tm_k);
         prefetch_tmap(&tm_v);
-        prefetch_tmap(&tm_q2);
         prefetch_tmap(&tm_k2);
         prefetch_tmap(&tm_v2);
-        prefetch_tmap(&tm_qh);
+        prefetch_tmap(&tm_qs);
     }
     __syncthreads();
     if (warp == 2) {
@@ -215,13 +209,14 @@ attn128_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
     if (blockIdx.x == 0 && tid == 0 && p.status) *p.status = error;
     const int num_units = error ? 0 : p.header_ro->num_units;
     const int G = p.num_q_heads / p.num_kv_heads;
-    // Items: (unit, pair of q-heads) for the units of several rows, then (unit, kv-head) for the single-token units at the
-    // end of the list, which run packed when a kv-head's group fits a tile.
-    const int num_packed = G <= kTileM && !error ? p.header_ro->num_single : 0;
+    // Items: the short units' (unit, group of q-heads), which run packed (their groups are larger where a kv-head's group
+    // does not fill a tile well), then those of the units of two tiles.  The short units come first because decode rows
+    // sit at the end of long contexts: one of them started last would run alone.
+    const int num_packed = error ? 0 : p.header_ro->num_short;
     const int num_normal = num_units - num_packed;
-    const int heads_per_item = same_head ? 1 : 2;
-    const int normal_items = num_normal * (p.num_q_heads / heads_per_item);
-    const int total_items = normal_items + num_packed * p.num_kv_heads;
+    const int normal_slots = p.num_q_heads / p.group, packed_slots = p.num_q_heads / p.short_group;
+    const int packed_items = num_packed * packed_slots, unit_block = p.header_ro->unit_block;
+    const int total_items = packed_items + num_normal * normal_slots;
 
     if (warp < 4) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kWsRegsLow));
@@ -324,16 +319,15 @@ attn128_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                 WorkUnit u{};
                 int h0 = 0;
                 bool packed = false;
-                if (have && item < normal_items) {
-                    int ui, hp;
-                    decode_item(item, num_normal, p.num_q_heads / heads_per_item, G / heads_per_item, ui, hp);
-                    u = p.units[ui];
-                    h0 = heads_per_item * hp;
-                } else if (have) {
-                    const int k = item - normal_items;
-                    u = p.units[num_normal + k / p.num_kv_heads];
-                    h0 = (k % p.num_kv_heads) * G;
+                if (have && item < packed_items) {
+                    u = p.units[num_normal + item / packed_slots];
+                    h0 = (item % packed_slots) * p.short_group;
                     packed = true;
+                } else if (have) {
+                    int ui, hs;
+                    decode_item(item - packed_items, num_normal, unit_block, normal_slots, G / p.group, ui, hs);
+                    u = p.units[ui];
+                    h0 = hs * p.group;
                 }
                 const uint32_t slot = item_it & 1;
                 bool ok = true;
@@ -353,17 +347,19 @@ attn128_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
 
                 if (lane == 0) {
                     ok = mbar_wait(bar_q_empty, (q_it & 1) ^ 1, s_abort, 202);
+                    // (tokens past the end of q read as zero; rows of a following request are never stored; tile rows the
+                    // boxes do not cover keep whatever they held)
                     if (ok && packed) {
-                        // rows = the G heads of this kv-head for the one token; rows G..127 keep whatever they held
-                        mbar_arrive_expect_tx(bar_q_full, 2 * G * 128);
-                        tma_load_3d(sQ, &tm_qh, bar_q_full, 0, h0, u.q_row0);
-                        tma_load_3d(sQ + kSlabBytes, &tm_qh, bar_q_full, 64, h0, u.q_row0);
+                        mbar_arrive_expect_tx(bar_q_full, 2 * p.short_group * p.short_box_tokens * 128);
+                        tma_load_3d(sQ, &tm_qs, bar_q_full, 0, h0, u.q_row0);
+                        tma_load_3d(sQ + kSlabBytes, &tm_qs, bar_q_full, 64, h0, u.q_row0);
                     } else if (ok) {
-                        mbar_arrive_expect_tx(bar_q_full, 2 * kTileBytes);
-                        tma_load_4d(sQ, &tm_q2, bar_q_full, 0, u.q_row0, 0, h0);
-                        // (rows past the end of q read as zero; rows of a following request are never stored)
-                        tma_load_4d(sQ + kTileBytes, &tm_q2, bar_q_full, 0, u.q_row0 + (same_head ? kTileM : 0), 0,
-                                    h0 + (same_head ? 0 : 1));
+                        mbar_arrive_expect_tx(bar_q_full, 4 * p.group * p.tile_tokens * 128);
+#pragma unroll
+                        for (int t = 0; t < 2; ++t) {
+                            tma_load_3d(sQ + t * kTileBytes, &tm_q, bar_q_full, 0, h0, u.q_row0 + t * p.tile_tokens);
+                            tma_load_3d(sQ + t * kTileBytes + kSlabBytes, &tm_q, bar_q_full, 64, h0, u.q_row0 + t * p.tile_tokens);
+                        }
                     }
                 }
                 ok = __shfl_sync(0xffffffffu, ok, 0);
@@ -584,9 +580,13 @@ attn128_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
             if (!mbar_wait(bar_item_full + 8 * slot, (item_it >> 1) & 1, s_abort, 401)) break;
             const WorkUnit u = ring[slot].u;
             const bool packed = ring[slot].packed != 0;
-            // packed: row r of tile 0 is q-head h0 + r; otherwise tile t is q-head h0 + t, or rows 128 t .. of q-head h0
-            const int h = ring[slot].h0 + (packed ? row : (same_head ? 0 : t));
-            const int row_base = (!packed && same_head) ? t * kTileM : 0;
+            // this thread's row: token `tok` of the unit, q-head h0 + row % grp
+            const int grp = packed ? p.short_group : p.group;
+            const int tile_tok0 = packed ? 0 : t * p.tile_tokens;     // first token of the tile within the unit
+            const int tok = tile_tok0 + row / grp;
+            const int out_row0 = (u.q_row0 + tok) * p.num_q_heads + ring[slot].h0 + row % grp;   // its row of out / lse
+            const int tile_toks = packed || u.rows - tile_tok0 < p.tile_tokens ? u.rows - tile_tok0 : p.tile_tokens;
+            const int tile_rows = tile_toks * grp;                    // rows of this tile that exist (<= 0: none)
             const int valid = ring[slot].valid;
             __syncwarp();
             if (lane == 0) mbar_arrive(bar_item_empty + 8 * slot);
@@ -596,13 +596,11 @@ attn128_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
             // prefill path keeps the registers and the instruction count it had without it.
             auto run_item = [&](auto packed_tag) -> bool {
             constexpr bool kPacked = decltype(packed_tag)::value;
-            // rows of this thread's warp that exist: a packed tile has G rows, a warp without any only keeps the
-            // barriers moving
-            const int tile_rows = kPacked ? G : u.rows - row_base;   // (<= 0: tile 1 of a unit of at most 128 rows is idle)
-            const bool warp_idle = kPacked && (warp & 3) * 32 >= G;
+            // a warp of a packed tile without a row that exists only keeps the barriers moving
+            const bool warp_idle = kPacked && (warp & 3) * 32 >= tile_rows;
 
-            const int tile_pos0 = u.pos0 + row_base;               // position of the tile's first row
-            const int my_pos = kPacked ? u.pos0 : tile_pos0 + row;
+            const int tile_pos0 = u.pos0 + tile_tok0;              // position of the tile's first row
+            const int my_pos = u.pos0 + tok;
             float m_ref = -INFINITY, l_run = 0.f;
             bool ok = true;
             // a packed item: this group's tile takes every second KV tile
@@ -713,6 +711,8 @@ attn128_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                 ++o_it;
             }
             tc_fence_after();
+            // the row of out / lse, or of the partials (split, token, q-head)
+            const long long part_row = u.split < 0 ? out_row0 : static_cast<long long>(u.split) * p.total_q * p.num_q_heads + out_row0;
             if (kPacked && t == 1) {
                 // hand (m, l) of every row to group 0, which also reads O_1; wait until it is done with them
                 xm[row] = m_ref;
@@ -731,8 +731,8 @@ attn128_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                 if (!ok) return false;
                 ++x_it;
                 tc_fence_after();
-                ws_packed_merge(p.out, p.lse, p.o_parts, p.lse_parts, p.total_q, p.num_q_heads, u.split, u.q_row0,
-                                u.kv_begin + 1 < u.kv_end /* O_1 was written at all */, xm, tO, row, tile_rows, h, m_ref, l_run);
+                ws_packed_merge(p.out, p.lse, p.o_parts, p.lse_parts, u.split < 0, part_row,
+                                u.kv_begin + 1 < u.kv_end /* O_1 was written at all */, xm, tO, row, tile_rows, m_ref, l_run);
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(bar_x0);
@@ -741,7 +741,6 @@ attn128_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
             {
                 const float inv_l = 1.f / l_run;
                 const bool live = row < tile_rows;
-                const long long grow_idx = static_cast<long long>(u.q_row0) + row_base + row;
                 uint32_t r[32];
 #pragma unroll 1
                 for (int c = 0; c < 4; ++c) {
@@ -749,8 +748,7 @@ attn128_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                     tc_wait_ld();
                     if (!live) continue;
                     if (u.split < 0) {
-                        uint4* dst = reinterpret_cast<uint4*>(static_cast<uint8_t*>(p.out) +
-                                                              ((grow_idx * p.num_q_heads + h) * 128 + c * 32) * 2);
+                        uint4* dst = reinterpret_cast<uint4*>(static_cast<uint8_t*>(p.out) + (part_row * 128 + c * 32) * 2);
 #pragma unroll
                         for (int q4 = 0; q4 < 4; ++q4) {
                             uint32_t w[4];
@@ -761,9 +759,7 @@ attn128_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                             dst[q4] = make_uint4(w[0], w[1], w[2], w[3]);
                         }
                     } else {
-                        float4* dst = reinterpret_cast<float4*>(
-                            p.o_parts +
-                            ((static_cast<long long>(u.split) * p.total_q + grow_idx) * p.num_q_heads + h) * 128 + c * 32);
+                        float4* dst = reinterpret_cast<float4*>(p.o_parts + part_row * 128 + c * 32);
 #pragma unroll
                         for (int q4 = 0; q4 < 8; ++q4)
                             dst[q4] = make_float4(__uint_as_float(r[q4 * 4]) * inv_l, __uint_as_float(r[q4 * 4 + 1]) * inv_l,
@@ -774,9 +770,9 @@ attn128_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                 if (live) {
                     const float lse = (m_ref + log2f(l_run)) * 0.6931471805599453f;
                     if (u.split < 0) {
-                        if (p.lse) p.lse[grow_idx * p.num_q_heads + h] = lse;
+                        if (p.lse) p.lse[part_row] = lse;
                     } else {
-                        p.lse_parts[(static_cast<long long>(u.split) * p.total_q + grow_idx) * p.num_q_heads + h] = lse;
+                        p.lse_parts[part_row] = lse;
                     }
                 }
             }

@@ -8,12 +8,12 @@ namespace vpp {
 constexpr int kTileM = 128;  // query rows per MMA tile
 constexpr int kTileN = 128;  // keys per KV tile
 
-// One schedulable unit: a 128-row query tile of one request restricted to a range of KV tiles.
+// One schedulable unit: a run of consecutive query rows of one request restricted to a range of KV tiles.
 // The attention kernel turns (unit, head slot) pairs into work items.
 struct __align__(16) WorkUnit {
     int32_t req;        // request index
     int32_t q_row0;     // first packed query row of the tile
-    int32_t rows;       // valid rows in the unit (1..128; up to 256 when an item is two tiles of one q-head)
+    int32_t rows;       // query rows (tokens) of the unit
     int32_t pos0;       // absolute position of the tile's first row (prefix_len + row offset)
     int32_t kv_begin;   // first KV tile (units of kTileN keys)
     int32_t kv_end;     // one past the last KV tile
@@ -28,7 +28,8 @@ struct WorkHeader {
     int32_t num_units;    // units in the sorted list
     int32_t counter;      // persistent-kernel work counter
     int32_t error;        // VPP_DEV_* (0 = ok) of the lengths
-    int32_t num_single;   // the last num_single units of the list are single-token units (rows == 1)
+    int32_t num_short;    // the last num_short units of the list are the short ones: their rows fill at most one tile
+    int32_t unit_block;   // units per locality block of the item order (see decode_item)
     int32_t num_checkers; // blocks that checked a part of the block table
     int32_t bad_table[kMaxCheckers];   // one word each: VPP_DEV_BAD_BLOCK if it found an entry out of range, else 0
 };
@@ -60,6 +61,9 @@ struct AttnParams {
     int32_t num_q_heads;
     int32_t num_kv_heads;
     int32_t total_q;
+    // d = 128 kernel, how tile rows are packed: row r of a tile is q-head h0 + r % group of token r / group
+    int32_t group, tile_tokens;               // items of two tiles
+    int32_t short_group, short_box_tokens;    // items of one tile (short units); tokens a copy of its Q tile brings
     float scale_log2e;            // softmax_scale * log2(e)
     void* out;                    // bf16 [T, Hq, Dv]
     float* lse;                   // [T, Hq] or null
@@ -73,21 +77,20 @@ struct AttnParams {
 
 constexpr int kSlabBytes = kTileM * 128;  // 128 rows x 64 bf16, 128B-swizzled
 
-// Which (unit, kv-head, q-head) a flat work index means.  Units arrive sorted by decreasing cost; inside
-// a block of kUnitBlock consecutive units the items are ordered kv-head-major so that CTAs running at
-// the same time read the same K/V pages (L2 reuse), while blocks keep the longest-first order.
-constexpr int kUnitBlock = 32;
-__device__ __forceinline__ void decode_item(int w, int num_units, int items_per_unit, int per_kv_head, int& unit,
+// Which (unit, head slot) a flat work index means.  Units arrive sorted by decreasing cost; inside
+// a block of `unit_block` consecutive units the items are ordered kv-head-major so that CTAs
+// running at the same time read the same K/V pages (L2 reuse), while blocks keep the longest-first order.
+__device__ __forceinline__ void decode_item(int w, int num_units, int unit_block, int items_per_unit, int per_kv_head, int& unit,
                                             int& slot) {
-    const int blk_items = kUnitBlock * items_per_unit;
+    const int blk_items = unit_block * items_per_unit;
     const int ub = w / blk_items;
     const int rem = w - ub * blk_items;
-    const int left = num_units - ub * kUnitBlock;
-    const int nblk = left < kUnitBlock ? left : kUnitBlock;
+    const int left = num_units - ub * unit_block;
+    const int nblk = left < unit_block ? left : unit_block;
     const int per_g = nblk * per_kv_head;
     const int g = rem / per_g;
     const int rem2 = rem - g * per_g;
-    unit = ub * kUnitBlock + rem2 / per_kv_head;
+    unit = ub * unit_block + rem2 / per_kv_head;
     slot = g * per_kv_head + rem2 % per_kv_head;
 }
 

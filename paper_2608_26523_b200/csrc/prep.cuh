@@ -1,18 +1,21 @@
 // Work decomposition: from the per-request (prefix_len, chunk_len) on the device, build the list of
-// work units (query tile of 128 -- or 256 -- rows x key-range split) ordered by decreasing cost, so that the
+// work units (a run of query rows x key-range split) ordered by decreasing cost, so that the
 // persistent attention kernel can hand out tiles of very unequal cost longest-first.
 //
-// A query tile whose first row sits at absolute position pos0 needs the KV tiles
+// A unit whose first row sits at absolute position pos0 needs the KV tiles
 // [0, ceil((pos0 + rows) / 128)); its cost is that count -- it grows linearly with the prefix,
 // which is the per-chunk imbalance the paper's Eq. 2 models.
+//
+// Latency-bound (a launch of a few work items waits for it), so: one block of as many threads as the launch has units,
+// the requests' lengths and scans in shared memory, one scan for both prefix sums, two cost bins per thread.
 #pragma once
 #include "common.cuh"
 #include "ptx.cuh"
 
 namespace vpp {
 
-constexpr int kPrepThreads = 1024;
-constexpr int kCostBins = 2048;
+constexpr int kPrepMinThreads = 128, kPrepMaxThreads = 1024;
+constexpr int kPrepSmemReqs = 1024;   // up to so many requests the lengths and scans live in shared memory
 
 struct PrepParams {
     const int32_t* prefix_len;
@@ -26,8 +29,9 @@ struct PrepParams {
     int32_t num_blocks;
     int32_t splits;      // S >= 1
     int32_t max_units;
-    int32_t max_cost;    // ceil(max_seq_len / 128), >= 1
-    int32_t tile_m;      // query rows per unit: 128, or 256 when a work item is two 128-row tiles of one q-head
+    int32_t unit_rows;   // query rows per unit
+    int32_t short_rows;  // units of at most so many rows go to the end of the list (packed items)
+    int32_t unit_block, ragged_unit_block;   // units per locality block of the item order (common.cuh): about equally long units, others
     int32_t partial;     // 1: key-range restricted launch whose results are partial (o fp32, lse) of "split 0"
     int32_t range_begin; // first KV tile of the key range (partial launches)
     int32_t range_end;   // one past its last KV tile
@@ -38,36 +42,42 @@ struct PrepParams {
     int32_t* tile_start;  // [num_reqs + 1] scratch
 };
 
-// Exclusive scan of one value per thread over the block; returns the block total through `total`.
-__device__ __forceinline__ int block_exclusive_scan(int v, int* warp_sums, int& total) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int incl = v;
-#pragma unroll
+// Exclusive scan of two counts per thread over the block: (before a, before b, total a, total b).  Out of line and rolled up:
+// the kernel runs once through its code, which comes from far away, so its size is its latency.
+__device__ __noinline__ int4 block_scan2(int a, int b, int2* warp_sums) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    int ia = a, ib = b;
+#pragma unroll 1
     for (int o = 1; o < 32; o <<= 1) {
-        int t = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += t;
-    }
-    if (lane == 31) warp_sums[warp] = incl;
-    __syncthreads();
-    if (warp == 0) {
-        int w = warp_sums[lane];
-        int wi = w;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            int t = __shfl_up_sync(0xffffffffu, wi, o);
-            if (lane >= o) wi += t;
+        const int ta = __shfl_up_sync(0xffffffffu, ia, o), tb = __shfl_up_sync(0xffffffffu, ib, o);
+        if (lane >= o) {
+            ia += ta;
+            ib += tb;
         }
-        warp_sums[lane] = wi - w;          // exclusive warp offsets
-        if (lane == 31) warp_sums[32] = wi;  // block total
     }
+    if (lane == 31) warp_sums[warp] = make_int2(ia, ib);
     __syncthreads();
-    const int res = warp_sums[warp] + incl - v;
-    total = warp_sums[32];
+    // every warp scans the warp totals for itself
+    const int2 w = lane < nw ? warp_sums[lane] : make_int2(0, 0);
+    int wa = w.x, wb = w.y;
+#pragma unroll 1
+    for (int o = 1; o < 32; o <<= 1) {
+        const int ta = __shfl_up_sync(0xffffffffu, wa, o), tb = __shfl_up_sync(0xffffffffu, wb, o);
+        if (lane >= o) {
+            wa += ta;
+            wb += tb;
+        }
+    }
+    int4 r;
+    r.z = __shfl_sync(0xffffffffu, wa, 31);
+    r.w = __shfl_sync(0xffffffffu, wb, 31);
+    r.x = __shfl_sync(0xffffffffu, wa - w.x, warp) + ia - a;
+    r.y = __shfl_sync(0xffffffffu, wb - w.y, warp) + ib - b;
     __syncthreads();
-    return res;
+    return r;
 }
 
-// Number of key-range splits of the query tile whose first row is at absolute position pos0:
+// Number of key-range splits of the unit whose first row is at absolute position pos0:
 // every split must start at or before pos0 so that each row sees at least one key in each split.
 __device__ __forceinline__ int tile_num_splits(int pos0, int S) {
     const int splittable = pos0 / kTileN + 1;  // KV tiles that start at or before pos0
@@ -78,13 +88,6 @@ __device__ __forceinline__ void split_range(int pos0, int n_tiles, int nsplit, i
     const int splittable = pos0 / kTileN + 1;
     kb = static_cast<int>((static_cast<long long>(s) * splittable) / nsplit);
     ke = (s + 1 == nsplit) ? n_tiles : static_cast<int>((static_cast<long long>(s + 1) * splittable) / nsplit);
-}
-
-__device__ __forceinline__ int cost_bin(int cost, int max_cost) {
-    long long b = (static_cast<long long>(cost) * (kCostBins - 1)) / max_cost;
-    if (b > kCostBins - 1) b = kCostBins - 1;
-    if (b < 0) b = 0;
-    return kCostBins - 1 - static_cast<int>(b);  // bin 0 = most expensive
 }
 
 // Every block-table entry a request needs must name a real block.  A batch of decode rows over small pages needs a
@@ -120,273 +123,170 @@ __device__ __forceinline__ void check_block_table(const PrepParams& p, int check
     if (threadIdx.x == 0) p.header->bad_table[checker] = any ? 2 /* VPP_DEV_BAD_BLOCK */ : 0;
 }
 
-__global__ void __launch_bounds__(kPrepThreads, 1) prep_kernel(const PrepParams p) {
-    __shared__ int warp_sums[33];
-    __shared__ int bins[2 * kCostBins];   // [0, kCostBins): units of several rows; [kCostBins, ..): single-token units
-    __shared__ int s_error;
-    __shared__ int s_carry_q, s_carry_t;
-    const int tid = threadIdx.x;
+__global__ void __launch_bounds__(kPrepMaxThreads, 1) prep_kernel(const PrepParams p) {
+    __shared__ int2 warp_sums[32];
+    __shared__ int bins[2 * kPrepMaxThreads];   // blockDim.x bins of decreasing cost, then as many for the short units
+    __shared__ int s_P[kPrepSmemReqs], s_C[kPrepSmemReqs], s_q[kPrepSmemReqs], s_t[kPrepSmemReqs + 1];
+    __shared__ int s_error, s_max, s_min;
+    const int tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31;
     pdl_launch_dependents();   // the attention kernel may set itself up (barriers, tensor memory) while this runs
     pdl_wait();                // the lengths may come from the kernel launched just before; the workspace may be in use by it
     if (blockIdx.x > 0) {
         check_block_table(p, blockIdx.x - 1, gridDim.x - 1);
         return;
     }
+    const bool in_smem = p.num_reqs <= kPrepSmemReqs;
+    int* const qs = in_smem ? s_q : p.q_start;     // first packed row / first unit of every request
+    int* const ts = in_smem ? s_t : p.tile_start;
+    const int* const Ps = in_smem ? s_P : p.prefix_len;
+    const int* const Cs = in_smem ? s_C : p.chunk_len;
     if (tid == 0) {
-        p.header->num_checkers = gridDim.x - 1;
         s_error = 0;
-        s_carry_q = 0;
-        s_carry_t = 0;
+        s_max = 1;
+        s_min = 1 << 30;
+        p.header->num_checkers = gridDim.x - 1;
     }
-    for (int b = tid; b < 2 * kCostBins; b += kPrepThreads) bins[b] = 0;
+    bins[tid] = 0;
+    bins[nthr + tid] = 0;
     __syncthreads();
 
-    // ---- phase 1: validate lengths, scan chunk lengths and query-tile counts over requests ----
-    for (int base = 0; base < p.num_reqs; base += kPrepThreads) {
+    // ---- phase 1: validate lengths, scan chunk lengths and unit counts over requests ----
+    int carry_q = 0, carry_t = 0;
+#pragma unroll 1
+    for (int base = 0; base < p.num_reqs; base += nthr) {
         const int r = base + tid;
-        int c = 0, nt = 0;
+        int P = 0, c = 0;
         if (r < p.num_reqs) {
-            const int P = p.prefix_len[r];
+            P = p.prefix_len[r];
             c = p.chunk_len[r];
             // (a key range must start inside every request's prefix, so that each query row sees at least one of its keys)
             if (P < 0 || c < 0 || static_cast<long long>(P) + c > p.max_seq_len ||
                 (p.partial && c > 0 && P < p.range_begin * kTileN)) {
-                atomicExch(&s_error, 1 /* VPP_DEV_BAD_LENGTHS */);
+                s_error = 1;
                 c = 0;
             }
-            nt = (c + p.tile_m - 1) / p.tile_m;
+            if (c > 0) {
+                atomicMax(&s_max, (P + c + kTileN - 1) / kTileN);                                      // longest unit,
+                atomicMin(&s_min, (P + (c < p.unit_rows ? c : p.unit_rows) + kTileN - 1) / kTileN);   // shortest
+            }
         }
-        int tot_q, tot_t;
-        const int eq = block_exclusive_scan(c, warp_sums, tot_q);
-        const int et = block_exclusive_scan(nt, warp_sums, tot_t);
+        const int4 sc = block_scan2(c, (c + p.unit_rows - 1) / p.unit_rows, warp_sums);
         if (r < p.num_reqs) {
-            p.q_start[r] = s_carry_q + eq;
-            p.tile_start[r] = s_carry_t + et;
+            if (in_smem) {
+                s_P[r] = P;
+                s_C[r] = c;
+            }
+            qs[r] = carry_q + sc.x;
+            ts[r] = carry_t + sc.y;
         }
-        __syncthreads();
-        if (tid == 0) {
-            s_carry_q += tot_q;
-            s_carry_t += tot_t;
-        }
-        __syncthreads();
+        carry_q += sc.z;
+        carry_t += sc.w;
     }
-    const int total_tiles = s_carry_t;
-    if (tid == 0) {
-        p.q_start[p.num_reqs] = s_carry_q;
-        p.tile_start[p.num_reqs] = s_carry_t;
-        if (s_carry_q != p.total_q) s_error = 1;
-    }
+    const int total_units = carry_t;
+    if (tid == 0) ts[p.num_reqs] = total_units;
     __syncthreads();
-
-    if (s_error != 0) {
+    if (s_error != 0 || carry_q != p.total_q) {
         if (tid == 0) {
             p.header->num_units = 0;
-            p.header->num_single = 0;
+            p.header->num_short = 0;
             p.header->counter = 0;
-            p.header->error = s_error;
+            p.header->error = 1 /* VPP_DEV_BAD_LENGTHS */;
         }
         return;
     }
 
-    // ---- phases 2-4: counting sort of the units by decreasing cost ----
-    for (int pass = 0; pass < 2; ++pass) {
-        for (int gt = tid; gt < total_tiles; gt += kPrepThreads) {
-            // request of global query tile gt: last r with tile_start[r] <= gt
-            int lo = 0, hi = p.num_reqs - 1;
-            while (lo < hi) {
-                const int mid = (lo + hi + 1) >> 1;
-                if (p.tile_start[mid] <= gt) lo = mid; else hi = mid - 1;
+    // ---- phase 2: counting sort of the units by decreasing cost, two passes ----
+    float bin_scale = static_cast<float>(nthr - 1) / static_cast<float>(s_max);
+    const bool once = total_units <= nthr;   // (then this thread's unit is worked out once)
+    int r = 0, row_off = 0, rows = 0, pos0 = 0, n_tiles = 0, nsplit = 0;
+#pragma unroll 1
+    for (int pass = 1; pass < 3; ++pass) {
+#pragma unroll 1
+        for (int base = 0; base < total_units; base += nthr) {
+            const int gt = base + tid;
+            if (pass == 1 || !once) {
+                r = 0;
+                n_tiles = 0;
+                rows = 0;
+                nsplit = 0;
+                if (gt < total_units) {
+                    int hi = p.num_reqs - 1;          // request of unit gt: last r with ts[r] <= gt
+                    while (r < hi) {
+                        const int mid = (r + hi + 1) >> 1;
+                        if (ts[mid] <= gt) r = mid; else hi = mid - 1;
+                    }
+                    row_off = (gt - ts[r]) * p.unit_rows;
+                    rows = Cs[r] - row_off < p.unit_rows ? Cs[r] - row_off : p.unit_rows;
+                    pos0 = Ps[r] + row_off;
+                    n_tiles = (pos0 + rows + kTileN - 1) / kTileN;
+                }
             }
-            const int r = lo;
-            const int qt = gt - p.tile_start[r];
-            const int P = p.prefix_len[r], C = p.chunk_len[r];
-            const int row_off = qt * p.tile_m;
-            const int rows = (C - row_off) < p.tile_m ? (C - row_off) : p.tile_m;
-            const int pos0 = P + row_off;
-            const int n_tiles = (pos0 + rows + kTileN - 1) / kTileN;
-            const int nsplit = p.partial ? 1 : tile_num_splits(pos0, p.splits);
+            const bool is_short = rows <= p.short_rows;
+            if ((pass == 1 || !once) && n_tiles > 0) {
+                nsplit = p.partial ? 1 : tile_num_splits(pos0, p.splits);
+            }
+            int* const my_bins = bins + (is_short ? nthr : 0);
+            auto bin = [&](int n) {
+                const int b = nthr - 1 - static_cast<int>(static_cast<float>(n) * bin_scale);
+                return my_bins + (b < 0 ? 0 : b);
+            };
+            int slot = 0;
+            if (nsplit > 0) slot = atomicAdd(bin((n_tiles + nsplit - 1) / nsplit), nsplit);
+            if (pass == 1) continue;
+#pragma unroll 1
             for (int s = 0; s < nsplit; ++s) {
                 int kb, ke;
+                split_range(pos0, n_tiles, nsplit, s, kb, ke);
+                int at = slot + s;
                 if (p.partial) {
                     kb = p.range_begin;
                     ke = n_tiles < p.range_end ? n_tiles : p.range_end;
-                } else {
-                    split_range(pos0, n_tiles, nsplit, s, kb, ke);
                 }
-                // single-token units go to the end of the list (each part ordered by decreasing cost): the attention
-                // kernels may run them with the q-heads of a kv-head packed into one tile
-                const int bin = cost_bin(ke - kb, p.max_cost) + (rows == 1 ? kCostBins : 0);
-                if (pass == 0) {
-                    atomicAdd(&bins[bin], 1);
-                } else {
-                    const int slot = atomicAdd(&bins[bin], 1);
-                    if (slot < p.max_units) {
-                        WorkUnit u;
-                        u.req = r;
-                        u.q_row0 = p.q_start[r] + row_off;
-                        u.rows = rows;
-                        u.pos0 = pos0;
-                        u.kv_begin = kb;
-                        u.kv_end = ke;
-                        u.split = (nsplit > 1 || p.partial) ? s : -1;
-                        u.kv_len = P + C;
-                        p.units[slot] = u;
-                    }
+                if (at < p.max_units) {
+                    WorkUnit u;
+                    u.req = r;
+                    u.q_row0 = qs[r] + row_off;
+                    u.rows = rows;
+                    u.pos0 = pos0;
+                    u.kv_begin = kb;
+                    u.kv_end = ke;
+                    u.split = (nsplit > 1 || p.partial) ? s : -1;
+                    u.kv_len = Ps[r] + Cs[r];
+                    p.units[at] = u;
                 }
             }
-            if (pass == 1 && p.splits > 1) {
-                for (int i = 0; i < rows; ++i) p.row_splits[p.q_start[r] + row_off + i] = nsplit;
+            if (p.splits > 1) {
+                // per-row split counts: a unit of a few rows by its thread, a longer one by the whole warp
+                const int q0 = qs[r] + row_off;
+                if (rows <= 4)
+                    for (int i = 0; i < rows; ++i) p.row_splits[q0 + i] = nsplit;
+#pragma unroll 1
+                for (uint32_t todo = __ballot_sync(0xffffffffu, rows > 4); todo; todo &= todo - 1) {
+                    const int l = __ffs(todo) - 1;
+                    const int l_rows = __shfl_sync(0xffffffffu, rows, l), l_ns = __shfl_sync(0xffffffffu, nsplit, l),
+                              l_q0 = __shfl_sync(0xffffffffu, q0, l);
+#pragma unroll 1
+                    for (int i = lane; i < l_rows; i += 32) p.row_splits[l_q0 + i] = l_ns;
+                }
             }
         }
         __syncthreads();
-        if (pass == 0) {
-            // exclusive scan of the bins (bin 0 = most expensive first)
-            static_assert(2 * kCostBins == 4 * kPrepThreads, "four bins per thread");
-            const int b0 = bins[4 * tid], b1 = bins[4 * tid + 1], b2 = bins[4 * tid + 2], b3 = bins[4 * tid + 3];
-            int total;
-            const int ex = block_exclusive_scan(b0 + b1 + b2 + b3, warp_sums, total);
-            bins[4 * tid] = ex;
-            bins[4 * tid + 1] = ex + b0;
-            bins[4 * tid + 2] = ex + b0 + b1;
-            bins[4 * tid + 3] = ex + b0 + b1 + b2;
-            __syncthreads();
-            if (tid == 0) {
-                const int n = total < p.max_units ? total : p.max_units;
-                const int first_single = bins[kCostBins] < n ? bins[kCostBins] : n;
+        if (pass == 1) {
+            // exclusive scan of the bins, two per thread (bin 0 = most expensive first, the short units' bins last)
+            const int b0 = bins[2 * tid], b1 = bins[2 * tid + 1];
+            const int4 sc = block_scan2(b0 + b1, 0, warp_sums);
+            bins[2 * tid] = sc.x;
+            bins[2 * tid + 1] = sc.x + b0;
+            if (2 * tid == nthr) {   // the first of the short units' bins
+                const int n = sc.z < p.max_units ? sc.z : p.max_units;
                 p.header->num_units = n;
-                p.header->num_single = n - first_single;
+                p.header->num_short = n - (sc.x < n ? sc.x : n);
+                p.header->unit_block = 4 * s_min >= 3 * s_max ? p.unit_block : p.ragged_unit_block;
                 p.header->counter = 0;
                 p.header->error = 0;
             }
             __syncthreads();
         }
-    }
-}
-
-// The same decomposition for small launches (at most 32 requests and 32 query tiles: a short chunk, a small decode
-// batch), by ONE warp of block 0: a lane per request, then a lane per query tile, scans by shuffles, no block-wide
-// synchronisation, no sort -- the units of such a launch all start in the first wave of work items, so their order
-// does not matter (units of several rows first, single-token units last, as the attention kernels expect).  About a
-// third of the big kernel's latency, which is most of what a launch of a few work items costs.
-constexpr int kPrepSmallMax = 32;
-constexpr int kPrepSmallThreads = 256;   // (block 0 uses its first warp; the other blocks check the block table)
-
-__global__ void __launch_bounds__(kPrepSmallThreads, 1) prep_small_kernel(const PrepParams p) {
-    __shared__ int s_P[kPrepSmallMax], s_C[kPrepSmallMax], s_q0[kPrepSmallMax + 1], s_t0[kPrepSmallMax + 1];
-    const int lane = threadIdx.x;
-    pdl_launch_dependents();
-    pdl_wait();
-    if (blockIdx.x > 0) {
-        check_block_table(p, blockIdx.x - 1, gridDim.x - 1);
-        return;
-    }
-    if (lane >= 32) return;
-    if (lane == 0) p.header->num_checkers = gridDim.x - 1;
-    // ---- requests: validate, scan chunk lengths and tile counts ----
-    int P = 0, c = 0, nt = 0, bad = 0;
-    if (lane < p.num_reqs) {
-        P = p.prefix_len[lane];
-        c = p.chunk_len[lane];
-        if (P < 0 || c < 0 || static_cast<long long>(P) + c > p.max_seq_len ||
-            (p.partial && c > 0 && P < p.range_begin * kTileN)) {
-            bad = 1;
-            c = 0;
-        }
-        nt = (c + p.tile_m - 1) / p.tile_m;
-    }
-    int iq = c, it = nt;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int a = __shfl_up_sync(0xffffffffu, iq, o), b = __shfl_up_sync(0xffffffffu, it, o);
-        if (lane >= o) {
-            iq += a;
-            it += b;
-        }
-    }
-    const int total_q = __shfl_sync(0xffffffffu, iq, 31), total_tiles = __shfl_sync(0xffffffffu, it, 31);
-    if (lane < p.num_reqs) {
-        s_P[lane] = P;
-        s_C[lane] = c;
-        s_q0[lane] = iq - c;
-        s_t0[lane] = it - nt;
-        p.q_start[lane] = iq - c;
-        p.tile_start[lane] = it - nt;
-    }
-    if (lane == 0) {
-        s_t0[p.num_reqs] = total_tiles;
-        p.q_start[p.num_reqs] = total_q;
-        p.tile_start[p.num_reqs] = total_tiles;
-    }
-    const int error = __any_sync(0xffffffffu, bad) || total_q != p.total_q || total_tiles > kPrepSmallMax ? 1 : 0;
-    __syncwarp();
-    if (error != 0) {
-        if (lane == 0) {
-            p.header->num_units = 0;
-            p.header->num_single = 0;
-            p.header->counter = 0;
-            p.header->error = error;
-        }
-        return;
-    }
-    // ---- a lane per query tile: its units, placed by two scans (units of several rows, then single-token units) ----
-    int r = 0, rows = 0, pos0 = 0, n_tiles = 0, nsplit = 0, row_off = 0;
-    if (lane < total_tiles) {
-        while (s_t0[r + 1] <= lane) ++r;
-        row_off = (lane - s_t0[r]) * p.tile_m;
-        rows = s_C[r] - row_off < p.tile_m ? s_C[r] - row_off : p.tile_m;
-        pos0 = s_P[r] + row_off;
-        n_tiles = (pos0 + rows + kTileN - 1) / kTileN;
-        nsplit = p.partial ? 1 : tile_num_splits(pos0, p.splits);
-    }
-    const bool single = rows == 1;
-    int in = single ? 0 : nsplit, is = single ? nsplit : 0;
-    const int mine_n = in, mine_s = is;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int a = __shfl_up_sync(0xffffffffu, in, o), b = __shfl_up_sync(0xffffffffu, is, o);
-        if (lane >= o) {
-            in += a;
-            is += b;
-        }
-    }
-    const int total_n = __shfl_sync(0xffffffffu, in, 31), total_s = __shfl_sync(0xffffffffu, is, 31);
-    const int first = single ? total_n + is - mine_s : in - mine_n;
-    for (int s = 0; s < nsplit; ++s) {
-        int kb, ke;
-        if (p.partial) {
-            kb = p.range_begin;
-            ke = n_tiles < p.range_end ? n_tiles : p.range_end;
-        } else {
-            split_range(pos0, n_tiles, nsplit, s, kb, ke);
-        }
-        if (first + s < p.max_units) {
-            WorkUnit u;
-            u.req = r;
-            u.q_row0 = s_q0[r] + row_off;
-            u.rows = rows;
-            u.pos0 = pos0;
-            u.kv_begin = kb;
-            u.kv_end = ke;
-            u.split = (nsplit > 1 || p.partial) ? s : -1;
-            u.kv_len = s_P[r] + s_C[r];
-            p.units[first + s] = u;
-        }
-    }
-    if (p.splits > 1) {
-        // per-row split counts, written by the whole warp tile by tile
-        for (int t = 0; t < total_tiles; ++t) {
-            const int t_rows = __shfl_sync(0xffffffffu, rows, t), t_ns = __shfl_sync(0xffffffffu, nsplit, t);
-            const int t_q0 = __shfl_sync(0xffffffffu, lane < total_tiles ? s_q0[r] + row_off : 0, t);
-            for (int i = lane; i < t_rows; i += 32) p.row_splits[t_q0 + i] = t_ns;
-        }
-    }
-    if (lane == 0) {
-        const int n = total_n + total_s < p.max_units ? total_n + total_s : p.max_units;
-        const int first_single = total_n < n ? total_n : n;
-        p.header->num_units = n;
-        p.header->num_single = n - first_single;
-        p.header->counter = 0;
-        p.header->error = 0;
     }
 }
 
