@@ -269,9 +269,18 @@ vpp_status validate_pointers(const vpp_chunk_attn_args* a) {
     return VPP_OK;
 }
 
-// Upper bound on key-range splits per query tile for this launch.
-int choose_splits(const vpp_chunk_attn_args* a, int heads_per_item) {
-    if (a->num_kv_splits >= 1) return a->num_kv_splits;
+// Key-range splits of a launch: the most a work unit may get, and whether the work decomposition chooses each unit's own
+// number so that the KV tiles are shared out evenly over the SMs (prep.cuh) instead of cutting every unit into that many.
+struct SplitPlan {
+    int splits;
+    bool balanced;
+};
+// How the work decomposition counts work items of this launch.
+struct ItemCounts {
+    int unit_rows, unit_items, short_items, slots;
+};
+
+int uniform_splits(const vpp_chunk_attn_args* a, int heads_per_item) {
     const int group = a->num_q_heads / a->num_kv_heads;
     if (heads_per_item == 2 && a->total_q > 0 && a->total_q <= a->num_reqs && group <= vpp::kTileM) {
         // A decode batch of the d = 128 family: one packed item per (token, kv-head), all about max_seq_len long.  Equal
@@ -362,6 +371,46 @@ int heads_per_item(const vpp_chunk_attn_args* a, Family fam) {
     return even_groups(a) ? 2 : 1;
 }
 
+ItemCounts item_counts(const vpp_chunk_attn_args* a, Family fam) {
+    const int sms = sm_count_or_default();
+    if (fam == Family::kMla576) {
+        const bool packs = a->num_q_heads <= 2 * vpp::kMla2Rows;
+        return {vpp::kTileM, a->num_q_heads, packs ? 1 : a->num_q_heads, sms / 2 > 0 ? sms / 2 : 1};
+    }
+    const RowPacking r = row_packing(a);
+    return {r.unit_rows, a->num_q_heads / r.group, a->num_q_heads / r.short_group, sms};
+}
+
+constexpr int kMinLen = 2, kMinShortLen = 4;   // fewest KV tiles worth a work item (start-up ~4 us, ~2 / ~1 us per tile)
+
+SplitPlan plan_splits(const vpp_chunk_attn_args* a, Family fam) {
+    if (a->num_kv_splits >= 1) return {a->num_kv_splits, false};
+    if (a->total_q <= 0 || a->num_reqs <= 0) return {1, false};
+    // An upper bound on the work items of an uncut launch.  Where they fill the slots several times the dynamic longest-first
+    // order balances them well enough; where they do not, the shares are cut to measure.
+    const ItemCounts c = item_counts(a, fam);
+    const bool decode = a->total_q <= a->num_reqs;
+    const long long units = decode ? a->total_q : (a->total_q + c.unit_rows - 1) / c.unit_rows + (a->num_reqs > 1 ? a->num_reqs : 0);
+    const long long items = units * (decode ? c.short_items : c.unit_items);
+    const long long tiles = (a->max_seq_len + vpp::kTileN - 1) / vpp::kTileN;
+    // (one request, or a batch of decode rows, of the d = 128 family: from 80 % of the SMs on the split count that leaves the
+    //  least idle last wave, below; mixed batches and MLA: up to two items per slot)
+    const bool one_kind = decode || a->num_reqs == 1;
+    const bool few = fam == Family::kGqa128 && one_kind ? items * 5 < c.slots * 4ll : items < 2ll * c.slots;
+    if (few) {
+        // what a unit may need: its share of the slots when all are equally long; several times that when they are ragged (one
+        // long context among short ones gets most of the slots)
+        long long s = a->num_reqs == 1 ? (c.slots + items - 1) / items + 1 : (2ll * c.slots + items - 1) / items + 2;
+        const long long by_len = tiles / (decode ? kMinShortLen : kMinLen);
+        if (s > by_len) s = by_len;
+        if (s > vpp::kMergeMaxSplits) s = vpp::kMergeMaxSplits;
+        if (s < 2) return {1, false};
+        return {static_cast<int>(s), true};
+    }
+    if (fam == Family::kMla576) return {1, false};
+    return {uniform_splits(a, heads_per_item(a, fam)), false};
+}
+
 using MergeKernel = void (*)(const float*, const float*, int, long long, int, int, const int32_t*, const vpp::WorkHeader*, __nv_bfloat16*,
                              float*);
 // The kernel and the grid for a merge of `splits` partials of total_q x num_q_heads rows of head_dim_v features.
@@ -384,7 +433,7 @@ MergeKernel pick_merge_kernel(int splits, long long total_q, int num_q_heads, in
 
 vpp::WorkspaceLayout layout_for(const vpp_chunk_attn_args* a, Family fam) {
     vpp::WorkspaceLayout L{};
-    const int S = choose_splits(a, heads_per_item(a, fam));
+    const int S = plan_splits(a, fam).splits;
     const int unit_rows = unit_rows_of(a, fam);
     const long long tiles = (a->total_q + unit_rows - 1) / unit_rows + a->num_reqs;
     L.splits = S;
@@ -578,6 +627,16 @@ vpp_status run_chunk_attn(const vpp_chunk_attn_args* a, vpp_stream_t stream_, co
     pp.block_shift = paged ? ilog2(B) : 0;
     pp.num_blocks = n_blocks;
     pp.splits = L.splits;
+    {
+        const ItemCounts c = item_counts(a, fam);
+        pp.balanced = plan_splits(a, fam).balanced && L.splits > 1 ? 1 : 0;
+        pp.slots = c.slots;
+        pp.unit_items = c.unit_items;
+        pp.short_items = c.short_items;
+        pp.unit_weight = fam == Family::kMla576 ? 1 : 2;   // (a short unit's two tiles share its KV tiles)
+        pp.min_len = kMinLen;
+        pp.min_short_len = kMinShortLen;
+    }
     pp.max_units = L.max_units;
     pp.unit_rows = unit_rows_of(a, fam);
     pp.short_rows = fam == Family::kGqa128 ? rp.short_tokens : 1;

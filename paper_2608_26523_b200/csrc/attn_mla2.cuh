@@ -25,8 +25,9 @@
 // tcgen05.commit adds a bubble of ~90 clk.  Hence few commits (five per KV tile), each doubling as several
 // signals, and K / V handed back to the producers in groups (3 x 3 slabs, 2 x 32 KB) so that the copy of the
 // next tile overlaps the MMAs of this one although shared memory holds only one K and one V tile.
-// Pairs walk the work list round-robin (pair p takes items p, p + #pairs, ...), so the two CTAs of a pair agree
-// on the item sequence without exchanging anything.
+// Pairs walk the work list round-robin, every other round in reverse (the list is ordered by decreasing cost: who had the
+// longest item of a round gets the shortest of the next), so the two CTAs of a pair agree on the item sequence without
+// exchanging anything.
 // The math per row is the paper's Eq. 1 with the causal rule, KV tile by KV tile with a running maximum.
 #pragma once
 #include <type_traits>
@@ -275,13 +276,14 @@ attn_mla2_kernel(const __grid_constant__ CUtensorMap tm_q1, const __grid_constan
     const int num_units = error ? 0 : p.header_ro->num_units;
     const int num_pairs = gridDim.x >> 1;
     const int pair = blockIdx.x >> 1;
-    // Items: (unit, q-head) for the units of several rows, then one item per single-token unit (the end of the list):
-    // those run "packed" -- the q-heads are the rows of the tile (64 per CTA; they all share the one latent kv-head), so
-    // the cache is streamed once per token instead of once per head.
+    // Items: one per single-token unit (the end of the list): those run "packed" -- the q-heads are the rows of the tile (64 per
+    // CTA; they all share the one latent kv-head), so the cache is streamed once per token instead of once per head -- then
+    // (unit, q-head) for the units of several rows.
     const int num_packed = p.num_q_heads <= 2 * kMla2Rows && !error ? p.header_ro->num_short : 0;
     const int num_normal = num_units - num_packed;
-    const int normal_items = num_normal * p.num_q_heads, unit_block = p.header_ro->unit_block;
-    const int total_items = normal_items + num_packed;
+    const int total_items = num_packed + num_normal * p.num_q_heads, unit_block = p.header_ro->unit_block;
+    // the pair's item of a round (rounds alternate in direction)
+    auto item_of = [&](int round) { return round * num_pairs + ((round & 1) ? num_pairs - 1 - pair : pair); };
 
     // KV tiles (128 keys) of a unit: [kv_begin, min(kv_end, ceil((pos0 + rows) / 128)))
     auto tile_hi = [](const WorkUnit& u) {
@@ -289,13 +291,13 @@ attn_mla2_kernel(const __grid_constant__ CUtensorMap tm_q1, const __grid_constan
         return u.kv_end < need ? u.kv_end : need;
     };
     auto get_item = [&](int item, WorkUnit& u, int& h) -> bool {
-        if (item < normal_items) {
-            int ui;
-            decode_item(item, num_normal, unit_block, p.num_q_heads, p.num_q_heads, ui, h);
-            u = p.units[ui];
-        } else {
-            u = p.units[num_normal + (item - normal_items)];
+        if (item < num_packed) {
+            u = p.units[num_normal + item];
             h = 0;
+        } else {
+            int ui;
+            decode_item(item - num_packed, num_normal, unit_block, p.num_q_heads, p.num_q_heads, ui, h);
+            u = p.units[ui];
         }
         return true;
     };
@@ -342,7 +344,7 @@ attn_mla2_kernel(const __grid_constant__ CUtensorMap tm_q1, const __grid_constan
             const int np = 64 / kv_box_rows, pq = lane % np;
             uint32_t q_it = 0, kc = 0;
             bool ok = true;
-            for (int item = pair; item < total_items && ok; item += num_pairs) {
+            for (int round = 0, item = pair; item < total_items && ok; item = item_of(++round)) {
                 WorkUnit u;
                 int h;
                 if (!get_item(item, u, h)) continue;
@@ -385,7 +387,7 @@ attn_mla2_kernel(const __grid_constant__ CUtensorMap tm_q1, const __grid_constan
         } else if (lane == 0) {
             uint32_t q_it = 0, kc = 0, item_it = 0;
             bool ok = true;
-            for (int item = pair; item < total_items && ok; item += num_pairs) {
+            for (int round = 0, item = pair; item < total_items && ok; item = item_of(++round)) {
                 WorkUnit u;
                 int h;
                 if (!get_item(item, u, h)) continue;
@@ -428,7 +430,7 @@ attn_mla2_kernel(const __grid_constant__ CUtensorMap tm_q1, const __grid_constan
         uint32_t vc = 0, tails = 0;
         bool ok = true;
         const uint32_t own_v_full = leader ? bar_v_full : bar_v_local;
-        for (int item = pair; item < total_items && ok; item += num_pairs) {
+        for (int round = 0, item = pair; item < total_items && ok; item = item_of(++round)) {
             WorkUnit u;
             int h;
             if (!get_item(item, u, h)) continue;
@@ -539,7 +541,7 @@ attn_mla2_kernel(const __grid_constant__ CUtensorMap tm_q1, const __grid_constan
             tc_commit2(g < kKGroups - 1 ? bar_k_empty + 8 * g : bar_last, 3);
         };
         static_assert(kKGroups == 3, "one call per K group");
-        for (int item = pair; item < total_items && ok; item += num_pairs) {
+        for (int round = 0, item = pair; item < total_items && ok; item = item_of(++round)) {
             WorkUnit u;
             int h;
             if (!get_item(item, u, h)) continue;
@@ -593,7 +595,7 @@ attn_mla2_kernel(const __grid_constant__ CUtensorMap tm_q1, const __grid_constan
             tc_commit2(g < kVGroups - 1 ? bar_v_empty + 8 * g : bar_pv_done, 3);
         };
         static_assert(kVGroups == 2, "one call per V group");
-        for (int item = pair; item < total_items && ok; item += num_pairs) {
+        for (int round = 0, item = pair; item < total_items && ok; item = item_of(++round)) {
             WorkUnit u;
             int h;
             if (!get_item(item, u, h)) continue;
@@ -641,7 +643,7 @@ attn_mla2_kernel(const __grid_constant__ CUtensorMap tm_q1, const __grid_constan
             return true;
         };
         bool ok = true;
-        for (int item = pair; item < total_items && ok; item += num_pairs) {
+        for (int round = 0, item = pair; item < total_items && ok; item = item_of(++round)) {
             WorkUnit u;
             int h;
             if (!get_item(item, u, h)) continue;

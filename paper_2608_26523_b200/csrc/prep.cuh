@@ -32,6 +32,12 @@ struct PrepParams {
     int32_t unit_rows;   // query rows per unit
     int32_t short_rows;  // units of at most so many rows go to the end of the list (packed items)
     int32_t unit_block, ragged_unit_block;   // units per locality block of the item order (common.cuh): about equally long units, others
+    // Balanced cut (the library's own choice of splits for launches of few work items; see balanced_ranges):
+    int32_t balanced;    // 1: cut the launch's KV tiles into equal shares of the SMs, `splits` being the most a unit may get
+    int32_t slots;       // CTAs (or CTA pairs) that take work items
+    int32_t unit_items, short_items;      // work items of a unit and of a short unit
+    int32_t unit_weight;                  // cost of a KV tile of a unit's item, in those of a short unit's
+    int32_t min_len, min_short_len;       // fewest KV tiles worth a work item
     int32_t partial;     // 1: key-range restricted launch whose results are partial (o fp32, lse) of "split 0"
     int32_t range_begin; // first KV tile of the key range (partial launches)
     int32_t range_end;   // one past its last KV tile
@@ -123,6 +129,23 @@ __device__ __forceinline__ void check_block_table(const PrepParams& p, int check
     if (threadIdx.x == 0) p.header->bad_table[checker] = any ? 2 /* VPP_DEV_BAD_BLOCK */ : 0;
 }
 
+// Into how many equal ranges the KV tiles of a launch are cut when every unit has `items` work items (one per head slot):
+// the smallest number of rounds over the slots whose items fill at least 90 % of them.
+__device__ __forceinline__ int balanced_ranges(int slots, int items) {
+    int ranges = 1;
+    float best = 0.f;
+#pragma unroll 1
+    for (int k = 1; k <= 4 && best < 0.9f; ++k) {
+        const int r = k * slots / items;
+        const float fill = static_cast<float>(r * items) / static_cast<float>(k * slots);
+        if (r >= 1 && fill > best) {
+            best = fill;
+            ranges = r;
+        }
+    }
+    return ranges;
+}
+
 __global__ void __launch_bounds__(kPrepMaxThreads, 1) prep_kernel(const PrepParams p) {
     __shared__ int2 warp_sums[32];
     __shared__ int bins[2 * kPrepMaxThreads];   // blockDim.x bins of decreasing cost, then as many for the short units
@@ -195,16 +218,26 @@ __global__ void __launch_bounds__(kPrepMaxThreads, 1) prep_kernel(const PrepPara
         return;
     }
 
-    // ---- phase 2: counting sort of the units by decreasing cost, two passes ----
+    // ---- phase 2: counting sort of the units by decreasing cost, two passes; before them, for a balanced cut, one that
+    //      adds the KV tiles up: how many of them does a work item get? ----
+    // Units of one kind: their KV tiles laid end to end are cut at the multiples of `len`, so that every range is one slot's
+    // share and a unit is cut only where a share ends in it (few partial results).  Units of both kinds: each unit by itself
+    // into parts of at most its kind's share.
+    int sum = 0, sum_short = 0, len = 0, len_short = 0;
+    bool stream = false;
     float bin_scale = static_cast<float>(nthr - 1) / static_cast<float>(s_max);
-    const bool once = total_units <= nthr;   // (then this thread's unit is worked out once)
+    // this thread's unit, its parts: the first of `first` KV tiles, then `part` each, the last what is left (part = 0: equal parts)
+    const bool once = total_units <= nthr;   // (then both are worked out once)
     int r = 0, row_off = 0, rows = 0, pos0 = 0, n_tiles = 0, nsplit = 0;
+    int before = 0, first = 0, part = 0;
+    const int first_pass = p.balanced ? 0 : 1;
 #pragma unroll 1
-    for (int pass = 1; pass < 3; ++pass) {
+    for (int pass = first_pass; pass < 3; ++pass) {
+        int carry = 0;
 #pragma unroll 1
         for (int base = 0; base < total_units; base += nthr) {
             const int gt = base + tid;
-            if (pass == 1 || !once) {
+            if (pass == first_pass || !once) {
                 r = 0;
                 n_tiles = 0;
                 rows = 0;
@@ -222,22 +255,60 @@ __global__ void __launch_bounds__(kPrepMaxThreads, 1) prep_kernel(const PrepPara
                 }
             }
             const bool is_short = rows <= p.short_rows;
+            if (p.balanced && (pass == 0 || !once)) {
+                const int4 sc = block_scan2(is_short ? 0 : n_tiles, is_short ? n_tiles : 0, warp_sums);
+                before = carry + sc.x + sc.y;
+                carry += sc.z + sc.w;
+                if (pass == 0) {
+                    sum += sc.z;
+                    sum_short += sc.w;
+                }
+            }
+            if (pass == 0) continue;
             if ((pass == 1 || !once) && n_tiles > 0) {
                 nsplit = p.partial ? 1 : tile_num_splits(pos0, p.splits);
+                part = 0;
+                if (p.balanced) {
+                    const int most = nsplit, share = is_short ? len_short : len;
+                    if (stream) {
+                        const int least = share / 8 > 1 ? share / 8 : 1;    // no slivers: such a cut is left out
+                        first = share - before % share;
+                        if (first < least) first += share;
+                        const int last = min(n_tiles - least, pos0 / kTileN);   // (a part starts at or before the first row)
+                        nsplit = last >= first ? (last - first) / share + 2 : 1;
+                        if (nsplit > 1) part = share;
+                    } else {
+                        nsplit = (n_tiles + share - 1) / share;
+                    }
+                    if (nsplit > most) {
+                        nsplit = most;
+                        part = 0;
+                    }
+                }
             }
             int* const my_bins = bins + (is_short ? nthr : 0);
             auto bin = [&](int n) {
                 const int b = nthr - 1 - static_cast<int>(static_cast<float>(n) * bin_scale);
                 return my_bins + (b < 0 ? 0 : b);
             };
-            int slot = 0;
-            if (nsplit > 0) slot = atomicAdd(bin((n_tiles + nsplit - 1) / nsplit), nsplit);
+            const int ends = part > 0 ? 2 : 0;     // parts that are not of the common length
+            int slot = 0, slot_first = 0, slot_last = 0;
+            if (nsplit > ends) slot = atomicAdd(bin(part > 0 ? part : (n_tiles + nsplit - 1) / nsplit), nsplit - ends);
+            if (ends > 0) {
+                slot_first = atomicAdd(bin(first), 1);
+                slot_last = atomicAdd(bin(n_tiles - first - (nsplit - 2) * part), 1);
+            }
             if (pass == 1) continue;
 #pragma unroll 1
             for (int s = 0; s < nsplit; ++s) {
                 int kb, ke;
                 split_range(pos0, n_tiles, nsplit, s, kb, ke);
                 int at = slot + s;
+                if (part > 0) {
+                    kb = s == 0 ? 0 : first + (s - 1) * part;
+                    ke = s + 1 == nsplit ? n_tiles : first + s * part;
+                    at = s == 0 ? slot_first : s + 1 == nsplit ? slot_last : at - 1;
+                }
                 if (p.partial) {
                     kb = p.range_begin;
                     ke = n_tiles < p.range_end ? n_tiles : p.range_end;
@@ -271,6 +342,21 @@ __global__ void __launch_bounds__(kPrepMaxThreads, 1) prep_kernel(const PrepPara
             }
         }
         __syncthreads();
+        if (pass == 0) {
+            stream = sum == 0 || sum_short == 0;
+            if (stream) {
+                const int ranges = balanced_ranges(p.slots, sum ? p.unit_items : p.short_items), least = sum ? p.min_len : p.min_short_len;
+                len = (sum + sum_short + ranges - 1) / ranges;
+                if (len < least) len = least;
+                len_short = len;
+            } else {
+                const float share = (static_cast<float>(sum) * p.unit_items * p.unit_weight + static_cast<float>(sum_short) * p.short_items) / p.slots;
+                len = max(static_cast<int>(share / p.unit_weight) + 1, p.min_len);
+                len_short = max(static_cast<int>(share) + 1, p.min_short_len);
+            }
+            const int longest = max(len, len_short);
+            bin_scale = static_cast<float>(nthr - 1) / static_cast<float>(min(s_max, longest + longest / 8));
+        }
         if (pass == 1) {
             // exclusive scan of the bins, two per thread (bin 0 = most expensive first, the short units' bins last)
             const int b0 = bins[2 * tid], b1 = bins[2 * tid + 1];
