@@ -271,17 +271,16 @@ attn_mla2_kernel(const __grid_constant__ CUtensorMap tm_q1, const __grid_constan
 
     pdl_wait();                  // the work list comes from the work-decomposition kernel launched just before
     pdl_launch_dependents();
-    const int error = launch_error(p.header_ro);
-    if (blockIdx.x == 0 && tid == 0 && p.status) *p.status = error;
-    const int num_units = error ? 0 : p.header_ro->num_units;
+    const WorkList list = read_header(p.header_ro);
+    if (blockIdx.x == 0 && tid == 0 && p.status) *p.status = list.error;
     const int num_pairs = gridDim.x >> 1;
     const int pair = blockIdx.x >> 1;
     // Items: one per single-token unit (the end of the list): those run "packed" -- the q-heads are the rows of the tile (64 per
     // CTA; they all share the one latent kv-head), so the cache is streamed once per token instead of once per head -- then
     // (unit, q-head) for the units of several rows.
-    const int num_packed = p.num_q_heads <= 2 * kMla2Rows && !error ? p.header_ro->num_short : 0;
-    const int num_normal = num_units - num_packed;
-    const int total_items = num_packed + num_normal * p.num_q_heads, unit_block = p.header_ro->unit_block;
+    const int num_packed = p.num_q_heads <= 2 * kMla2Rows ? list.num_short : 0;
+    const int num_normal = list.num_units - num_packed;
+    const int total_items = num_packed + num_normal * p.num_q_heads, unit_block = list.unit_block;
     // the pair's item of a round (rounds alternate in direction)
     auto item_of = [&](int round) { return round * num_pairs + ((round & 1) ? num_pairs - 1 - pair : pair); };
 

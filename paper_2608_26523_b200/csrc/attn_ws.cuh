@@ -1,7 +1,7 @@
 // Warp-specialised persistent chunked-prefill attention kernel for head_dim 128 (MHA / GQA / MQA).
 //
 // One CTA per SM, 12 warps:
-//   warp 0      scheduler + TMA producer: pops work items from the global counter, publishes them in a
+//   warp 0      scheduler + TMA producer: takes work item blockIdx.x, then pops from the global counter, publishes them in a
 //               2-deep shared ring, loads the two Q tiles of the item and streams K/V pages through a
 //               ring of 128B-swizzled 32 KB stages (K0 V0 K1 V1 ...), gathered through the block table.
 //   warp 1      MMA issuer: tcgen05.mma  S_t = Q_t K^T  and  O_t += P_t V  for the two query tiles
@@ -205,17 +205,16 @@ attn128_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
 
     pdl_wait();                  // the work list comes from the work-decomposition kernel launched just before
     pdl_launch_dependents();     // (the merge kernel, if any, waits for this grid to finish in the same way)
-    const int error = launch_error(p.header_ro);
-    if (blockIdx.x == 0 && tid == 0 && p.status) *p.status = error;
-    const int num_units = error ? 0 : p.header_ro->num_units;
+    const WorkList list = read_header(p.header_ro);
+    if (blockIdx.x == 0 && tid == 0 && p.status) *p.status = list.error;
     const int G = p.num_q_heads / p.num_kv_heads;
     // Items: the short units' (unit, group of q-heads), which run packed (their groups are larger where a kv-head's group
     // does not fill a tile well), then those of the units of two tiles.  The short units come first because decode rows
     // sit at the end of long contexts: one of them started last would run alone.
-    const int num_packed = error ? 0 : p.header_ro->num_short;
-    const int num_normal = num_units - num_packed;
+    const int num_packed = list.num_short;
+    const int num_normal = list.num_units - num_packed;
     const int normal_slots = p.num_q_heads / p.group, packed_slots = p.num_q_heads / p.short_group;
-    const int packed_items = num_packed * packed_slots, unit_block = p.header_ro->unit_block;
+    const int packed_items = num_packed * packed_slots, unit_block = list.unit_block;
     const int total_items = packed_items + num_normal * normal_slots;
 
     if (warp < 4) {
@@ -312,9 +311,11 @@ attn128_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
             // ============================ scheduler + TMA producer ============================
             uint32_t item_it = 0, q_it = 0, kv_it = 0, vfix_cnt = 0;
             while (true) {
-                int item = 0;
-                if (lane == 0) item = atomicAdd(&p.header->counter, 1);
-                item = __shfl_sync(0xffffffffu, item, 0);
+                int item = blockIdx.x;     // (the first without a round trip to the counter)
+                if (item_it > 0) {
+                    if (lane == 0) item = gridDim.x + atomicAdd(&p.header->counter, 1);
+                    item = __shfl_sync(0xffffffffu, item, 0);
+                }
                 const bool have = item < total_items;
                 WorkUnit u{};
                 int h0 = 0;

@@ -23,23 +23,33 @@ struct __align__(16) WorkUnit {
 
 constexpr int kMaxCheckers = 8;   // blocks of the work-decomposition kernel that check the block table
 
-// Head of the workspace; written by the work-decomposition kernel.
-struct WorkHeader {
+// Head of the workspace; written by the work-decomposition kernel, read in one go (read_header).
+struct __align__(16) WorkHeader {
     int32_t num_units;    // units in the sorted list
-    int32_t counter;      // persistent-kernel work counter
-    int32_t error;        // VPP_DEV_* (0 = ok) of the lengths
     int32_t num_short;    // the last num_short units of the list are the short ones: their rows fill at most one tile
     int32_t unit_block;   // units per locality block of the item order (see decode_item)
+    int32_t error;        // VPP_DEV_* (0 = ok) of the lengths
+    int32_t counter;      // persistent-kernel work counter
     int32_t num_checkers; // blocks that checked a part of the block table
+    int32_t pad[2];
     int32_t bad_table[kMaxCheckers];   // one word each: VPP_DEV_BAD_BLOCK if it found an entry out of range, else 0
 };
+static_assert(kMaxCheckers == 8, "read_header");
 
-// What the checks of the work decomposition found (0 = ok): the kernels after it do nothing when it is not 0.
-__device__ __forceinline__ int launch_error(const WorkHeader* h) {
-    int e = h->error;
-    const int n = h->num_checkers;
-    for (int i = 0; i < n && e == 0; ++i) e = h->bad_table[i];
-    return e;
+// The head of the work list as the kernels after the decomposition see it: nothing to do when a check failed.
+struct WorkList {
+    int32_t num_units, num_short, unit_block, error;
+};
+__device__ __forceinline__ WorkList read_header(const WorkHeader* h) {
+    const int4* q = reinterpret_cast<const int4*>(h);
+    const int4 a = q[0], b = q[1], c = q[2], d = q[3];   // (independent loads: one round trip)
+    const int bad[8] = {c.x, c.y, c.z, c.w, d.x, d.y, d.z, d.w};
+    WorkList w{a.x, a.y, a.z, a.w};
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+        if (w.error == 0 && i < b.y) w.error = bad[i];
+    if (w.error != 0) w.num_units = w.num_short = 0;
+    return w;
 }
 
 struct WorkspaceLayout {

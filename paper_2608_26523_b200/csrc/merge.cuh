@@ -30,7 +30,7 @@ lse_merge_kernel(const float* __restrict__ o_parts, const float* __restrict__ ls
                  const WorkHeader* header, __nv_bfloat16* __restrict__ out, float* __restrict__ lse) {
     pdl_launch_dependents();
     pdl_wait();   // partials come from the attention kernel launched just before
-    if (header != nullptr && launch_error(header) != 0) return;   // (nothing was computed and row_splits was not written)
+    if (header != nullptr && read_header(header).error != 0) return;   // (nothing was computed and row_splits was not written)
     const long long n_pairs = total_q * num_q_heads;
     const int lane = threadIdx.x & 31;
     const long long warps_total = static_cast<long long>(gridDim.x) * (kMergeThreads / 32);
@@ -132,7 +132,7 @@ lse_merge_small_kernel(const float* __restrict__ o_parts, const float* __restric
                        const WorkHeader* header, __nv_bfloat16* __restrict__ out, float* __restrict__ lse) {
     pdl_launch_dependents();
     pdl_wait();   // partials come from the attention kernel launched just before
-    if (header != nullptr && launch_error(header) != 0) return;   // (nothing was computed and row_splits was not written)
+    if (header != nullptr && read_header(header).error != 0) return;   // (nothing was computed and row_splits was not written)
     const long long n_pairs = total_q * num_q_heads;
     const uint32_t per_row = static_cast<uint32_t>(head_dim_v) >> 2;            // 16-byte pieces per output row
     const uint32_t n_pieces = static_cast<uint32_t>(n_pairs) * per_row;

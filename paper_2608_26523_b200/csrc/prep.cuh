@@ -92,8 +92,9 @@ __device__ __forceinline__ int tile_num_splits(int pos0, int S) {
 
 __device__ __forceinline__ void split_range(int pos0, int n_tiles, int nsplit, int s, int& kb, int& ke) {
     const int splittable = pos0 / kTileN + 1;
-    kb = static_cast<int>((static_cast<long long>(s) * splittable) / nsplit);
-    ke = (s + 1 == nsplit) ? n_tiles : static_cast<int>((static_cast<long long>(s + 1) * splittable) / nsplit);
+    // (at most 64 splits of at most 2^24 tiles: 32 bits are enough, and a division of 64 is the longest step of a small launch)
+    kb = static_cast<uint32_t>(s) * splittable / static_cast<uint32_t>(nsplit);
+    ke = (s + 1 == nsplit) ? n_tiles : static_cast<uint32_t>(s + 1) * splittable / static_cast<uint32_t>(nsplit);
 }
 
 // Every block-table entry a request needs must name a real block.  A batch of decode rows over small pages needs a
@@ -301,17 +302,16 @@ __global__ void __launch_bounds__(kPrepMaxThreads, 1) prep_kernel(const PrepPara
             if (pass == 1) continue;
 #pragma unroll 1
             for (int s = 0; s < nsplit; ++s) {
-                int kb, ke;
-                split_range(pos0, n_tiles, nsplit, s, kb, ke);
-                int at = slot + s;
+                int kb, ke, at = slot + s;
                 if (part > 0) {
                     kb = s == 0 ? 0 : first + (s - 1) * part;
                     ke = s + 1 == nsplit ? n_tiles : first + s * part;
                     at = s == 0 ? slot_first : s + 1 == nsplit ? slot_last : at - 1;
-                }
-                if (p.partial) {
+                } else if (p.partial) {
                     kb = p.range_begin;
                     ke = n_tiles < p.range_end ? n_tiles : p.range_end;
+                } else {
+                    split_range(pos0, n_tiles, nsplit, s, kb, ke);
                 }
                 if (at < p.max_units) {
                     WorkUnit u;
