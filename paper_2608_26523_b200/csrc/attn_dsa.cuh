@@ -581,29 +581,48 @@ dsa_attn_kernel(const __grid_constant__ CUtensorMap tm_qh, const __grid_constant
             const bool live = h < p.num_q_heads;
             // row of out / lse, or of the partials (part, token, q-head)
             const long long out_row = (kParts ? static_cast<long long>(item - t * p.splits) * p.total_q + t : t) * p.num_q_heads + h;
-            uint32_t r[32];
+            constexpr int row_step = 1;                           // the warp's 32 rows: consecutive q-heads
+            const int warp_rows = p.num_q_heads - (h - lane);
+            const long long first_row = out_row - lane;
+            // (P V of the last tile is done, so the warp's own rows of P serve as the stage of its stores)
+            uint8_t* const stage = p_row - lane * 128;
+            if (!kParts) {
 #pragma unroll 1
-            for (int c = 0; c < 8; ++c) {
-                tmem_ld32((c < 4 ? tO0 : tO1) + (c & 3) * 32, r);
-                tc_wait_ld();
-                if (!live) continue;
-                const int col0 = (c >> 2) * 256 + half * 128 + (c & 3) * 32;
-                if (!kParts) {
-                    uint4* dst = reinterpret_cast<uint4*>(static_cast<uint8_t*>(p.out) + (out_row * kMlaDv + col0) * 2);
+                for (int k = 0; k < 4; ++k) {     // 64 bf16 columns of 32 rows
 #pragma unroll
-                    for (int q4 = 0; q4 < 4; ++q4) {
-                        uint32_t w[4];
+                    for (int hf = 0; hf < 2; ++hf) {
+                        uint32_t r[32];
+                        tmem_ld32((k < 2 ? tO0 : tO1) + (k & 1) * 64 + hf * 32, r);
+                        tc_wait_ld();
 #pragma unroll
-                        for (int e = 0; e < 4; ++e)
-                            w[e] = pack_bf16x2(__uint_as_float(r[q4 * 8 + 2 * e]) * inv_l, __uint_as_float(r[q4 * 8 + 2 * e + 1]) * inv_l);
-                        dst[q4] = make_uint4(w[0], w[1], w[2], w[3]);
+                        for (int q4 = 0; q4 < 4; ++q4) {
+                            uint32_t w[4];
+#pragma unroll
+                            for (int e = 0; e < 4; ++e)
+                                w[e] = pack_bf16x2(__uint_as_float(r[q4 * 8 + 2 * e]) * inv_l, __uint_as_float(r[q4 * 8 + 2 * e + 1]) * inv_l);
+                            stage_put(stage, lane, hf * 4 + q4, make_uint4(w[0], w[1], w[2], w[3]));
+                        }
                     }
-                } else {
-                    float4* dst = reinterpret_cast<float4*>(p.o_parts + out_row * kMlaDv + col0);
+                    stage_flush(stage, lane, [&](int i) -> uint8_t* {
+                        return i < warp_rows ? static_cast<uint8_t*>(p.out) + ((first_row + i * row_step) * kMlaDv + (k >> 1) * 256 + half * 128 + (k & 1) * 64) * 2
+                                             : nullptr;
+                    });
+                }
+            } else {
+#pragma unroll 1
+                for (int c = 0; c < 8; ++c) {     // 32 fp32 columns of 32 rows
+                    uint32_t r[32];
+                    tmem_ld32((c < 4 ? tO0 : tO1) + (c & 3) * 32, r);
+                    tc_wait_ld();
 #pragma unroll
                     for (int q4 = 0; q4 < 8; ++q4)
-                        dst[q4] = make_float4(__uint_as_float(r[q4 * 4]) * inv_l, __uint_as_float(r[q4 * 4 + 1]) * inv_l,
-                                              __uint_as_float(r[q4 * 4 + 2]) * inv_l, __uint_as_float(r[q4 * 4 + 3]) * inv_l);
+                        stage_put(stage, lane, q4,
+                                  make_uint4(__float_as_uint(__uint_as_float(r[q4 * 4]) * inv_l), __float_as_uint(__uint_as_float(r[q4 * 4 + 1]) * inv_l),
+                                             __float_as_uint(__uint_as_float(r[q4 * 4 + 2]) * inv_l), __float_as_uint(__uint_as_float(r[q4 * 4 + 3]) * inv_l)));
+                    stage_flush(stage, lane, [&](int i) -> uint8_t* {
+                        return i < warp_rows ? reinterpret_cast<uint8_t*>(p.o_parts + (first_row + i * row_step) * kMlaDv + (c >> 2) * 256 + half * 128 + (c & 3) * 32)
+                                             : nullptr;
+                    });
                 }
             }
             if (live && half == 0) {

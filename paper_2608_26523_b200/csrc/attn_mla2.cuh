@@ -749,43 +749,56 @@ attn_mla2_kernel(const __grid_constant__ CUtensorMap tm_q1, const __grid_constan
             tc_fence_after();
             const float inv_l = 1.f / l_tot;
             const bool live = packed ? my_row < p.num_q_heads : my_row < u.rows;
-            const long long grow_idx = static_cast<long long>(u.q_row0) + (packed ? 0 : my_row);
-            uint32_t r[32];
+            // row of out / lse, or of the partials (split, token, q-head), of this thread
+            const long long out_row = ((u.split < 0 ? 0ll : static_cast<long long>(u.split) * p.total_q) + u.q_row0 + (packed ? 0 : my_row)) * p.num_q_heads + h;
+            // the warp's 32 rows: consecutive q-heads of a packed tile, otherwise one head of consecutive tokens
+            const int row_step = packed ? 1 : p.num_q_heads, warp_rows = (packed ? p.num_q_heads : u.rows) - (my_row - lane);
+            const long long first_row = out_row - static_cast<long long>(lane) * row_step;
+            // (P V of the last tile is done, so the warp's own rows of P serve as the stage of its stores)
+            uint8_t* const stage = p_row - lane * 128;
+            if (u.split < 0) {
 #pragma unroll 1
-            for (int c = 0; c < 8; ++c) {
-                tmem_ld32((c < 4 ? tO0 : tO1) + (c & 3) * 32, r);
-                tc_wait_ld();
-                if (!live) continue;
-                const int col0 = (c >> 2) * 256 + half * 128 + (c & 3) * 32;
-                if (u.split < 0) {
-                    uint4* dst = reinterpret_cast<uint4*>(static_cast<uint8_t*>(p.out) +
-                                                          ((grow_idx * p.num_q_heads + h) * kMlaDv + col0) * 2);
+                for (int k = 0; k < 4; ++k) {     // 64 bf16 columns of 32 rows
 #pragma unroll
-                    for (int q4 = 0; q4 < 4; ++q4) {
-                        uint32_t w[4];
+                    for (int hf = 0; hf < 2; ++hf) {
+                        uint32_t r[32];
+                        tmem_ld32((k < 2 ? tO0 : tO1) + (k & 1) * 64 + hf * 32, r);
+                        tc_wait_ld();
 #pragma unroll
-                        for (int e = 0; e < 4; ++e)
-                            w[e] = pack_bf16x2(__uint_as_float(r[q4 * 8 + 2 * e]) * inv_l,
-                                               __uint_as_float(r[q4 * 8 + 2 * e + 1]) * inv_l);
-                        dst[q4] = make_uint4(w[0], w[1], w[2], w[3]);
+                        for (int q4 = 0; q4 < 4; ++q4) {
+                            uint32_t w[4];
+#pragma unroll
+                            for (int e = 0; e < 4; ++e)
+                                w[e] = pack_bf16x2(__uint_as_float(r[q4 * 8 + 2 * e]) * inv_l, __uint_as_float(r[q4 * 8 + 2 * e + 1]) * inv_l);
+                            stage_put(stage, lane, hf * 4 + q4, make_uint4(w[0], w[1], w[2], w[3]));
+                        }
                     }
-                } else {
-                    float4* dst = reinterpret_cast<float4*>(
-                        p.o_parts + ((static_cast<long long>(u.split) * p.total_q + grow_idx) * p.num_q_heads + h) * kMlaDv +
-                        col0);
+                    stage_flush(stage, lane, [&](int i) -> uint8_t* {
+                        return i < warp_rows ? static_cast<uint8_t*>(p.out) + ((first_row + i * row_step) * kMlaDv + (k >> 1) * 256 + half * 128 + (k & 1) * 64) * 2
+                                             : nullptr;
+                    });
+                }
+            } else {
+#pragma unroll 1
+                for (int c = 0; c < 8; ++c) {     // 32 fp32 columns of 32 rows
+                    uint32_t r[32];
+                    tmem_ld32((c < 4 ? tO0 : tO1) + (c & 3) * 32, r);
+                    tc_wait_ld();
 #pragma unroll
                     for (int q4 = 0; q4 < 8; ++q4)
-                        dst[q4] = make_float4(__uint_as_float(r[q4 * 4]) * inv_l, __uint_as_float(r[q4 * 4 + 1]) * inv_l,
-                                              __uint_as_float(r[q4 * 4 + 2]) * inv_l, __uint_as_float(r[q4 * 4 + 3]) * inv_l);
+                        stage_put(stage, lane, q4,
+                                  make_uint4(__float_as_uint(__uint_as_float(r[q4 * 4]) * inv_l), __float_as_uint(__uint_as_float(r[q4 * 4 + 1]) * inv_l),
+                                             __float_as_uint(__uint_as_float(r[q4 * 4 + 2]) * inv_l), __float_as_uint(__uint_as_float(r[q4 * 4 + 3]) * inv_l)));
+                    stage_flush(stage, lane, [&](int i) -> uint8_t* {
+                        return i < warp_rows ? reinterpret_cast<uint8_t*>(p.o_parts + (first_row + i * row_step) * kMlaDv + (c >> 2) * 256 + half * 128 + (c & 3) * 32)
+                                             : nullptr;
+                    });
                 }
             }
             if (live && half == 0) {
                 const float lse = (m_ref + log2f(l_tot)) * 0.6931471805599453f;
-                if (u.split < 0) {
-                    if (p.lse) p.lse[grow_idx * p.num_q_heads + h] = lse;
-                } else {
-                    p.lse_parts[(static_cast<long long>(u.split) * p.total_q + grow_idx) * p.num_q_heads + h] = lse;
-                }
+                if (u.split >= 0) p.lse_parts[out_row] = lse;
+                else if (p.lse) p.lse[out_row] = lse;
             }
             tc_fence_before();
         }

@@ -45,7 +45,9 @@ constexpr int kTileBytes = 2 * kSlabBytes;    // one 128 x 128 bf16 tile
 // (the two alternating slots of the V-tail barrier cover a producer that runs at most two V tiles ahead of the MMA thread:
 //  a ring of more than four stages would need more slots -- five stages failed parity on short items)
 static_assert(kWsStages <= 4, "V-tail barrier slots");
-constexpr int kWsSmemBytes = 2 * kTileBytes + kWsStages * kTileBytes + 1024 /*align*/ + 2048 /*barriers, ring, merge exchange*/;
+constexpr int kWsStageBytes = 8 * 32 * 128;   // 4 KB per softmax warp for the epilogue's stores
+constexpr int kWsSmemBytes = 2 * kTileBytes + kWsStages * kTileBytes + 1024 /*align*/ + 2048 /*barriers, ring, merge exchange*/ + kWsStageBytes;
+static_assert(kWsSmemBytes <= 232448, "shared memory of one CTA");
 constexpr float kRescaleThreshold = 8.f;      // log2 units
 // 0: P is handed to the MMA thread whole; c in 1..3: the first 32*c key columns are handed over early so that
 // O += P V can start on them while the rest of the exponentials are computed
@@ -742,30 +744,48 @@ attn128_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
             {
                 const float inv_l = 1.f / l_run;
                 const bool live = row < tile_rows;
-                uint32_t r[32];
+                // whole runs of 128 bytes: 64 bf16 or 32 fp32 columns of the warp's 32 rows at a time
+                uint8_t* const stage = gen_bar + 2048 + (warp - 4) * 4096;
+                const int warp_row0 = (warp & 3) * 32;
+                if (u.split < 0) {
 #pragma unroll 1
-                for (int c = 0; c < 4; ++c) {
-                    tmem_ld32(tO + c * 32, r);
-                    tc_wait_ld();
-                    if (!live) continue;
-                    if (u.split < 0) {
-                        uint4* dst = reinterpret_cast<uint4*>(static_cast<uint8_t*>(p.out) + (part_row * 128 + c * 32) * 2);
+                    for (int c = 0; c < 2; ++c) {
 #pragma unroll
-                        for (int q4 = 0; q4 < 4; ++q4) {
-                            uint32_t w[4];
+                        for (int hf = 0; hf < 2; ++hf) {
+                            uint32_t r[32];
+                            tmem_ld32(tO + c * 64 + hf * 32, r);
+                            tc_wait_ld();
 #pragma unroll
-                            for (int e = 0; e < 4; ++e)
-                                w[e] = pack_bf16x2(__uint_as_float(r[q4 * 8 + 2 * e]) * inv_l,
-                                                   __uint_as_float(r[q4 * 8 + 2 * e + 1]) * inv_l);
-                            dst[q4] = make_uint4(w[0], w[1], w[2], w[3]);
+                            for (int q4 = 0; q4 < 4; ++q4) {
+                                uint32_t w[4];
+#pragma unroll
+                                for (int e = 0; e < 4; ++e)
+                                    w[e] = pack_bf16x2(__uint_as_float(r[q4 * 8 + 2 * e]) * inv_l,
+                                                       __uint_as_float(r[q4 * 8 + 2 * e + 1]) * inv_l);
+                                stage_put(stage, lane, hf * 4 + q4, make_uint4(w[0], w[1], w[2], w[3]));
+                            }
                         }
-                    } else {
-                        float4* dst = reinterpret_cast<float4*>(p.o_parts + part_row * 128 + c * 32);
+                        stage_flush(stage, lane, [&](int i) -> uint8_t* {
+                            const int orow = __shfl_sync(0xffffffffu, out_row0, i);
+                            return warp_row0 + i < tile_rows ? static_cast<uint8_t*>(p.out) + (static_cast<long long>(orow) * 128 + c * 64) * 2 : nullptr;
+                        });
+                    }
+                } else {
+                    const long long part0 = part_row - out_row0;
+#pragma unroll 1
+                    for (int c = 0; c < 4; ++c) {
+                        uint32_t r[32];
+                        tmem_ld32(tO + c * 32, r);
+                        tc_wait_ld();
 #pragma unroll
                         for (int q4 = 0; q4 < 8; ++q4)
-                            dst[q4] = make_float4(__uint_as_float(r[q4 * 4]) * inv_l, __uint_as_float(r[q4 * 4 + 1]) * inv_l,
-                                                  __uint_as_float(r[q4 * 4 + 2]) * inv_l,
-                                                  __uint_as_float(r[q4 * 4 + 3]) * inv_l);
+                            stage_put(stage, lane, q4,
+                                      make_uint4(__float_as_uint(__uint_as_float(r[q4 * 4]) * inv_l), __float_as_uint(__uint_as_float(r[q4 * 4 + 1]) * inv_l),
+                                                 __float_as_uint(__uint_as_float(r[q4 * 4 + 2]) * inv_l), __float_as_uint(__uint_as_float(r[q4 * 4 + 3]) * inv_l)));
+                        stage_flush(stage, lane, [&](int i) -> uint8_t* {
+                            const int orow = __shfl_sync(0xffffffffu, out_row0, i);
+                            return warp_row0 + i < tile_rows ? reinterpret_cast<uint8_t*>(p.o_parts + (part0 + orow) * 128 + c * 32) : nullptr;
+                        });
                     }
                 }
                 if (live) {
