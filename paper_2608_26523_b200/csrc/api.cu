@@ -381,6 +381,9 @@ ItemCounts item_counts(const vpp_chunk_attn_args* a, Family fam) {
     return {r.unit_rows, a->num_q_heads / r.group, a->num_q_heads / r.short_group, sms};
 }
 
+// The start and end of a work item (query load, first K/V, epilogue) in KV tiles: ~4 us of ~2 us a tile; packed and MLA items
+// ~4.5 us of ~1.5 us.
+constexpr int kLead = 2, kShortLead = 3;
 constexpr int kMinLen = 2, kMinShortLen = 4;   // fewest KV tiles worth a work item (start-up ~4 us, ~2 / ~1 us per tile)
 
 SplitPlan plan_splits(const vpp_chunk_attn_args* a, Family fam) {
@@ -636,6 +639,8 @@ vpp_status run_chunk_attn(const vpp_chunk_attn_args* a, vpp_stream_t stream_, co
         pp.unit_weight = fam == Family::kMla576 ? 1 : 2;   // (a short unit's two tiles share its KV tiles)
         pp.min_len = kMinLen;
         pp.min_short_len = kMinShortLen;
+        pp.lead = fam == Family::kMla576 ? kShortLead : kLead;
+        pp.short_lead = kShortLead;
     }
     pp.max_units = L.max_units;
     pp.unit_rows = unit_rows_of(a, fam);

@@ -38,6 +38,7 @@ struct PrepParams {
     int32_t unit_items, short_items;      // work items of a unit and of a short unit
     int32_t unit_weight;                  // cost of a KV tile of a unit's item, in those of a short unit's
     int32_t min_len, min_short_len;       // fewest KV tiles worth a work item
+    int32_t lead, short_lead;             // what starting and ending a work item costs, in KV tiles
     int32_t partial;     // 1: key-range restricted launch whose results are partial (o fp32, lse) of "split 0"
     int32_t range_begin; // first KV tile of the key range (partial launches)
     int32_t range_end;   // one past its last KV tile
@@ -222,8 +223,9 @@ __global__ void __launch_bounds__(kPrepMaxThreads, 1) prep_kernel(const PrepPara
     // ---- phase 2: counting sort of the units by decreasing cost, two passes; before them, for a balanced cut, one that
     //      adds the KV tiles up: how many of them does a work item get? ----
     // Units of one kind: their KV tiles laid end to end are cut at the multiples of `len`, so that every range is one slot's
-    // share and a unit is cut only where a share ends in it (few partial results).  Units of both kinds: each unit by itself
-    // into parts of at most its kind's share.
+    // share and a unit is cut only where a share ends in it (few partial results); every unit begins with `lead` tiles that
+    // stand for the start and end of one more item in the share it begins in.  Units of both kinds: each unit by itself into
+    // parts of at most its kind's share.
     int sum = 0, sum_short = 0, len = 0, len_short = 0;
     bool stream = false;
     float bin_scale = static_cast<float>(nthr - 1) / static_cast<float>(s_max);
@@ -257,8 +259,9 @@ __global__ void __launch_bounds__(kPrepMaxThreads, 1) prep_kernel(const PrepPara
             }
             const bool is_short = rows <= p.short_rows;
             if (p.balanced && (pass == 0 || !once)) {
-                const int4 sc = block_scan2(is_short ? 0 : n_tiles, is_short ? n_tiles : 0, warp_sums);
-                before = carry + sc.x + sc.y;
+                const int lead = is_short ? p.short_lead : p.lead, n = n_tiles > 0 ? n_tiles + lead : 0;
+                const int4 sc = block_scan2(is_short ? 0 : n, is_short ? n : 0, warp_sums);
+                before = carry + sc.x + sc.y + lead;
                 carry += sc.z + sc.w;
                 if (pass == 0) {
                     sum += sc.z;
