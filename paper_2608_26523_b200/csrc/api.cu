@@ -655,7 +655,6 @@ vpp_status run_chunk_attn(const vpp_chunk_attn_args* a, vpp_stream_t stream_, co
     pp.range_end = range ? range->end_tile : 0;
     pp.header = reinterpret_cast<vpp::WorkHeader*>(ws + L.header);
     pp.units = reinterpret_cast<vpp::WorkUnit*>(ws + L.units);
-    pp.row_splits = row_splits;
     pp.q_start = row_splits + a->total_q;
     pp.tile_start = pp.q_start + a->num_reqs + 1;
     {
@@ -698,6 +697,7 @@ vpp_status run_chunk_attn(const vpp_chunk_attn_args* a, vpp_stream_t stream_, co
     ap.header_ro = pp.header;
     ap.header = pp.header;
     ap.units = pp.units;
+    ap.row_splits = L.splits > 1 ? row_splits : nullptr;
     ap.status = a->status;
 
     const int sms = sm_count_or_default();

@@ -289,6 +289,7 @@ attn_mla2_kernel(const __grid_constant__ CUtensorMap tm_q1, const __grid_constan
         const int need = (u.pos0 + u.rows + kTileN - 1) / kTileN;
         return u.kv_end < need ? u.kv_end : need;
     };
+    int n_splits = 0;            // split count of the item's unit
     auto get_item = [&](int item, WorkUnit& u, int& h) -> bool {
         if (item < num_packed) {
             u = p.units[num_normal + item];
@@ -298,6 +299,7 @@ attn_mla2_kernel(const __grid_constant__ CUtensorMap tm_q1, const __grid_constan
             decode_item(item - num_packed, num_normal, unit_block, p.num_q_heads, p.num_q_heads, ui, h);
             u = p.units[ui];
         }
+        n_splits = take_splits(u);
         return true;
     };
     auto is_packed = [&](const WorkUnit& u) { return num_packed > 0 && u.rows == 1; };
@@ -754,6 +756,8 @@ attn_mla2_kernel(const __grid_constant__ CUtensorMap tm_q1, const __grid_constan
             // the warp's 32 rows: consecutive q-heads of a packed tile, otherwise one head of consecutive tokens
             const int row_step = packed ? 1 : p.num_q_heads, warp_rows = (packed ? p.num_q_heads : u.rows) - (my_row - lane);
             const long long first_row = out_row - static_cast<long long>(lane) * row_step;
+            // the first part and head of a unit says how many partial results its rows have
+            if (p.row_splits && u.split <= 0 && h == 0 && half == 0 && live) p.row_splits[u.q_row0 + (packed ? 0 : my_row)] = n_splits;
             // (P V of the last tile is done, so the warp's own rows of P serve as the stage of its stores)
             uint8_t* const stage = p_row - lane * 128;
             if (u.split < 0) {

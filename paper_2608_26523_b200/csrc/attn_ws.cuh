@@ -338,7 +338,7 @@ attn128_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                 ok = __shfl_sync(0xffffffffu, ok, 0);
                 if (!ok) break;
                 if (lane == 0) {
-                    ring[slot].u = u;
+                    ring[slot].u = u;     // (its split count with it)
                     ring[slot].h0 = h0;
                     ring[slot].valid = have ? 1 : 0;
                     ring[slot].packed = packed ? 1 : 0;
@@ -389,7 +389,8 @@ attn128_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                 if (lane == 0) ok = mbar_wait(bar_item_full + 8 * slot, (item_it >> 1) & 1, s_abort, 211);
                 ok = __shfl_sync(0xffffffffu, ok, 0);
                 if (!ok) break;
-                const WorkUnit u = ring[slot].u;
+                WorkUnit u = ring[slot].u;
+                take_splits(u);
                 const int g = ring[slot].h0 / G;
                 const int valid = ring[slot].valid;
                 __syncwarp();
@@ -452,7 +453,8 @@ attn128_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
             while (true) {
                 const uint32_t slot = item_it & 1;
                 if (!wait1(bar_item_full + 8 * slot, (item_it >> 1) & 1, 301)) break;
-                const WorkUnit u = ring[slot].u;
+                WorkUnit u = ring[slot].u;
+                take_splits(u);
                 const int valid = ring[slot].valid;
                 const bool packed = ring[slot].packed != 0;
                 mbar_arrive(bar_item_empty + 8 * slot);
@@ -581,13 +583,15 @@ attn128_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
         while (true) {
             const uint32_t slot = item_it & 1;
             if (!mbar_wait(bar_item_full + 8 * slot, (item_it >> 1) & 1, s_abort, 401)) break;
-            const WorkUnit u = ring[slot].u;
+            WorkUnit u = ring[slot].u;
+            const int n_splits = take_splits(u);
             const bool packed = ring[slot].packed != 0;
             // this thread's row: token `tok` of the unit, q-head h0 + row % grp
             const int grp = packed ? p.short_group : p.group;
             const int tile_tok0 = packed ? 0 : t * p.tile_tokens;     // first token of the tile within the unit
             const int tok = tile_tok0 + row / grp;
-            const int out_row0 = (u.q_row0 + tok) * p.num_q_heads + ring[slot].h0 + row % grp;   // its row of out / lse
+            const int ring_h0 = ring[slot].h0;
+            const int out_row0 = (u.q_row0 + tok) * p.num_q_heads + ring_h0 + row % grp;   // its row of out / lse
             const int tile_toks = packed || u.rows - tile_tok0 < p.tile_tokens ? u.rows - tile_tok0 : p.tile_tokens;
             const int tile_rows = tile_toks * grp;                    // rows of this tile that exist (<= 0: none)
             const int valid = ring[slot].valid;
@@ -595,6 +599,8 @@ attn128_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
             if (lane == 0) mbar_arrive(bar_item_empty + 8 * slot);
             ++item_it;
             if (!valid) break;
+            // the first part and head of a unit says how many partial results its rows have
+            if (p.row_splits && u.split <= 0 && ring_h0 == 0 && row < tile_rows && row % grp == 0 && !(packed && t == 1)) p.row_splits[u.q_row0 + tok] = n_splits;
             // One item's softmax work.  The packed variant (single-token items) is compiled separately so that the
             // prefill path keeps the registers and the instruction count it had without it.
             auto run_item = [&](auto packed_tag) -> bool {

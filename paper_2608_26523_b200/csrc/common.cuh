@@ -13,13 +13,19 @@ constexpr int kTileN = 128;  // keys per KV tile
 struct __align__(16) WorkUnit {
     int32_t req;        // request index
     int32_t q_row0;     // first packed query row of the tile
-    int32_t rows;       // query rows (tokens) of the unit
+    int32_t rows;       // query rows (tokens) of the unit (at most 256) and its number of splits (merge launches): rows | splits << 16
     int32_t pos0;       // absolute position of the tile's first row (prefix_len + row offset)
     int32_t kv_begin;   // first KV tile (units of kTileN keys)
     int32_t kv_end;     // one past the last KV tile
     int32_t split;      // split index of this unit, or -1 when the tile is not split (final output)
     int32_t kv_len;     // prefix_len + chunk_len of the request: keys at or beyond it do not exist
 };
+// A unit as the attention kernels use it: `rows` alone, the split count aside.
+__device__ __forceinline__ int take_splits(WorkUnit& u) {
+    const int n = u.rows >> 16;
+    u.rows &= 0xffff;
+    return n;
+}
 
 constexpr int kMaxCheckers = 8;   // blocks of the work-decomposition kernel that check the block table
 
@@ -82,6 +88,7 @@ struct AttnParams {
     const WorkHeader* header_ro;
     WorkHeader* header;
     const WorkUnit* units;
+    int32_t* row_splits;          // [T] number of partial results of every query row, for the merge kernel (null: no merge)
     int32_t* status;              // may be null
 };
 

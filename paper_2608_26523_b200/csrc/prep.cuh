@@ -44,7 +44,6 @@ struct PrepParams {
     int32_t range_end;   // one past its last KV tile
     WorkHeader* header;
     WorkUnit* units;
-    int32_t* row_splits;  // [total_q], only written when splits > 1
     int32_t* q_start;     // [num_reqs + 1] scratch
     int32_t* tile_start;  // [num_reqs + 1] scratch
 };
@@ -153,7 +152,7 @@ __global__ void __launch_bounds__(kPrepMaxThreads, 1) prep_kernel(const PrepPara
     __shared__ int bins[2 * kPrepMaxThreads];   // blockDim.x bins of decreasing cost, then as many for the short units
     __shared__ int s_P[kPrepSmemReqs], s_C[kPrepSmemReqs], s_q[kPrepSmemReqs], s_t[kPrepSmemReqs + 1];
     __shared__ int s_error, s_max, s_min;
-    const int tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31;
+    const int tid = threadIdx.x, nthr = blockDim.x;
     pdl_launch_dependents();   // the attention kernel may set itself up (barriers, tensor memory) while this runs
     pdl_wait();                // the lengths may come from the kernel launched just before; the workspace may be in use by it
     if (blockIdx.x > 0) {
@@ -320,27 +319,13 @@ __global__ void __launch_bounds__(kPrepMaxThreads, 1) prep_kernel(const PrepPara
                     WorkUnit u;
                     u.req = r;
                     u.q_row0 = qs[r] + row_off;
-                    u.rows = rows;
+                    u.rows = rows | nsplit << 16;
                     u.pos0 = pos0;
                     u.kv_begin = kb;
                     u.kv_end = ke;
                     u.split = (nsplit > 1 || p.partial) ? s : -1;
                     u.kv_len = Ps[r] + Cs[r];
                     p.units[at] = u;
-                }
-            }
-            if (p.splits > 1) {
-                // per-row split counts: a unit of a few rows by its thread, a longer one by the whole warp
-                const int q0 = qs[r] + row_off;
-                if (rows <= 4)
-                    for (int i = 0; i < rows; ++i) p.row_splits[q0 + i] = nsplit;
-#pragma unroll 1
-                for (uint32_t todo = __ballot_sync(0xffffffffu, rows > 4); todo; todo &= todo - 1) {
-                    const int l = __ffs(todo) - 1;
-                    const int l_rows = __shfl_sync(0xffffffffu, rows, l), l_ns = __shfl_sync(0xffffffffu, nsplit, l),
-                              l_q0 = __shfl_sync(0xffffffffu, q0, l);
-#pragma unroll 1
-                    for (int i = lane; i < l_rows; i += 32) p.row_splits[l_q0 + i] = l_ns;
                 }
             }
         }
