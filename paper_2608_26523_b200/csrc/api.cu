@@ -8,6 +8,7 @@
 #include <cstdio>
 #include <cstring>
 #include <mutex>
+#include <numeric>
 
 #include "../../include/vpp.h"
 #include "attn_mla2.cuh"
@@ -209,6 +210,34 @@ TmapKey make_key(const void* base, int rank, const uint64_t* dims, const uint64_
 bool make_tmap(CUtensorMap* m, const void* base, int rank, const uint64_t* dims, const uint64_t* strides_bytes,
                const uint32_t* box) {
     return g_tmaps.get(make_key(base, rank, dims, strides_bytes, box), encode_with_driver, m);
+}
+
+// The two maps of a K or V cache of the d = 128 kernel (attn_ws.cuh) and how (block, kv-head) becomes one coordinate of the
+// first: both strides are whole numbers of `unit`.  Where that coordinate would not fit an int32 (strides with hardly a common
+// divisor in a huge cache) every tile takes the exact map.
+bool make_kv_maps(const void* base, int64_t block_stride, int64_t token_stride, int64_t head_stride, int B, int n_blocks, int heads, int box_rows,
+                  CUtensorMap* tm, CUtensorMap* tm_exact, int32_t* block_units, int32_t* head_units, int32_t* end, int32_t* exact_from) {
+    const uint64_t dx[5] = {64, static_cast<uint64_t>(B), 2, static_cast<uint64_t>(heads), static_cast<uint64_t>(n_blocks)};
+    const uint64_t sx[4] = {static_cast<uint64_t>(token_stride) * 2, 128, static_cast<uint64_t>(head_stride) * 2,
+                            static_cast<uint64_t>(block_stride) * 2};
+    const uint32_t bx[5] = {64, vpp::kExactRows, 2, 1, 1};
+    if (!make_tmap(tm_exact, base, 5, dx, sx, bx)) return false;
+    const int64_t unit = std::gcd(block_stride, head_stride);
+    const int64_t last = ((n_blocks - 1) * block_stride + (heads - 1) * head_stride) / unit;
+    if (last >= INT32_MAX) {
+        *tm = *tm_exact;
+        *exact_from = 0;
+        return true;
+    }
+    *block_units = static_cast<int32_t>(block_stride / unit);
+    *head_units = static_cast<int32_t>(head_stride / unit);
+    *end = static_cast<int32_t>(last + 1);
+    const int groups = B / vpp::kExactRows;
+    const uint64_t d[5] = {64, vpp::kExactRows, 2, static_cast<uint64_t>(groups > 0 ? groups : 1), static_cast<uint64_t>(last + 1)};
+    const uint64_t s[4] = {static_cast<uint64_t>(token_stride) * 2, 128, static_cast<uint64_t>(token_stride) * 2 * vpp::kExactRows,
+                           static_cast<uint64_t>(unit) * 2};
+    const uint32_t b[5] = {64, vpp::kExactRows, 2, static_cast<uint32_t>(box_rows / vpp::kExactRows), 1};
+    return make_tmap(tm, base, 5, d, s, b);
 }
 
 // ---- validation -------------------------------------------------------------------------------------
@@ -548,25 +577,8 @@ vpp_status run_chunk_attn(const vpp_chunk_attn_args* a, vpp_stream_t stream_, co
     const int box_rows = paged ? (B < tile_n ? B : tile_n) : tile_n;
 
     // ---- tensor maps ----
-    CUtensorMap tm_q, tm_k, tm_v;
-    {
-        const uint64_t d[4] = {static_cast<uint64_t>(a->head_dim_qk), static_cast<uint64_t>(B),
-                               static_cast<uint64_t>(a->num_kv_heads), static_cast<uint64_t>(n_blocks)};
-        const uint64_t s[3] = {static_cast<uint64_t>(a->k_token_stride) * 2, static_cast<uint64_t>(a->k_head_stride) * 2,
-                               static_cast<uint64_t>(a->k_block_stride) * 2};
-        const uint32_t b[4] = {64, static_cast<uint32_t>(box_rows), 1, 1};
-        if (!make_tmap(&tm_k, a->k_cache, 4, d, s, b)) return fail(VPP_ERR_CUDA, "cuTensorMapEncodeTiled(k) failed");
-    }
-    if (fam != Family::kMla576) {
-        const uint64_t d[4] = {static_cast<uint64_t>(a->head_dim_v), static_cast<uint64_t>(B),
-                               static_cast<uint64_t>(a->num_kv_heads), static_cast<uint64_t>(n_blocks)};
-        const uint64_t s[3] = {static_cast<uint64_t>(a->v_token_stride) * 2, static_cast<uint64_t>(a->v_head_stride) * 2,
-                               static_cast<uint64_t>(a->v_block_stride) * 2};
-        const uint32_t b[4] = {64, static_cast<uint32_t>(box_rows), 1, 1};
-        if (!make_tmap(&tm_v, a->v_cache, 4, d, s, b)) return fail(VPP_ERR_CUDA, "cuTensorMapEncodeTiled(v) failed");
-    }
-
-    CUtensorMap tm_k2, tm_v2, tm_qs;
+    CUtensorMap tm_q, tm_qs, tm_k, tm_v, tm_kx, tm_vx;
+    vpp::AttnParams ap{};
     const RowPacking rp = row_packing(a);
     // a batch of decode rows: a packed item's box brings its one token only
     const int short_box_tokens = a->total_q <= a->num_reqs ? 1 : rp.short_tokens;
@@ -579,16 +591,18 @@ vpp_status run_chunk_attn(const vpp_chunk_attn_args* a, vpp_stream_t stream_, co
         const uint32_t bs[3] = {64, static_cast<uint32_t>(rp.short_group), static_cast<uint32_t>(short_box_tokens)};
         if (!make_tmap(&tm_q, a->q, 3, dq, sq, bq) || !make_tmap(&tm_qs, a->q, 3, dq, sq, bs))
             return fail(VPP_ERR_CUDA, "cuTensorMapEncodeTiled(q) failed");
-        // the 128 features viewed as (64, 2): a box holds both 64-column slabs of a tile
-        const uint64_t d[5] = {64, static_cast<uint64_t>(B), 2, static_cast<uint64_t>(a->num_kv_heads),
-                               static_cast<uint64_t>(n_blocks)};
-        const uint64_t sk[4] = {static_cast<uint64_t>(a->k_token_stride) * 2, 128, static_cast<uint64_t>(a->k_head_stride) * 2,
+        ap.exact_from = paged || B % vpp::kExactRows == 0 ? INT32_MAX : B / vpp::kExactRows * vpp::kExactRows;
+        if (!make_kv_maps(a->k_cache, a->k_block_stride, a->k_token_stride, a->k_head_stride, B, n_blocks, a->num_kv_heads, box_rows, &tm_k,
+                          &tm_kx, &ap.k_block_units, &ap.k_head_units, &ap.k_end, &ap.exact_from) ||
+            !make_kv_maps(a->v_cache, a->v_block_stride, a->v_token_stride, a->v_head_stride, B, n_blocks, a->num_kv_heads, box_rows, &tm_v,
+                          &tm_vx, &ap.v_block_units, &ap.v_head_units, &ap.v_end, &ap.exact_from))
+            return fail(VPP_ERR_CUDA, "cuTensorMapEncodeTiled(k/v) failed");
+    } else {
+        const uint64_t d[4] = {static_cast<uint64_t>(a->head_dim_qk), static_cast<uint64_t>(B), 1, static_cast<uint64_t>(n_blocks)};
+        const uint64_t sk[3] = {static_cast<uint64_t>(a->k_token_stride) * 2, static_cast<uint64_t>(a->k_head_stride) * 2,
                                 static_cast<uint64_t>(a->k_block_stride) * 2};
-        const uint64_t sv[4] = {static_cast<uint64_t>(a->v_token_stride) * 2, 128, static_cast<uint64_t>(a->v_head_stride) * 2,
-                                static_cast<uint64_t>(a->v_block_stride) * 2};
-        const uint32_t b5[5] = {64, static_cast<uint32_t>(box_rows), 2, 1, 1};
-        if (!make_tmap(&tm_k2, a->k_cache, 5, d, sk, b5) || !make_tmap(&tm_v2, a->v_cache, 5, d, sv, b5))
-            return fail(VPP_ERR_CUDA, "cuTensorMapEncodeTiled(k/v tiles) failed");
+        const uint32_t b[4] = {64, static_cast<uint32_t>(box_rows), 1, 1};
+        if (!make_tmap(&tm_k, a->k_cache, 4, d, sk, b)) return fail(VPP_ERR_CUDA, "cuTensorMapEncodeTiled(k) failed");
     }
     CUtensorMap tm_q9, tm_qh9, tm_k93, tm_k92;  // 64 rows of one 64-column slab per box (tm_k93 / tm_k92: of 3 / 2 slabs)
     const bool mla_pair = fam == Family::kMla576;
@@ -676,7 +690,6 @@ vpp_status run_chunk_attn(const vpp_chunk_attn_args* a, vpp_stream_t stream_, co
     ++g_launches;
 
     // ---- attention ----
-    vpp::AttnParams ap{};
     ap.block_table = a->block_table;
     ap.max_blocks_per_req = a->max_blocks_per_req;
     ap.block_shift = pp.block_shift;
@@ -709,12 +722,13 @@ vpp_status run_chunk_attn(const vpp_chunk_attn_args* a, vpp_stream_t stream_, co
             ce = launch(kern, static_cast<unsigned>((sms / 2) * 2), vpp::kMla2Threads, vpp::kMla2SmemBytes, stream, tm_q9, tm_qh9, tm_k93,
                         tm_k92, tm_k, ap, box_rows);
     } else {
-        // a second producer warp for launches bound by the arrival of K/V: pages smaller than a KV tile, batches of decode rows
-        const bool v_warp = box_rows < vpp::kTileN || a->total_q <= a->num_reqs;
+        // a second producer warp for launches bound by the arrival of K/V: batches of decode rows.  (Prefill loses 1 to 2 % with it,
+        // over pages of any size: 2048 tokens of 64 heads at prefix 16385 1003 us with it, 989 without.)
+        const bool v_warp = a->total_q <= a->num_reqs;
         auto kern = v_warp ? vpp::attn128_ws_kernel<true> : vpp::attn128_ws_kernel<false>;
         ce = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, vpp::kWsSmemBytes);
         if (ce == cudaSuccess)
-            ce = launch(kern, static_cast<unsigned>(sms), vpp::kWsThreads, vpp::kWsSmemBytes, stream, tm_q, tm_k, tm_v, tm_k2, tm_v2, tm_qs,
+            ce = launch(kern, static_cast<unsigned>(sms), vpp::kWsThreads, vpp::kWsSmemBytes, stream, tm_q, tm_qs, tm_k, tm_v, tm_kx, tm_vx,
                         ap, box_rows);
     }
     if (ce != cudaSuccess) return fail(VPP_ERR_CUDA, "attention kernel attributes: %s", cudaGetErrorString(ce));

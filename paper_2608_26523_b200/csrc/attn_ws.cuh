@@ -121,18 +121,25 @@ __device__ __noinline__ void ws_packed_merge(void* out, float* lse_out, float* o
     }
 }
 
+// K / V tile in shared memory: 8-key groups of 2 KB, features 0-63 then 64-127 of the eight keys, 128-byte swizzle.  Keys of a
+// page are consecutive in it, so a page of any size is ONE copy (issuing a copy costs a producer lane over 100 clk; with the
+// two 64-feature slabs 16 KB apart a page under 128 tokens took two).  256 decode rows over pages of 16
+// tokens: 576 -> 543 us; 2048-token chunks over pages of 16 .. 64: 1020 -> 989 us, as over pages of 128.
+constexpr int kGroupBytes = 2048, kHalfBytes = 1024;
+constexpr int kExactRows = 8;                 // keys per copy of the exact map
+
 template <bool kVWarp>
 __global__ void __launch_bounds__(kWsThreads, 1)
-attn128_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
-                  const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_k2,
-                  const __grid_constant__ CUtensorMap tm_v2, const __grid_constant__ CUtensorMap tm_qs, const AttnParams p,
+attn128_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_qs,
+                  const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
+                  const __grid_constant__ CUtensorMap tm_kx, const __grid_constant__ CUtensorMap tm_vx, const AttnParams p,
                   const int kv_box_rows) {
     // tm_q:  q with a box of (64 features, group heads, tile_tokens tokens): one 64-column slab of a tile
     // tm_qs: the same with (64, short_group, short_box_tokens), for packed items
-    // tm_k2 / tm_v2 are views of the caches with the 128 features split into (64, 2): one box
-    // of them brings both 64-column slabs of a 128-row tile, i.e. a whole tile per copy instruction.  Issuing a
-    // copy costs the producer thread several hundred cycles, so fewer, larger copies matter.  tm_k / tm_v
-    // (one slab of kv_box_rows keys per box) serve pages smaller than a KV tile.
+    // tm_k / tm_v: (64 features, 8 keys, 2 halves, 8-key groups, (block, kv-head)), box (64, 8, 2, kv_box_rows / 8, 1): the keys of
+    //        a page, or of a whole tile where pages are that large
+    // tm_kx / tm_vx: (64 features, keys, 2 halves, kv-head, block), box (64, 8, 2, 1, 1): eight keys, the extent of the keys exact --
+    //        for the last tile of a contiguous cache whose length is no multiple of 8, and strides the other maps cannot express
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t* gen_base = smem_raw + (smem_base - smem_u32(smem_raw));
@@ -191,8 +198,6 @@ attn128_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
         prefetch_tmap(&tm_q);
         prefetch_tmap(&tm_k);
         prefetch_tmap(&tm_v);
-        prefetch_tmap(&tm_k2);
-        prefetch_tmap(&tm_v2);
         prefetch_tmap(&tm_qs);
     }
     __syncthreads();
@@ -228,57 +233,36 @@ attn128_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                 const uint32_t ph = (kv_it / kWsStages) & 1;
                 const uint32_t dst = sKV + st * kTileBytes;
                 const uint32_t full = bar_kv_full + 8 * st;
-                const CUtensorMap* tm = which == 0 ? &tm_k : &tm_v;
-                const CUtensorMap* tm2 = which == 0 ? &tm_k2 : &tm_v2;
+                // a lane per page (or per eight keys); its page is looked up before the wait for the stage
+                const bool exact = tile0 + kTileN > p.exact_from;
+                const int rows = exact ? kExactRows : kv_box_rows, off = lane * rows, pos = tile0 + off;
+                int blk = p.num_blocks, slot_in = 0;     // (past the end: reads as zero)
+                if (off < kTileN) {
+                    if (p.block_table == nullptr) {
+                        blk = u.req;
+                        slot_in = pos;
+                    } else if (pos < u.kv_len) {
+                        blk = __ldg(p.block_table + static_cast<long long>(u.req) * p.max_blocks_per_req + (pos >> p.block_shift));
+                        slot_in = pos & ((1 << p.block_shift) - 1);
+                    }
+                }
                 if (lane == 0) {
                     ok = mbar_wait(bar_kv_empty + 8 * st, ph ^ 1, s_abort, 203);
-                    if (ok) {
-                        mbar_arrive_expect_tx(full, kTileBytes);
-                        if (kv_box_rows == kTileN) {
-                            int blk, slot_in;
-                            if (p.block_table == nullptr) {
-                                blk = u.req;
-                                slot_in = tile0;
-                            } else if (tile0 < u.kv_len) {
-                                blk = __ldg(p.block_table + static_cast<long long>(u.req) * p.max_blocks_per_req +
-                                            (tile0 >> p.block_shift));
-                                slot_in = tile0 & ((1 << p.block_shift) - 1);
-                            } else {
-                                blk = p.num_blocks;
-                                slot_in = 0;
-                            }
-                            tma_load_5d(dst, tm2, full, 0, slot_in, 0, g, blk);
-                        }
-                    }
+                    if (ok) mbar_arrive_expect_tx(full, kTileBytes);
                 }
                 ok = __shfl_sync(0xffffffffu, ok, 0);
                 if (!ok) return false;
-                if (kv_box_rows != kTileN) {
-                    // Pages smaller than a KV tile: one copy per (page, 64-column slab), each issued by a lane of its
-                    // own -- every lane looks up its page itself, and a lane's copy costs the warp a third of what a
-                    // single thread spends on one with its address arithmetic.  (The byte count was posted above.)
-                    const int per = kTileN / kv_box_rows;             // pages per tile: 2 .. 8
-                    if (lane < 2 * per) {
-                        const int off = (lane >> 1) * kv_box_rows, sl = lane & 1;
-                        const int pos = tile0 + off;
-                        int blk, slot_in;
-                        if (p.block_table == nullptr) {
-                            blk = u.req;
-                            slot_in = pos;
-                        } else if (pos < u.kv_len) {
-                            blk = __ldg(p.block_table + static_cast<long long>(u.req) * p.max_blocks_per_req +
-                                        (pos >> p.block_shift));
-                            slot_in = pos & ((1 << p.block_shift) - 1);
-                        } else {
-                            blk = p.num_blocks;  // out of range: the copy engine fills zeros
-                            slot_in = 0;
-                        }
-                        tma_load_4d(dst + sl * kSlabBytes + static_cast<uint32_t>(off) * 128u, tm, full, sl * 64, slot_in, g, blk);
+                if (off < kTileN) {
+                    const uint32_t d = dst + static_cast<uint32_t>(off) * (kGroupBytes / 8);
+                    if (exact) {
+                        tma_load_5d(d, which == 0 ? &tm_kx : &tm_vx, full, 0, slot_in, 0, g, blk);
+                    } else {
+                        const int at = blk == p.num_blocks ? (which == 0 ? p.k_end : p.v_end)
+                                       : which == 0 ? blk * p.k_block_units + g * p.k_head_units : blk * p.v_block_units + g * p.v_head_units;
+                        tma_load_5d(d, which == 0 ? &tm_k : &tm_v, full, 0, 0, 0, slot_in >> 3, at);
                     }
-                    __syncwarp();
                 }
-                ok = __shfl_sync(0xffffffffu, ok, 0);
-                if (!ok) return false;
+                __syncwarp();
                 if (which == 1 && tile0 + kTileN > u.kv_len) {
                     // Keys at or beyond kv_len do not exist; zero their V rows so that 0 * garbage
                     // cannot poison O.  The MMA warp waits for bar_vfix on such a tile.
@@ -289,8 +273,8 @@ attn128_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                     const int first = u.kv_len > tile0 ? u.kv_len - tile0 : 0;
                     const uint4 z = make_uint4(0, 0, 0, 0);
                     for (int r = first + lane; r < kTileN; r += 32) {
-                        uint4* a = reinterpret_cast<uint4*>(vb + r * 128);
-                        uint4* b = reinterpret_cast<uint4*>(vb + kSlabBytes + r * 128);
+                        uint4* a = reinterpret_cast<uint4*>(vb + (r >> 3) * kGroupBytes + (r & 7) * 128);
+                        uint4* b = a + kHalfBytes / 16;
 #pragma unroll
                         for (int c = 0; c < 8; ++c) {
                             a[c] = z;
@@ -305,9 +289,8 @@ attn128_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
             return true;
         };
         // kVWarp: a second producer warp (warp 2) loads the V tiles, warp 0 the K tiles.  The host chooses it for the launches
-        // that are bound by how fast K/V arrives: pages smaller than a KV tile (a tile is then 4 to 16 copies per operand)
-        // and batches of decode rows, which stream K/V at memory speed (+10 to 18 % with K and V requested by two warps).
-        // Prefill over large pages keeps the single producer (a second one costs it 1 to 2 %).
+        // that are bound by how fast K/V arrives: batches of decode rows, which stream K/V at memory speed (+10 to 18 % with K
+        // and V requested by two warps).  Prefill keeps the single producer (a second one costs it 1 to 2 %).
         constexpr bool split_v = kVWarp;
         if (warp == 0) {
             // ============================ scheduler + TMA producer ============================
@@ -380,7 +363,7 @@ attn128_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                 if (!ok) break;
             }
         } else if (warp == 2 && split_v) {
-            // ============================ second producer: the V tiles when pages are small ============================
+            // ============================ second producer: the V tiles ============================
             // (follows the item ring like every other role)
             uint32_t item_it = 0, kv_it = 0, vfix_cnt = 0;
             while (true) {
@@ -415,21 +398,21 @@ attn128_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
             };
             // Descriptors are advanced by adding constants to their low word: the single issuing thread
             // must not spend longer building operands than the tensor core spends on the MMA.
-            constexpr uint32_t kHi = desc_hi_sw128(1024);
+            constexpr uint32_t kHiQ = desc_hi_sw128(1024), kHiKV = desc_hi_sw128(kGroupBytes);
             const uint32_t q_lo0 = desc_lo_sw128(sQ, 16), q_lo1 = desc_lo_sw128(sQ + kTileBytes, 16);
             auto issue_qk = [&](uint32_t tS, uint32_t q_lo, uint32_t k_stage) {
                 const uint32_t k_lo = desc_lo_sw128(k_stage, 16);
 #pragma unroll
                 for (int k = 0; k < 8; ++k) {
-                    const uint32_t koff = ((k >> 2) * kSlabBytes + (k & 3) * 32) >> 4;
-                    mma_ss_lh(tS, q_lo + koff, k_lo + koff, kHi, kIdescQK, k > 0);
+                    const uint32_t qoff = ((k >> 2) * kSlabBytes + (k & 3) * 32) >> 4, koff = ((k >> 2) * kHalfBytes + (k & 3) * 32) >> 4;
+                    mma_ss_lhh(tS, q_lo + qoff, kHiQ, k_lo + koff, kHiKV, kIdescQK, k > 0);
                 }
             };
             auto issue_pv = [&](uint32_t tO, uint32_t tP, uint32_t v_stage, bool first, int k0, int k1) {
-                const uint32_t v_lo = desc_lo_sw128(v_stage, kSlabBytes);
+                const uint32_t v_lo = desc_lo_sw128(v_stage, kHalfBytes);
 #pragma unroll
                 for (int k = k0; k < k1; ++k) {
-                    mma_ts_lh(tO, tP + k * 8, v_lo + k * (2048 >> 4), kHi, kIdescPV, (!first || k > 0) ? 1u : 0u);
+                    mma_ts_lh(tO, tP + k * 8, v_lo + k * (2 * kGroupBytes >> 4), kHiKV, kIdescPV, (!first || k > 0) ? 1u : 0u);
                 }
             };
             // O_t += P_t V for one KV tile, following the hand-overs: every early part as soon as it is there, the rest after
