@@ -163,11 +163,12 @@ private:
         CUtensorMap map;
         bool valid = false;
     };
-    static uint64_t hash(const TmapKey& k) {   // FNV-1a over the key's bytes (the key is zero-initialised, padding included)
-        const unsigned char* b = reinterpret_cast<const unsigned char*>(&k);
-        uint64_t h = 1469598103934665603ull;
-        for (size_t i = 0; i < sizeof k; ++i) h = (h ^ b[i]) * 1099511628211ull;
-        return h;
+    static uint64_t hash(const TmapKey& k) {   // over the key's words (the key is zero-initialised, padding included)
+        static_assert(sizeof(TmapKey) % 8 == 0, "whole words");
+        uint64_t w[sizeof k / 8], h = 1469598103934665603ull;
+        std::memcpy(w, &k, sizeof k);
+        for (uint64_t x : w) h = (h ^ x ^ (h >> 29)) * 0x9E3779B97F4A7C15ull;
+        return h ^ (h >> 32);
     }
     std::mutex mu_;
     Slot slots_[kSets * kWays];
@@ -410,9 +411,9 @@ ItemCounts item_counts(const vpp_chunk_attn_args* a, Family fam) {
     return {r.unit_rows, a->num_q_heads / r.group, a->num_q_heads / r.short_group, sms};
 }
 
-// The start and end of a work item (query load, first K/V, epilogue) in KV tiles: ~4 us of ~2 us a tile; packed and MLA items
-// ~4.5 us of ~1.5 us.
-constexpr int kLead = 2, kShortLead = 3;
+// The start and end of a work item (query load, first K/V, epilogue) in KV tiles: ~4 us of ~2 us a tile; packed items
+// ~4.5 us of ~1.5 us; MLA items (144 KB of queries, 256 KB of partial results) ~9 us of ~1.9.
+constexpr int kLead = 2, kShortLead = 3, kMlaLead = 5;
 constexpr int kMinLen = 2, kMinShortLen = 4;   // fewest KV tiles worth a work item (start-up ~4 us, ~2 / ~1 us per tile)
 
 SplitPlan plan_splits(const vpp_chunk_attn_args* a, Family fam) {
@@ -653,8 +654,8 @@ vpp_status run_chunk_attn(const vpp_chunk_attn_args* a, vpp_stream_t stream_, co
         pp.unit_weight = fam == Family::kMla576 ? 1 : 2;   // (a short unit's two tiles share its KV tiles)
         pp.min_len = kMinLen;
         pp.min_short_len = kMinShortLen;
-        pp.lead = fam == Family::kMla576 ? kShortLead : kLead;
-        pp.short_lead = kShortLead;
+        pp.lead = fam == Family::kMla576 ? kMlaLead : kLead;
+        pp.short_lead = fam == Family::kMla576 ? kMlaLead : kShortLead;
     }
     pp.max_units = L.max_units;
     pp.unit_rows = unit_rows_of(a, fam);
