@@ -598,31 +598,27 @@ vpp_status run_chunk_attn(const vpp_chunk_attn_args* a, vpp_stream_t stream_, co
             !make_kv_maps(a->v_cache, a->v_block_stride, a->v_token_stride, a->v_head_stride, B, n_blocks, a->num_kv_heads, box_rows, &tm_v,
                           &tm_vx, &ap.v_block_units, &ap.v_head_units, &ap.v_end, &ap.exact_from))
             return fail(VPP_ERR_CUDA, "cuTensorMapEncodeTiled(k/v) failed");
-    } else {
-        const uint64_t d[4] = {static_cast<uint64_t>(a->head_dim_qk), static_cast<uint64_t>(B), 1, static_cast<uint64_t>(n_blocks)};
-        const uint64_t sk[3] = {static_cast<uint64_t>(a->k_token_stride) * 2, static_cast<uint64_t>(a->k_head_stride) * 2,
-                                static_cast<uint64_t>(a->k_block_stride) * 2};
-        const uint32_t b[4] = {64, static_cast<uint32_t>(box_rows), 1, 1};
-        if (!make_tmap(&tm_k, a->k_cache, 4, d, sk, b)) return fail(VPP_ERR_CUDA, "cuTensorMapEncodeTiled(k) failed");
     }
-    CUtensorMap tm_q9, tm_qh9, tm_k93, tm_k92;  // 64 rows of one 64-column slab per box (tm_k93 / tm_k92: of 3 / 2 slabs)
-    const bool mla_pair = fam == Family::kMla576;
+    CUtensorMap tm_q9, tm_qh9, tm_k93, tm_k92;  // attn_mla2.cuh
+    const bool mla_pair = fam == Family::kMla576, mla_small_pages = mla_pair && box_rows < vpp::kMla2BoxRows;
     if (mla_pair) {
         const uint64_t dq[4] = {64, static_cast<uint64_t>(a->total_q), static_cast<uint64_t>(vpp::kMlaSlabs),
                                 static_cast<uint64_t>(a->num_q_heads)};
         const uint64_t sq[3] = {static_cast<uint64_t>(a->head_dim_qk) * a->num_q_heads * 2, 128,
                                 static_cast<uint64_t>(a->head_dim_qk) * 2};
         const uint32_t bq[4] = {vpp::kMla2BoxCols, vpp::kMla2BoxRows, static_cast<uint32_t>(vpp::kMlaSlabs), 1};   // all nine slabs in one copy
-        const uint64_t d[5] = {64, static_cast<uint64_t>(B), static_cast<uint64_t>(vpp::kMlaSlabs),
-                               static_cast<uint64_t>(a->num_kv_heads), static_cast<uint64_t>(n_blocks)};
-        const uint64_t sk[4] = {static_cast<uint64_t>(a->k_token_stride) * 2, 128, static_cast<uint64_t>(a->k_head_stride) * 2,
-                                static_cast<uint64_t>(a->k_block_stride) * 2};
-        // (with pages under 64 tokens the kernel copies page by page through tm_k and these two maps go unused)
-        const uint32_t krows = static_cast<uint32_t>(paged && B < vpp::kMla2BoxRows ? B : vpp::kMla2BoxRows);
-        const uint32_t b3[5] = {vpp::kMla2BoxCols, krows, vpp::kKG, 1, 1};               // one K hand-back group
-        const uint32_t b2[5] = {vpp::kMla2BoxCols, krows, vpp::kMla2VBoxSlabs, 1, 1};    // one V chunk
-        if (!make_tmap(&tm_q9, a->q, 4, dq, sq, bq) ||
-            !make_tmap(&tm_k93, a->k_cache, 5, d, sk, b3) || !make_tmap(&tm_k92, a->k_cache, 5, d, sk, b2))
+        const uint64_t tok = static_cast<uint64_t>(a->k_token_stride) * 2, blk = static_cast<uint64_t>(a->k_block_stride) * 2;
+        const uint64_t slabs = static_cast<uint64_t>(vpp::kMlaSlabs), blocks = static_cast<uint64_t>(n_blocks);
+        const uint32_t rows = static_cast<uint32_t>(box_rows);
+        // pages under 64 tokens: the keys seen as 8-key groups; larger ones: 64 keys of three / two slabs
+        const uint64_t d8[5] = {64, 8, slabs, static_cast<uint64_t>(B) / 8, blocks}, s8[4] = {tok, 128, 8 * tok, blk};
+        const uint64_t d64[5] = {64, static_cast<uint64_t>(B), slabs, static_cast<uint64_t>(a->num_kv_heads), blocks};
+        const uint64_t s64[4] = {tok, 128, static_cast<uint64_t>(a->k_head_stride) * 2, blk};
+        auto kv_map = [&](CUtensorMap* m, uint32_t n_slabs) {
+            const uint32_t b8[5] = {vpp::kMla2BoxCols, 8, n_slabs, rows / 8, 1}, b64[5] = {vpp::kMla2BoxCols, rows, n_slabs, 1, 1};
+            return mla_small_pages ? make_tmap(m, a->k_cache, 5, d8, s8, b8) : make_tmap(m, a->k_cache, 5, d64, s64, b64);
+        };
+        if (!make_tmap(&tm_q9, a->q, 4, dq, sq, bq) || !kv_map(&tm_k93, vpp::kKG) || !kv_map(&tm_k92, vpp::kMla2VBoxSlabs))
             return fail(VPP_ERR_CUDA, "cuTensorMapEncodeTiled(mla pair) failed");
         // packed single-token items: 64 q-heads of one token as the rows of a CTA's Q tile
         const uint64_t dh[4] = {64, static_cast<uint64_t>(a->num_q_heads), static_cast<uint64_t>(vpp::kMlaSlabs),
@@ -717,11 +713,11 @@ vpp_status run_chunk_attn(const vpp_chunk_attn_args* a, vpp_stream_t stream_, co
     const int sms = sm_count_or_default();
     cudaError_t ce;
     if (mla_pair) {
-        auto kern = vpp::attn_mla2_kernel;
+        auto kern = mla_small_pages ? vpp::attn_mla2_kernel<true> : vpp::attn_mla2_kernel<false>;
         ce = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, vpp::kMla2SmemBytes);
         if (ce == cudaSuccess)
             ce = launch(kern, static_cast<unsigned>((sms / 2) * 2), vpp::kMla2Threads, vpp::kMla2SmemBytes, stream, tm_q9, tm_qh9, tm_k93,
-                        tm_k92, tm_k, ap, box_rows);
+                        tm_k92, ap, box_rows);
     } else {
         // a second producer warp for launches bound by the arrival of K/V: batches of decode rows.  (Prefill loses 1 to 2 % with it,
         // over pages of any size: 2048 tokens of 64 heads at prefix 16385 1003 us with it, 989 without.)

@@ -53,6 +53,17 @@ constexpr int kVG = 2;  // V chunks per hand-back group (2 groups per tile: key 
 constexpr int kKGroups = kMlaSlabs / kKG, kVGroups = kMla2VChunks / kVG;
 constexpr int kMla2SmemBytes = kMla2QBytes + kMla2KBytes + kMla2VBytes + kMla2PBytes + 1024 /*align*/ + 1536;
 
+// K and V in shared memory.  Pages of 64 tokens and more: slabs of 64 features, 8 KB apart.  Smaller pages (kSmallPages): 8-key
+// groups, in each the slabs of the hand-back group (K: three) or chunk (V: two) side by side, 1 KB of eight keys apiece -- the keys of
+// a page are consecutive then, so a group's or chunk's share of a page is ONE copy instead of one per slab (512 tokens at prefix
+// 8195, 128 heads: pages of 16 1176 -> 991 us, of 32 965 -> 918).  Pages of 64 keep the slabs: one copy either way, and the
+// MMAs read K groups of 3 KB 9 % slower (887 against 977 us).
+template <bool kSmallPages>
+struct MlaLayout {
+    static constexpr int kKSlab = kSmallPages ? 1024 : 8192, kKGroup = kSmallPages ? kKG * 1024 : 1024;   // from slab to slab, from eight keys to the next
+    static constexpr int kVSlab = kSmallPages ? 1024 : 8192, kVGroup = kSmallPages ? 2 * 1024 : 1024;
+};
+
 // ---- the pair protocol as checkable facts --------------------------------------------------------------------
 // Copy boxes (elements of the tensor maps the host encodes; the host uses these constants):
 constexpr int kMla2BoxCols = 64, kMla2BoxRows = 64;                       // 64 features x 64 rows / keys per slab
@@ -117,6 +128,18 @@ __device__ __forceinline__ void mma2_ss_lh(uint32_t d_tmem, uint32_t a_lo, uint3
         "mov.b64 db, {%2, %3};\n\t"
         "tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %4, p;\n\t}" ::"r"(d_tmem),
         "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+// (with the two operands' 8-row groups at different distances)
+__device__ __forceinline__ void mma2_ss_lhh(uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi, uint32_t idesc,
+                                            uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
+        "setp.ne.b32 p, %6, 0;\n\t"
+        "mov.b64 da, {%1, %2};\n\t"
+        "mov.b64 db, {%3, %4};\n\t"
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %5, p;\n\t}" ::"r"(d_tmem),
+        "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate)
         : "memory");
 }
 // arrive on the barrier at the same shared-memory offset in every CTA of `mask` once all MMAs issued so far are done
@@ -187,12 +210,14 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity,
     }
 }
 
+template <bool kSmallPages>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kMla2Threads, 1)
 attn_mla2_kernel(const __grid_constant__ CUtensorMap tm_q1, const __grid_constant__ CUtensorMap tm_qh,
                  const __grid_constant__ CUtensorMap tm_k3, const __grid_constant__ CUtensorMap tm_k2,
-                 const __grid_constant__ CUtensorMap tm_k1, const AttnParams p, const int kv_box_rows) {
-    // tm_k1: (64 cols, keys, head, block) box (64, kv_box_rows, 1, 1) -- one page's share of one slab, for pages under 64 tokens
-    //        (kv_box_rows < 64): a 64-key group then takes one copy per (slab, page), each issued by a lane of its own
+                 const AttnParams p, const int kv_box_rows) {
+    using Layout = MlaLayout<kSmallPages>;
+    // tm_k3 / tm_k2 with pages under 64 tokens: (64 cols, 8 keys, 9 slabs, 8-key groups, block), box (64, 8, 3 / 2, kv_box_rows / 8, 1) --
+    //        a page's share of a K hand-back group / a V chunk; each copy is issued by a lane of its own
     // tm_qh: (64 cols, Hq heads, 9 slabs, T rows) box (64, 64, 9, 1)      -- 64 q-heads of one token (packed items)
     // tm_q1: (64 cols, T rows, 9 slabs, Hq) box (64, 64, 9, 1)         -- 64 query rows, all nine 64-column slabs
     // tm_k3: (64 cols, keys, 9 slabs, head, block) box (64, 64, 3, 1, 1) -- 64 keys of three slabs: one K hand-back group
@@ -324,8 +349,8 @@ attn_mla2_kernel(const __grid_constant__ CUtensorMap tm_q1, const __grid_constan
         for (int rr = (r0 > 0 ? r0 : 0) + lane; rr < 64; rr += 32) {
 #pragma unroll
             for (int g = 0; g < 2; ++g) {
-                uint4* a = reinterpret_cast<uint4*>(gen_base + kMla2QBytes + kMla2KBytes + c * kMla2VChunk + g * 8192 +
-                                                    rr * 128);
+                uint4* a = reinterpret_cast<uint4*>(gen_base + kMla2QBytes + kMla2KBytes + c * kMla2VChunk + g * Layout::kVSlab +
+                                                    (rr >> 3) * Layout::kVGroup + (rr & 7) * 128);
 #pragma unroll
                 for (int q = 0; q < 8; ++q) a[q] = z;
             }
@@ -340,8 +365,8 @@ attn_mla2_kernel(const __grid_constant__ CUtensorMap tm_q1, const __grid_constan
     if (warp == 0) {
         // ===================================== Q / K producer =====================================
         // one thread: group g of the next tile is requested as soon as the MMAs that read group g of this tile are done
-        if (kv_box_rows < 64) {
-            // pages under 64 tokens: the waits and the Q copy by lane 0, the K copies of a group by 3 x (64 / page) lanes
+        if (kSmallPages) {
+            // pages under 64 tokens: the waits and the Q copy by lane 0, the K copies of a group by (64 / page) lanes
             const int np = 64 / kv_box_rows, pq = lane % np;
             uint32_t q_it = 0, kc = 0;
             bool ok = true;
@@ -376,10 +401,9 @@ attn_mla2_kernel(const __grid_constant__ CUtensorMap tm_q1, const __grid_constan
                         }
                         ok = __shfl_sync(0xffffffffu, ok, 0);
                         if (!ok) break;
-                        if (lane < kKG * np) {
-                            const int sl = g * kKG + lane / np;
-                            tma2_load_4d(sK + sl * 8192 + pq * kv_box_rows * 128, &tm_k1, pair_k_full + 8 * g, 64 * sl, slot_in, 0, blk);
-                        }
+                        if (lane < np)
+                            tma2_load_5d(sK + g * kKG * 8192 + pq * (kv_box_rows >> 3) * Layout::kKGroup, &tm_k3, pair_k_full + 8 * g, 0, 0, g * kKG,
+                                         slot_in >> 3, blk);
                         __syncwarp();
                     }
                     ++kc;
@@ -444,8 +468,8 @@ attn_mla2_kernel(const __grid_constant__ CUtensorMap tm_q1, const __grid_constan
             for (int j = u.kv_begin; j < t_hi && ok; ++j) {
                 const int tile0 = j * kTileN;
                 const bool tail = tile0 + kTileN > u.kv_len;
-                if (kv_box_rows < 64) {
-                    // pages under 64 tokens: a group's two chunks take 2 chunks x 2 slabs x (64 / page) copies, a lane each
+                if (kSmallPages) {
+                    // pages under 64 tokens: a group's two chunks take 2 x (64 / page) copies, a lane each
                     const int np = 64 / kv_box_rows, pq = lane % np;
                     const uint32_t par = (vc & 1) ^ 1;
 #pragma unroll 1
@@ -460,14 +484,13 @@ attn_mla2_kernel(const __grid_constant__ CUtensorMap tm_q1, const __grid_constan
                         }
                         ok = __shfl_sync(0xffffffffu, ok, 0);
                         if (!ok) break;
-                        if (lane < kVG * 2 * np) {
-                            const int c = g * kVG + lane / (2 * np), s2 = (lane / np) & 1;
-                            const int hf = c >> 1, slab = 4 * (c & 1) + 2 * static_cast<int>(rank) + s2;
+                        if (lane < kVG * np) {
+                            const int c = g * kVG + lane / np, slab0 = 4 * (c & 1) + 2 * static_cast<int>(rank);
                             int blk, slot_in;
-                            page_of(u, tile0 + 64 * hf + pq * kv_box_rows, blk, slot_in);
-                            const uint32_t dst = sV + c * kMla2VChunk + s2 * 8192 + pq * kv_box_rows * 128;
-                            if (tail) tma_load_4d(dst, &tm_k1, own_v_full + 8 * g, 64 * slab, slot_in, 0, blk);
-                            else tma2_load_4d(dst, &tm_k1, pair_v_full + 8 * g, 64 * slab, slot_in, 0, blk);
+                            page_of(u, tile0 + 64 * (c >> 1) + pq * kv_box_rows, blk, slot_in);
+                            const uint32_t dst = sV + c * kMla2VChunk + pq * (kv_box_rows >> 3) * Layout::kVGroup;
+                            if (tail) tma_load_5d(dst, &tm_k2, own_v_full + 8 * g, 0, 0, slab0, slot_in >> 3, blk);
+                            else tma2_load_5d(dst, &tm_k2, pair_v_full + 8 * g, 0, 0, slab0, slot_in >> 3, blk);
                         }
                         __syncwarp();
                     }
@@ -522,7 +545,7 @@ attn_mla2_kernel(const __grid_constant__ CUtensorMap tm_q1, const __grid_constan
         // Two issuing threads, this one and the P V issuer in warp 7: a single thread has nothing to hide the latency of
         // its own barrier tests, commits and MMA issue behind, and the tensor pipe idled between its groups.
         constexpr uint32_t kIdescQK = idesc_bf16(128, 128, false, false);
-        constexpr uint32_t kHi = desc_hi_sw128(1024);
+        constexpr uint32_t kHiQ = desc_hi_sw128(1024), kHiK = desc_hi_sw128(Layout::kKGroup);
         const uint32_t q_lo = desc_lo_sw128(sQ, 16), k_lo = desc_lo_sw128(sK, 16);
         uint32_t q_it = 0, kc = 0, item_it = 0;   // kc: score tiles issued so far (all items)
         bool ok = true;
@@ -535,8 +558,8 @@ attn_mla2_kernel(const __grid_constant__ CUtensorMap tm_q1, const __grid_constan
             for (int s = g * kKG; s < (g + 1) * kKG; ++s) {
 #pragma unroll
                 for (int kk = 0; kk < 4; ++kk) {
-                    mma2_ss_lh(tS, q_lo + ((s * 8192 + kk * 32) >> 4), k_lo + ((s * 8192 + kk * 32) >> 4), kHi, kIdescQK,
-                               (s > 0 || kk > 0) ? 1u : 0u);
+                    mma2_ss_lhh(tS, q_lo + ((s * 8192 + kk * 32) >> 4), kHiQ,
+                                k_lo + ((g * kKG * 8192 + (s - g * kKG) * Layout::kKSlab + kk * 32) >> 4), kHiK, kIdescQK, (s > 0 || kk > 0) ? 1u : 0u);
                 }
             }
             tc_commit2(g < kKGroups - 1 ? bar_k_empty + 8 * g : bar_last, 3);
@@ -574,9 +597,9 @@ attn_mla2_kernel(const __grid_constant__ CUtensorMap tm_q1, const __grid_constan
     } else if (warp == 7 && leader && lane == 0) {
         // ============ P V MMA issuer: one thread for both CTAs of the pair (O += P V) ============
         constexpr uint32_t kIdescPV = idesc_bf16(128, 256, false, true);
-        constexpr uint32_t kHi = desc_hi_sw128(1024);
+        constexpr uint32_t kHiP = desc_hi_sw128(1024), kHiV = desc_hi_sw128(Layout::kVGroup);
         const uint32_t p_lo = desc_lo_sw128(sP, 16);
-        const uint32_t v_lo = desc_lo_sw128(sV, 8192);  // MN-major: 64-column groups 8 KB apart
+        const uint32_t v_lo = desc_lo_sw128(sV, Layout::kVSlab);  // MN-major: distance of the 64-column groups
         const uint32_t tO0 = tmem_base + kMla2TmemO0, tO1 = tmem_base + kMla2TmemO1;
         uint32_t vc = 0, vfix_it = 0, item_it = 0;   // vc: P V tiles issued so far (all items)
         bool ok = true;
@@ -589,8 +612,9 @@ attn_mla2_kernel(const __grid_constant__ CUtensorMap tm_q1, const __grid_constan
                 const uint32_t tO = (c & 1) ? tO1 : tO0;
 #pragma unroll
                 for (int k4 = 0; k4 < 4; ++k4) {
-                    mma2_ss_lh(tO, p_lo + (((c >> 1) * 8192 + k4 * 32) >> 4), v_lo + ((c * kMla2VChunk + k4 * 2048) >> 4),
-                               kHi, kIdescPV, (!first_tile || c > 1 || k4 > 0) ? 1u : 0u);
+                    mma2_ss_lhh(tO, p_lo + (((c >> 1) * 8192 + k4 * 32) >> 4), kHiP,
+                                v_lo + ((c * kMla2VChunk + k4 * 2 * Layout::kVGroup) >> 4), kHiV, kIdescPV,
+                                (!first_tile || c > 1 || k4 > 0) ? 1u : 0u);
                 }
             }
             tc_commit2(g < kVGroups - 1 ? bar_v_empty + 8 * g : bar_pv_done, 3);
