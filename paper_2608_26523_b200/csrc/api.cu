@@ -416,31 +416,69 @@ ItemCounts item_counts(const vpp_chunk_attn_args* a, Family fam) {
 constexpr int kLead = 2, kShortLead = 3, kMlaLead = 5;
 constexpr int kMinLen = 2, kMinShortLen = 4;   // fewest KV tiles worth a work item (start-up ~4 us, ~2 / ~1 us per tile)
 
+// Time of a KV tile of a work item, measured at full clock.  (Packed items have a producer warp for V of their own in decode
+// batches only.)
+struct TileTimes {
+    double unit_us, short_us;
+};
+TileTimes tile_times(const vpp_chunk_attn_args* a, Family fam) {
+    if (fam == Family::kMla576) return {1.6, 1.6};
+    return {1.75, a->total_q <= a->num_reqs ? 0.85 : 1.3};
+}
+
+// Ranges of a balanced cut when every unit has `items` work items: as many as fill the slots in one round, or in up to four where
+// one would leave a fifth of them idle.
+int ranges_of(int slots, int items) {
+    int best = 1;
+    double fill = 0;
+    for (int k = 1; k <= 4 && fill < 0.8; ++k) {
+        const int r = k * slots / items;
+        const double f = static_cast<double>(r) * items / (k * slots);
+        if (r >= 1 && f > fill) {
+            fill = f;
+            best = r;
+        }
+    }
+    return best;
+}
+
 SplitPlan plan_splits(const vpp_chunk_attn_args* a, Family fam) {
     if (a->num_kv_splits >= 1) return {a->num_kv_splits, false};
     if (a->total_q <= 0 || a->num_reqs <= 0) return {1, false};
     // An upper bound on the work items of an uncut launch.  Where they fill the slots several times the dynamic longest-first
     // order balances them well enough; where they do not, the shares are cut to measure.
     const ItemCounts c = item_counts(a, fam);
-    const bool decode = a->total_q <= a->num_reqs;
-    const long long units = decode ? a->total_q : (a->total_q + c.unit_rows - 1) / c.unit_rows + (a->num_reqs > 1 ? a->num_reqs : 0);
-    const long long items = units * (decode ? c.short_items : c.unit_items);
-    const long long tiles = (a->max_seq_len + vpp::kTileN - 1) / vpp::kTileN;
+    const bool decode = a->total_q <= a->num_reqs, one_request = a->num_reqs == 1, mla = fam == Family::kMla576;
+    const long long units = decode ? a->total_q : (a->total_q + c.unit_rows - 1) / c.unit_rows + (one_request ? 0 : a->num_reqs);
+    const int per_unit = decode ? c.short_items : c.unit_items;
+    const long long items = units * per_unit, tiles = (a->max_seq_len + vpp::kTileN - 1) / vpp::kTileN;
     // (one request, or a batch of decode rows, of the d = 128 family: from 80 % of the SMs on the split count that leaves the
-    //  least idle last wave, below; mixed batches and MLA: up to two items per slot)
-    const bool one_kind = decode || a->num_reqs == 1;
-    const bool few = fam == Family::kGqa128 && one_kind ? items * 5 < c.slots * 4ll : items < 2ll * c.slots;
+    //  least idle last wave, below; MLA's pairs of SMs take their items in a fixed order, so more items than pairs are left alone:
+    //  110 decode rows 75 us uncut, 88 cut; mixed batches of d = 128: up to two items per slot)
+    const bool few = mla ? items <= c.slots : decode || one_request ? items * 5 < c.slots * 4ll : items < 2ll * c.slots;
     if (few) {
+        // Is it worth it?  Uncut, the longest unit takes tiles * us, or a ragged batch of more items than slots about half of that
+        // after the mean ends.  Cut, everybody takes its share, plus the decomposition's and the merge's part and the partial
+        // results, written and read once at ~3 TB/s.  (Lengths are only known to be at most max_seq_len: one request's units
+        // are taken to end there, a batch's to be half as long.)  200 tokens of 64 heads at 2048 keys: 40 us uncut, 47 cut; 256 tokens of 4
+        // heads at 1024 keys 24 uncut, 21 cut.
+        const TileTimes t = tile_times(a, fam);
+        const double us = decode ? t.short_us : t.unit_us, mean = one_request ? (decode ? tiles : tiles - a->total_q / 256.0) : 0.5 * tiles;
+        const int least = decode ? kMinShortLen : kMinLen;
+        double share = mean * units / ranges_of(c.slots, per_unit);
+        if (share < least) share = least;
+        const double uncut_us = us * (items <= c.slots ? tiles : std::fmax(tiles, mean * items / c.slots + 0.5 * tiles));
+        const double parts_us = 8.0 * a->total_q * a->num_q_heads * a->head_dim_v / 3e6;      // of one partial result per row
+        const double cut_us = us * share + (decode && !mla ? 6.0 : 8.0) + parts_us * (mean / share > 1 ? mean / share : 1);
+        if (cut_us >= uncut_us) return {1, false};
         // what a unit may need: its share of the slots when all are equally long; several times that when they are ragged (one
         // long context among short ones gets most of the slots)
-        long long s = a->num_reqs == 1 ? (c.slots + items - 1) / items + 1 : (2ll * c.slots + items - 1) / items + 2;
-        const long long by_len = tiles / (decode ? kMinShortLen : kMinLen);
-        if (s > by_len) s = by_len;
+        long long s = one_request ? (c.slots + items - 1) / items + 1 : (2ll * c.slots + items - 1) / items + 2;
+        if (s > tiles / least) s = tiles / least;
         if (s > vpp::kMergeMaxSplits) s = vpp::kMergeMaxSplits;
-        if (s < 2) return {1, false};
-        return {static_cast<int>(s), true};
+        return s < 2 ? SplitPlan{1, false} : SplitPlan{static_cast<int>(s), true};
     }
-    if (fam == Family::kMla576) return {1, false};
+    if (mla) return {1, false};
     return {uniform_splits(a, heads_per_item(a, fam)), false};
 }
 
@@ -647,7 +685,11 @@ vpp_status run_chunk_attn(const vpp_chunk_attn_args* a, vpp_stream_t stream_, co
         pp.slots = c.slots;
         pp.unit_items = c.unit_items;
         pp.short_items = c.short_items;
-        pp.unit_weight = fam == Family::kMla576 ? 1 : 2;   // (a short unit's two tiles share its KV tiles)
+        pp.ranges = ranges_of(c.slots, c.unit_items);
+        pp.short_ranges = ranges_of(c.slots, c.short_items);
+        const TileTimes t = tile_times(a, fam);
+        pp.unit_us = static_cast<float>(t.unit_us);
+        pp.short_us = static_cast<float>(t.short_us);
         pp.min_len = kMinLen;
         pp.min_short_len = kMinShortLen;
         pp.lead = fam == Family::kMla576 ? kMlaLead : kLead;

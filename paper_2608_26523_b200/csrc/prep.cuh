@@ -32,11 +32,12 @@ struct PrepParams {
     int32_t unit_rows;   // query rows per unit
     int32_t short_rows;  // units of at most so many rows go to the end of the list (packed items)
     int32_t unit_block, ragged_unit_block;   // units per locality block of the item order (common.cuh): about equally long units, others
-    // Balanced cut (the library's own choice of splits for launches of few work items; see balanced_ranges):
+    // Balanced cut (the library's own choice of splits for launches of few work items):
     int32_t balanced;    // 1: cut the launch's KV tiles into equal shares of the SMs, `splits` being the most a unit may get
     int32_t slots;       // CTAs (or CTA pairs) that take work items
     int32_t unit_items, short_items;      // work items of a unit and of a short unit
-    int32_t unit_weight;                  // cost of a KV tile of a unit's item, in those of a short unit's
+    int32_t ranges, short_ranges;         // into how many equal ranges a launch of one kind of units is cut
+    float unit_us, short_us;              // time of a KV tile of an item
     int32_t min_len, min_short_len;       // fewest KV tiles worth a work item
     int32_t lead, short_lead;             // what starting and ending a work item costs, in KV tiles
     int32_t partial;     // 1: key-range restricted launch whose results are partial (o fp32, lse) of "split 0"
@@ -130,23 +131,6 @@ __device__ __forceinline__ void check_block_table(const PrepParams& p, int check
     if (threadIdx.x == 0) p.header->bad_table[checker] = any ? 2 /* VPP_DEV_BAD_BLOCK */ : 0;
 }
 
-// Into how many equal ranges the KV tiles of a launch are cut when every unit has `items` work items (one per head slot):
-// the smallest number of rounds over the slots whose items fill at least 90 % of them.
-__device__ __forceinline__ int balanced_ranges(int slots, int items) {
-    int ranges = 1;
-    float best = 0.f;
-#pragma unroll 1
-    for (int k = 1; k <= 4 && best < 0.9f; ++k) {
-        const int r = k * slots / items;
-        const float fill = static_cast<float>(r * items) / static_cast<float>(k * slots);
-        if (r >= 1 && fill > best) {
-            best = fill;
-            ranges = r;
-        }
-    }
-    return ranges;
-}
-
 __global__ void __launch_bounds__(kPrepMaxThreads, 1) prep_kernel(const PrepParams p) {
     __shared__ int2 warp_sums[32];
     __shared__ int bins[2 * kPrepMaxThreads];   // blockDim.x bins of decreasing cost, then as many for the short units
@@ -221,12 +205,10 @@ __global__ void __launch_bounds__(kPrepMaxThreads, 1) prep_kernel(const PrepPara
 
     // ---- phase 2: counting sort of the units by decreasing cost, two passes; before them, for a balanced cut, one that
     //      adds the KV tiles up: how many of them does a work item get? ----
-    // Units of one kind: their KV tiles laid end to end are cut at the multiples of `len`, so that every range is one slot's
-    // share and a unit is cut only where a share ends in it (few partial results); every unit begins with `lead` tiles that
-    // stand for the start and end of one more item in the share it begins in.  Units of both kinds: each unit by itself into
-    // parts of at most its kind's share.
+    // The KV tiles of the units of a kind (the short ones, the others) laid end to end are cut at the multiples of the kind's `len`, so
+    // that every range is one slot's share and a unit is cut only where a share ends in it (few partial results); every unit
+    // begins with `lead` tiles that stand for the start and end of one more item in the share it begins in.
     int sum = 0, sum_short = 0, len = 0, len_short = 0;
-    bool stream = false;
     float bin_scale = static_cast<float>(nthr - 1) / static_cast<float>(s_max);
     // this thread's unit, its parts: the first of `first` KV tiles, then `part` each, the last what is left (part = 0: equal parts)
     const bool once = total_units <= nthr;   // (then both are worked out once)
@@ -235,7 +217,7 @@ __global__ void __launch_bounds__(kPrepMaxThreads, 1) prep_kernel(const PrepPara
     const int first_pass = p.balanced ? 0 : 1;
 #pragma unroll 1
     for (int pass = first_pass; pass < 3; ++pass) {
-        int carry = 0;
+        int carry = 0, carry_short = 0;
 #pragma unroll 1
         for (int base = 0; base < total_units; base += nthr) {
             const int gt = base + tid;
@@ -260,8 +242,9 @@ __global__ void __launch_bounds__(kPrepMaxThreads, 1) prep_kernel(const PrepPara
             if (p.balanced && (pass == 0 || !once)) {
                 const int lead = is_short ? p.short_lead : p.lead, n = n_tiles > 0 ? n_tiles + lead : 0;
                 const int4 sc = block_scan2(is_short ? 0 : n, is_short ? n : 0, warp_sums);
-                before = carry + sc.x + sc.y + lead;
-                carry += sc.z + sc.w;
+                before = (is_short ? carry_short + sc.y : carry + sc.x) + lead;
+                carry += sc.z;
+                carry_short += sc.w;
                 if (pass == 0) {
                     sum += sc.z;
                     sum_short += sc.w;
@@ -273,16 +256,12 @@ __global__ void __launch_bounds__(kPrepMaxThreads, 1) prep_kernel(const PrepPara
                 part = 0;
                 if (p.balanced) {
                     const int most = nsplit, share = is_short ? len_short : len;
-                    if (stream) {
-                        const int least = share / 8 > 1 ? share / 8 : 1;    // no slivers: such a cut is left out
-                        first = share - before % share;
-                        if (first < least) first += share;
-                        const int last = min(n_tiles - least, pos0 / kTileN);   // (a part starts at or before the first row)
-                        nsplit = last >= first ? (last - first) / share + 2 : 1;
-                        if (nsplit > 1) part = share;
-                    } else {
-                        nsplit = (n_tiles + share - 1) / share;
-                    }
+                    const int least = share / 8 > 1 ? share / 8 : 1;    // no slivers: such a cut is left out
+                    first = share - before % share;
+                    if (first < least) first += share;
+                    const int last = min(n_tiles - least, pos0 / kTileN);   // (a part starts at or before the first row)
+                    nsplit = last >= first ? (last - first) / share + 2 : 1;
+                    if (nsplit > 1) part = share;
                     if (nsplit > most) {
                         nsplit = most;
                         part = 0;
@@ -331,17 +310,14 @@ __global__ void __launch_bounds__(kPrepMaxThreads, 1) prep_kernel(const PrepPara
         }
         __syncthreads();
         if (pass == 0) {
-            stream = sum == 0 || sum_short == 0;
-            if (stream) {
-                const int ranges = balanced_ranges(p.slots, sum ? p.unit_items : p.short_items), least = sum ? p.min_len : p.min_short_len;
-                len = (sum + sum_short + ranges - 1) / ranges;
-                if (len < least) len = least;
-                len_short = len;
-            } else {
-                const float share = (static_cast<float>(sum) * p.unit_items * p.unit_weight + static_cast<float>(sum_short) * p.short_items) / p.slots;
-                len = max(static_cast<int>(share / p.unit_weight) + 1, p.min_len);
-                len_short = max(static_cast<int>(share) + 1, p.min_short_len);
+            int ranges = p.ranges, ranges_short = p.short_ranges;
+            if (sum > 0 && sum_short > 0) {     // both kinds share the slots by the work they have
+                const float work = sum * p.unit_items * p.unit_us, work_short = sum_short * p.short_items * p.short_us;
+                ranges = max(1, static_cast<int>(p.slots * (work / (work + work_short))) / p.unit_items);
+                ranges_short = max(1, (p.slots - ranges * p.unit_items) / p.short_items);
             }
+            len = max((sum + ranges - 1) / ranges, p.min_len);
+            len_short = max((sum_short + ranges_short - 1) / ranges_short, p.min_short_len);
             const int longest = max(len, len_short);
             bin_scale = static_cast<float>(nthr - 1) / static_cast<float>(min(s_max, longest + longest / 8));
         }
