@@ -47,3 +47,12 @@ def test_more_requests_than_the_decomposition_keeps_in_shared_memory():
     prob = W.make_problem(9900, [(7 * r) % 90 for r in range(R)], [1 + (r % 3) for r in range(R)], 2, 1, 128, 128, block_size=16, std=0.8)
     out, lse, _ = run_gpu(prob.to("cuda"), 0)
     print(compare(out, lse, prob, oracle.all_rows(prob.chunk_len.numpy(), 2), "many requests"))
+
+
+@pytest.mark.parametrize("chunk", [640, 577, 650])   # whole units, one row more than nine of them, ten of them and a bit
+def test_slivers_of_long_shares(chunk):
+    """Shares of 33 KV tiles: parts from the fewest tiles worth a start on are cut off."""
+    prob = W.make_problem(9950 + chunk, [60000], [chunk], 4, 1, 128, 128, block_size=64, std=0.8)
+    rows = oracle.all_rows(prob.chunk_len.numpy(), 4)[::13]
+    out, lse, _ = run_gpu(prob.to("cuda"), 0)
+    print(compare(out, lse, prob, rows, "slivers %d" % chunk))
