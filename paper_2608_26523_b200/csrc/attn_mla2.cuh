@@ -182,26 +182,30 @@ __device__ __forceinline__ void tma2_load_5d(uint32_t dst, const CUtensorMap* m,
         "l"(reinterpret_cast<uint64_t>(m)), "r"(bar_cluster), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4)
         : "memory");
 }
-__device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t parity, uint32_t ns) {
+__device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t parity) {
     uint32_t ok;
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2, %3;\n\t"
+        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
         "selp.u32 %0, 1, 0, p;\n\t}"
         : "=r"(ok)
-        : "r"(bar), "r"(parity), "r"(ns)
+        : "r"(bar), "r"(parity)
         : "memory");
     return ok != 0;
 }
 // bounded wait with cluster-scope acquire (the barrier may have been completed by the other CTA)
 __device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity, volatile int* abort_flag, int where) {
+    if (mbar_try_wait_cluster(bar, parity)) return true;
     const long long t0 = clock64();
+    int spins = 0;
     while (true) {
-        if (mbar_try_wait_cluster(bar, parity, kWaitSleepNs)) return true;
-        if (*abort_flag != 0) return false;
-        if (clock64() - t0 > kWaitLimitCycles) {
-            atomicCAS(const_cast<int*>(abort_flag), 0, where);
-            return false;
+        if (mbar_try_wait_cluster(bar, parity)) return true;
+        if ((++spins & 63) == 0) {
+            if (*abort_flag != 0) return false;
+            if (clock64() - t0 > kWaitLimitCycles) {
+                atomicCAS(const_cast<int*>(abort_flag), 0, where);
+                return false;
+            }
         }
     }
 }

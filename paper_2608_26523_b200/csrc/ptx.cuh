@@ -48,38 +48,24 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
     return ok != 0;
 }
 
-// (the thread may sleep for up to `ns` nanoseconds before the answer is no)
-__device__ __forceinline__ bool mbar_try_wait_ns(uint32_t bar, uint32_t parity, uint32_t ns) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.acquire.cta.shared::cta.b64 p, [%1], %2, %3;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(bar), "r"(parity), "r"(ns)
-        : "memory");
-    return ok != 0;
-}
-
 // Every wait in the kernels is bounded: after kWaitLimitCycles without progress (or as soon as
 // another role has raised the CTA's abort flag) the wait gives up, records which barrier it was
 // and returns false; the caller then drains and leaves through the normal teardown.
 constexpr long long kWaitLimitCycles = 1ll << 31;  // about a second at B200 clocks
-// How long one test of a barrier may sleep.  Without it a waiting warp polls, and where many warps wait at once that costs the
-// warps that compute: in the sparse kernel (17 producer warps beside four softmax warps) the row maximum of a tile took 530 clk
-// instead of 480, 2048 tokens with lists of 2048 1315 us instead of 1291; the kernels of 8 and 12 warps do not notice.
-constexpr uint32_t kWaitSleepNs = 10000;
 
 __device__ __forceinline__ bool mbar_wait_for(uint32_t bar, uint32_t parity, volatile int* abort_flag, int where,
                                               long long limit_cycles) {
     if (mbar_try_wait(bar, parity)) return true;
     const long long t0 = clock64();
+    int spins = 0;
     while (true) {
-        if (mbar_try_wait_ns(bar, parity, kWaitSleepNs)) return true;
-        if (*abort_flag != 0) return false;
-        if (clock64() - t0 > limit_cycles) {
-            atomicCAS(const_cast<int*>(abort_flag), 0, where);
-            return false;
+        if (mbar_try_wait(bar, parity)) return true;
+        if ((++spins & 63) == 0) {
+            if (*abort_flag != 0) return false;
+            if (clock64() - t0 > limit_cycles) {
+                atomicCAS(const_cast<int*>(abort_flag), 0, where);
+                return false;
+            }
         }
     }
 }
