@@ -56,3 +56,11 @@ def test_slivers_of_long_shares(chunk):
     rows = oracle.all_rows(prob.chunk_len.numpy(), 4)[::13]
     out, lse, _ = run_gpu(prob.to("cuda"), 0)
     print(compare(out, lse, prob, rows, "slivers %d" % chunk))
+
+
+def test_forced_splits_of_more_units_than_threads():
+    """Uniform splits, placed in rounds: requests of one to four splits, 1100 units."""
+    R = 1100
+    prob = W.make_problem(9990, [(7 * r) % 500 for r in range(R)], [1 + (r % 3) for r in range(R)], 2, 1, 128, 128, block_size=16, std=0.8)
+    out, lse, _ = run_gpu(prob.to("cuda"), 4)
+    print(compare(out, lse, prob, oracle.all_rows(prob.chunk_len.numpy(), 2), "many requests, four splits"))
