@@ -336,7 +336,7 @@ int uniform_splits(const vpp_chunk_attn_args* a, int heads_per_item) {
         return best;
     }
     if (heads_per_item == 2 && a->num_reqs == 1) {
-        // One request of the d = 128 family: the work items (query tile x pair of q-heads) are about equally long, so
+        // One request of the d = 128 family: the work items (256 rows each) are about equally long, so
         // they fill the SMs in waves here too.  Measured on 8192-token chunks at 64K-128K prefixes: 512 items (3.46
         // waves) gain 7-9 % from two splits, 256 items 1.5 % from four, 128 and 1024 items are best unsplit.
         const double items = static_cast<double>((a->total_q + vpp::kTileM - 1) / vpp::kTileM) * (a->num_q_heads / 2);

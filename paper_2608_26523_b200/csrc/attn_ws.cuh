@@ -49,8 +49,6 @@ constexpr int kWsStageBytes = 8 * 32 * 128;   // 4 KB per softmax warp for the e
 constexpr int kWsSmemBytes = 2 * kTileBytes + kWsStages * kTileBytes + 1024 /*align*/ + 2048 /*barriers, ring, merge exchange*/ + kWsStageBytes;
 static_assert(kWsSmemBytes <= 232448, "shared memory of one CTA");
 constexpr float kRescaleThreshold = 8.f;      // log2 units
-// 0: P is handed to the MMA thread whole; c in 1..3: the first 32*c key columns are handed over early so that
-// O += P V can start on them while the rest of the exponentials are computed
 // Early hand-overs of P: bit c set = the key columns up to 32 (c + 1) are handed to the MMA thread as soon as they are in
 // tensor memory, so that O += P V starts on them while the rest of the exponentials are computed (0: P is handed over whole).
 constexpr int kPartMask = 3;   // after 32 and after 64 columns (measured best: a hand-over after 96 columns costs more than it gains)
