@@ -700,9 +700,10 @@ vpp_status run_chunk_attn(const vpp_chunk_attn_args* a, vpp_stream_t stream_, co
     pp.short_rows = fam == Family::kGqa128 ? rp.short_tokens : 1;
     // Item order: kv-head-major inside blocks of so many query rows.  Large blocks keep more CTAs on the same K/V pages, small
     // ones keep the order longest-first where units differ (no long one is started near the end): a first chunk of 4096 tokens
-    // and 32 heads took 205 us with blocks of 4096 rows, 186 of 512; 8192 tokens at prefix 65536 16.46 ms against 16.58.
+    // and 32 heads took 205 us with blocks of 4096 rows, 186 of 512 (and later 182, 180 of 256, 184 of 1024); 8192 tokens at prefix
+    // 65536 16.46 ms with the large blocks against 16.58.
     pp.unit_block = 4096 / pp.unit_rows > 1 ? 4096 / pp.unit_rows : 1;
-    pp.ragged_unit_block = 512 / pp.unit_rows > 1 ? 512 / pp.unit_rows : 1;
+    pp.ragged_unit_block = 256 / pp.unit_rows > 1 ? 256 / pp.unit_rows : 1;
     pp.partial = range ? 1 : 0;
     pp.range_begin = range ? range->begin_tile : 0;
     pp.range_end = range ? range->end_tile : 0;
