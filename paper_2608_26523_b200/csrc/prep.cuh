@@ -277,43 +277,50 @@ __global__ void __launch_bounds__(kPrepMaxThreads, 1) prep_kernel(const PrepPara
                 return my_bins + (b < 0 ? 0 : b);
             };
             const int ends = part > 0 ? 2 : 0;     // parts that are not of the common length
-            int slot = 0, slot_first = 0, slot_last = 0;
             // Uniform splits take their places in rounds, one split of every unit after the other: CTAs that run at the same time
             // then stream the same key range, where a unit's splits side by side kept several ranges going at once (16384
-            // tokens at 344064 keys, four splits: 187 ms, so 166).
-            const bool rounds = pass == 2 && !p.balanced && p.splits > 1;
-            if (nsplit > ends && !rounds) slot = atomicAdd(bin(part > 0 ? part : (n_tiles + nsplit - 1) / nsplit), nsplit - ends);
-            if (ends > 0) {
-                slot_first = atomicAdd(bin(first), 1);
-                slot_last = atomicAdd(bin(n_tiles - first - (nsplit - 2) * part), 1);
-            }
-            if (pass == 1) continue;
+            // tokens at 344064 keys, four splits: 187 ms, so 164).
+            const int rounds = pass == 2 && !p.balanced ? p.splits : 1;
 #pragma unroll 1
-            for (int s = 0; s < (rounds ? p.splits : nsplit); ++s) {
-                if (rounds) __syncthreads();
-                if (s >= nsplit) continue;
-                int kb, ke, at = rounds ? atomicAdd(bin((n_tiles + nsplit - 1) / nsplit), 1) : slot + s;
-                if (part > 0) {
-                    kb = s == 0 ? 0 : first + (s - 1) * part;
-                    ke = s + 1 == nsplit ? n_tiles : first + s * part;
-                    at = s == 0 ? slot_first : s + 1 == nsplit ? slot_last : at - 1;
-                } else if (p.partial) {
-                    kb = p.range_begin;
-                    ke = n_tiles < p.range_end ? n_tiles : p.range_end;
-                } else {
-                    split_range(pos0, n_tiles, nsplit, s, kb, ke);
+            for (int round = 0; round < rounds; ++round) {
+                int s0 = 0, s1 = nsplit;
+                if (rounds > 1) {
+                    __syncthreads();
+                    s0 = min(round, nsplit);
+                    s1 = min(round + 1, nsplit);
                 }
-                if (at < p.max_units) {
-                    WorkUnit u;
-                    u.req = r;
-                    u.q_row0 = qs[r] + row_off;
-                    u.rows = rows | nsplit << 16;
-                    u.pos0 = pos0;
-                    u.kv_begin = kb;
-                    u.kv_end = ke;
-                    u.split = (nsplit > 1 || p.partial) ? s : -1;
-                    u.kv_len = Ps[r] + Cs[r];
-                    p.units[at] = u;
+                int slot = 0, slot_first = 0, slot_last = 0;
+                if (s1 - s0 > ends) slot = atomicAdd(bin(part > 0 ? part : (n_tiles + nsplit - 1) / nsplit), s1 - s0 - ends) - s0;
+                if (ends > 0) {
+                    slot_first = atomicAdd(bin(first), 1);
+                    slot_last = atomicAdd(bin(n_tiles - first - (nsplit - 2) * part), 1);
+                }
+                if (pass == 1) break;
+#pragma unroll 1
+                for (int s = s0; s < s1; ++s) {
+                    int kb, ke, at = slot + s;
+                    if (part > 0) {
+                        kb = s == 0 ? 0 : first + (s - 1) * part;
+                        ke = s + 1 == nsplit ? n_tiles : first + s * part;
+                        at = s == 0 ? slot_first : s + 1 == nsplit ? slot_last : at - 1;
+                    } else if (p.partial) {
+                        kb = p.range_begin;
+                        ke = n_tiles < p.range_end ? n_tiles : p.range_end;
+                    } else {
+                        split_range(pos0, n_tiles, nsplit, s, kb, ke);
+                    }
+                    if (at < p.max_units) {
+                        WorkUnit u;
+                        u.req = r;
+                        u.q_row0 = qs[r] + row_off;
+                        u.rows = rows | nsplit << 16;
+                        u.pos0 = pos0;
+                        u.kv_begin = kb;
+                        u.kv_end = ke;
+                        u.split = (nsplit > 1 || p.partial) ? s : -1;
+                        u.kv_len = Ps[r] + Cs[r];
+                        p.units[at] = u;
+                    }
                 }
             }
         }
