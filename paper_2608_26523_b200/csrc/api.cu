@@ -619,7 +619,9 @@ vpp_status run_chunk_attn(const vpp_chunk_attn_args* a, vpp_stream_t stream_, co
     CUtensorMap tm_q, tm_qs, tm_k, tm_v, tm_kx, tm_vx;
     vpp::AttnParams ap{};
     const RowPacking rp = row_packing(a);
-    // a batch of decode rows: a packed item's box brings its one token only
+    // Tokens of a packed item, and of the box its Q copy brings.  Batches of no more tokens than requests are decode rows as a
+    // rule, with the empty slots of a server among them: one token, a small copy.  A request of several tokens in such a batch
+    // takes ordinary items (pp.short_rows below).
     const int short_box_tokens = a->total_q <= a->num_reqs ? 1 : rp.short_tokens;
     if (fam == Family::kGqa128) {
         const uint64_t dq[3] = {static_cast<uint64_t>(a->head_dim_qk), static_cast<uint64_t>(a->num_q_heads),
@@ -697,7 +699,7 @@ vpp_status run_chunk_attn(const vpp_chunk_attn_args* a, vpp_stream_t stream_, co
     }
     pp.max_units = L.max_units;
     pp.unit_rows = unit_rows_of(a, fam);
-    pp.short_rows = fam == Family::kGqa128 ? rp.short_tokens : 1;
+    pp.short_rows = fam == Family::kGqa128 ? short_box_tokens : 1;   // (a packed item has no Q rows beyond its box)
     // Item order: kv-head-major inside blocks of so many query rows.  Large blocks keep more CTAs on the same K/V pages, small
     // ones keep the order longest-first where units differ (no long one is started near the end): a first chunk of 4096 tokens
     // and 32 heads took 205 us with blocks of 4096 rows, 186 of 512 (and later 182, 180 of 256, 184 of 1024); 8192 tokens at prefix
