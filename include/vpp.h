@@ -200,8 +200,8 @@ vpp_status vpp_chunk_attn_partial_fwd(const vpp_chunk_attn_args *args, int32_t k
  *    may also be the moment the CUDA runtime loads this part of the library onto the device and
  *    reserves the array, so make it at start-up, while device memory is still available: in a process
  *    that has already handed out all device memory it can fail (VPP_ERR_CUDA, "out of memory").
- *  - With num_kv_splits = 0 the library's own split choice is dropped (the launch runs unsplit) when its partials do
- *    not fit the array.
+ *  - With num_kv_splits = 0 the library's own choice of splits is reduced to what fits the array where its partials do
+ *    not; a launch in which every query tile would be cut into the same number runs unsplit then.
  *  - A launch whose vpp_chunk_attn_workspace_size exceeds VPP_STATIC_SCRATCH_BYTES is refused
  *    with VPP_ERR_WORKSPACE and nothing is enqueued; vpp_static_last_error() says how much was needed.
  *    (Split-KV partials dominate: 4 * num_kv_splits * total_q * num_q_heads * (head_dim_v + 1) bytes.)

@@ -66,7 +66,8 @@ struct WorkspaceLayout {
     size_t lse_parts;   // float[S][total_q][Hq]
     size_t total;
     int32_t max_units;
-    int32_t splits;     // S, the uniform upper bound on splits per tile
+    int32_t splits;     // S, the most parts a unit may get
+    int32_t balanced;   // 1: the work decomposition chooses each unit's own number (prep.cuh)
 };
 
 struct AttnParams {

@@ -7,6 +7,7 @@
 #include <mutex>
 
 #include "../../include/vpp.h"
+#include "bounded.h"
 
 namespace {
 
@@ -53,7 +54,7 @@ vpp_status vpp_chunk_attn_fwd_static(const vpp_chunk_attn_args* args, vpp_stream
         return VPP_ERR_INVALID_ARG;
     }
     vpp_chunk_attn_args a = *args;
-    size_t need = vpp_chunk_attn_workspace_size(&a);
+    const size_t need = vpp::workspace_size_within(&a, VPP_STATIC_SCRATCH_BYTES);   // (its own cut as fine as fits)
     if (need == 0) {
         // invalid or unsupported arguments: report what the ordinary entry point reports for them (its argument checks
         // come before the workspace check, so nothing is enqueued)
@@ -64,12 +65,7 @@ vpp_status vpp_chunk_attn_fwd_static(const vpp_chunk_attn_args* args, vpp_stream
         snprintf(g_static_err, sizeof g_static_err, "invalid or unsupported arguments: %s", vpp_last_error());
         return st;
     }
-    if (need > VPP_STATIC_SCRATCH_BYTES && a.num_kv_splits == 0) {
-        // the split count was the library's choice (a throughput matter): an unsplit launch needs no partials
-        a.num_kv_splits = 1;
-        need = vpp_chunk_attn_workspace_size(&a);
-    }
-    if (need == 0 || need > VPP_STATIC_SCRATCH_BYTES) {
+    if (need > VPP_STATIC_SCRATCH_BYTES) {
         snprintf(g_static_err, sizeof g_static_err,
                  "this launch needs %zu bytes of scratch but the built-in scratch holds %zu: use vpp_chunk_attn_fwd "
                  "with a workspace, or lower num_kv_splits / total_q",
@@ -84,7 +80,7 @@ vpp_status vpp_chunk_attn_fwd_static(const vpp_chunk_attn_args* args, vpp_stream
     }
     a.workspace = scratch;
     a.workspace_bytes = VPP_STATIC_SCRATCH_BYTES;
-    const vpp_status st = vpp_chunk_attn_fwd(&a, stream);
+    const vpp_status st = vpp::chunk_attn_fwd_within(&a, stream, VPP_STATIC_SCRATCH_BYTES);
     if (st != VPP_OK) snprintf(g_static_err, sizeof g_static_err, "%s", vpp_last_error());
     return st;
 }
