@@ -83,21 +83,52 @@ __device__ __forceinline__ bool append_scan(const AppendParams& p, int32_t* cu) 
     return !s_bad && cu[p.num_reqs] == p.total_q;
 }
 
-// The verdict on the launch (one block): lengths, and the pages of every row.
-__device__ __forceinline__ void append_status(const AppendParams& p, bool lengths_ok) {
+// Request of row g (0 <= g < total_q): the last r with cu[r] <= g.
+__device__ __forceinline__ int append_request(const int32_t* cu, int num_reqs, int g) {
+    int lo = 0, hi = num_reqs - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (cu[mid] <= g) lo = mid; else hi = mid - 1;
+    }
+    return lo;
+}
+
+// The verdict on the launch (one block): lengths, and the pages of every row.  Looked up are the pages of each request's first and
+// last row and of every block_size-th row of the launch: rows of a request that follow one another among these are at most a page
+// apart, so every page is among theirs.  The threads share the rows, not the requests (one long chunk among many short ones: 8192
+// rows in pages of 16 and 255 single rows took 37 us with a thread walking the long one's pages, 11.6 now), with kAppendProbes look-ups in flight each.
+constexpr int kAppendProbes = 4;
+__device__ __forceinline__ void append_status(const AppendParams& p, const int32_t* cu, bool lengths_ok) {
     bool bad = false;
     if (lengths_ok && p.block_table != nullptr) {
-        const int per_req = p.num_reqs < kAppendThreads ? kAppendThreads / p.num_reqs : 1;   // threads that share a request
-        const int groups = kAppendThreads / per_req, grp = threadIdx.x / per_req, part = threadIdx.x % per_req;
-        for (int r = grp; r < p.num_reqs && grp < groups; r += groups) {
-            const int pre = p.prefix_len[r], c = p.chunk_len[r];
-            if (c == 0) continue;
-            const int32_t* row = p.block_table + static_cast<long long>(r) * p.max_blocks_per_req;
-            const int last = (pre + c - 1) >> p.block_shift;
-            for (int b = (pre >> p.block_shift) + part; b <= last; b += per_req) {
-                const int e = __ldg(row + b);
-                bad |= e < 0 || e >= p.num_blocks;
+        auto outside = [&](int r, int pos) {
+            const int e = __ldg(p.block_table + static_cast<long long>(r) * p.max_blocks_per_req + (pos >> p.block_shift));
+            return e < 0 || e >= p.num_blocks;
+        };
+        for (int r0 = threadIdx.x; r0 < p.num_reqs; r0 += kAppendProbes * kAppendThreads) {
+            int pre[kAppendProbes], n[kAppendProbes];
+#pragma unroll
+            for (int i = 0; i < kAppendProbes; ++i) {
+                const int r = r0 + i * kAppendThreads;
+                n[i] = r < p.num_reqs ? cu[r + 1] - cu[r] : 0;
+                pre[i] = n[i] > 0 ? __ldg(p.prefix_len + r) : 0;
             }
+#pragma unroll
+            for (int i = 0; i < kAppendProbes; ++i)
+                if (n[i] > 0) bad |= outside(r0 + i * kAppendThreads, pre[i]) | outside(r0 + i * kAppendThreads, pre[i] + n[i] - 1);
+        }
+        const long long step = 1ll << p.block_shift;
+        for (long long g0 = threadIdx.x * step; g0 < p.total_q; g0 += kAppendProbes * kAppendThreads * step) {
+            int r[kAppendProbes], pos[kAppendProbes];
+#pragma unroll
+            for (int i = 0; i < kAppendProbes; ++i) {
+                const long long g = g0 + i * kAppendThreads * step;
+                r[i] = g < p.total_q ? append_request(cu, p.num_reqs, static_cast<int>(g)) : -1;
+                pos[i] = r[i] >= 0 ? __ldg(p.prefix_len + r[i]) + static_cast<int>(g - cu[r[i]]) : 0;
+            }
+#pragma unroll
+            for (int i = 0; i < kAppendProbes; ++i)
+                if (r[i] >= 0) bad |= outside(r[i], pos[i]);
         }
     }
     const int any = __syncthreads_or(bad);
@@ -112,7 +143,7 @@ __global__ void __launch_bounds__(kAppendThreads) kv_append_kernel(const AppendP
     pdl_wait();                       // the rows and the lengths may come from the kernel launched just before
     const bool ok = append_scan(p, cu);
     if (static_cast<int>(blockIdx.x) >= copy_blocks) {
-        append_status(p, ok);
+        append_status(p, cu, ok);
         return;
     }
     if (!ok) return;                  // lengths that do not describe this launch: write nothing
@@ -133,11 +164,7 @@ __global__ void __launch_bounds__(kAppendThreads) kv_append_kernel(const AppendP
         long long blk = 0;
         int slot = 0;
         if (lane == 0) {
-            int lo = 0, hi = p.num_reqs;          // last r with cu[r] <= row
-            while (hi - lo > 1) {
-                const int mid = (lo + hi) >> 1;
-                if (cu[mid] <= row) lo = mid; else hi = mid;
-            }
+            const int lo = append_request(cu, p.num_reqs, row);
             const int pos = p.prefix_len[lo] + (row - cu[lo]);
             if (p.block_table == nullptr) {
                 blk = lo;
