@@ -641,21 +641,20 @@ vpp_status run_chunk_attn(const vpp_chunk_attn_args* a, vpp_stream_t stream_, co
     const int box_rows = paged ? (B < tile_n ? B : tile_n) : tile_n;
 
     // ---- tensor maps ----
-    CUtensorMap tm_q, tm_qs, tm_k, tm_v, tm_kx, tm_vx;
+    CUtensorMap tm_q, tm_qs, tm_q1, tm_k, tm_v, tm_kx, tm_vx;
     vpp::AttnParams ap{};
     const RowPacking rp = row_packing(a);
-    // Tokens of a packed item, and of the box its Q copy brings.  Batches of no more tokens than requests are decode rows as a
-    // rule, with the empty slots of a server among them: one token, a small copy.  A request of several tokens in such a batch
-    // takes ordinary items (pp.short_rows below).
-    const int short_box_tokens = a->total_q <= a->num_reqs ? 1 : rp.short_tokens;
     if (fam == Family::kGqa128) {
         const uint64_t dq[3] = {static_cast<uint64_t>(a->head_dim_qk), static_cast<uint64_t>(a->num_q_heads),
                                 static_cast<uint64_t>(a->total_q)};
         const uint64_t sq[2] = {static_cast<uint64_t>(a->head_dim_qk) * 2,
                                 static_cast<uint64_t>(a->head_dim_qk) * a->num_q_heads * 2};
         const uint32_t bq[3] = {64, static_cast<uint32_t>(rp.group), static_cast<uint32_t>(rp.tile_tokens)};
-        const uint32_t bs[3] = {64, static_cast<uint32_t>(rp.short_group), static_cast<uint32_t>(short_box_tokens)};
-        if (!make_tmap(&tm_q, a->q, 3, dq, sq, bq) || !make_tmap(&tm_qs, a->q, 3, dq, sq, bs))
+        // a packed item of one token has a box of its own: with the box of all the tokens that such an item may have, 256 decode rows
+        // of 64/8 heads took 546 us instead of 538
+        const uint32_t b1[3] = {64, static_cast<uint32_t>(rp.short_group), 1};
+        const uint32_t bs[3] = {64, static_cast<uint32_t>(rp.short_group), static_cast<uint32_t>(rp.short_tokens)};
+        if (!make_tmap(&tm_q, a->q, 3, dq, sq, bq) || !make_tmap(&tm_qs, a->q, 3, dq, sq, bs) || !make_tmap(&tm_q1, a->q, 3, dq, sq, b1))
             return fail(VPP_ERR_CUDA, "cuTensorMapEncodeTiled(q) failed");
         ap.exact_from = paged || B % vpp::kExactRows == 0 ? INT32_MAX : B / vpp::kExactRows * vpp::kExactRows;
         if (!make_kv_maps(a->k_cache, a->k_block_stride, a->k_token_stride, a->k_head_stride, B, n_blocks, a->num_kv_heads, box_rows, &tm_k,
@@ -724,7 +723,7 @@ vpp_status run_chunk_attn(const vpp_chunk_attn_args* a, vpp_stream_t stream_, co
     }
     pp.max_units = L.max_units;
     pp.unit_rows = unit_rows_of(a, fam);
-    pp.short_rows = fam == Family::kGqa128 ? short_box_tokens : 1;   // (a packed item has no Q rows beyond its box)
+    pp.short_rows = fam == Family::kGqa128 ? rp.short_tokens : 1;   // (the box of a packed item's Q copy)
     // Item order: kv-head-major inside blocks of so many query rows.  Large blocks keep more CTAs on the same K/V pages, small
     // ones keep the order longest-first where units differ (no long one is started near the end): a first chunk of 4096 tokens
     // and 32 heads took 205 us with blocks of 4096 rows, 186 of 512 (and later 182, 180 of 256, 184 of 1024); 8192 tokens at prefix
@@ -767,7 +766,7 @@ vpp_status run_chunk_attn(const vpp_chunk_attn_args* a, vpp_stream_t stream_, co
     ap.group = rp.group;
     ap.tile_tokens = rp.tile_tokens;
     ap.short_group = rp.short_group;
-    ap.short_box_tokens = short_box_tokens;
+    ap.short_tokens = rp.short_tokens;
     ap.scale_log2e = a->softmax_scale * 1.4426950408889634f;
     ap.out = a->out;
     ap.lse = a->lse;
@@ -795,8 +794,8 @@ vpp_status run_chunk_attn(const vpp_chunk_attn_args* a, vpp_stream_t stream_, co
         auto kern = v_warp ? vpp::attn128_ws_kernel<true> : vpp::attn128_ws_kernel<false>;
         ce = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, vpp::kWsSmemBytes);
         if (ce == cudaSuccess)
-            ce = launch(kern, static_cast<unsigned>(sms), vpp::kWsThreads, vpp::kWsSmemBytes, stream, tm_q, tm_qs, tm_k, tm_v, tm_kx, tm_vx,
-                        ap, box_rows);
+            ce = launch(kern, static_cast<unsigned>(sms), vpp::kWsThreads, vpp::kWsSmemBytes, stream, tm_q, tm_qs, tm_q1, tm_k, tm_v, tm_kx,
+                        tm_vx, ap, box_rows);
     }
     if (ce != cudaSuccess) return fail(VPP_ERR_CUDA, "attention kernel attributes: %s", cudaGetErrorString(ce));
     ++g_launches;

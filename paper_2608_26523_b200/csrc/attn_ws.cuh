@@ -128,12 +128,12 @@ constexpr int kExactRows = 8;                 // keys per copy of the exact map
 
 template <bool kVWarp>
 __global__ void __launch_bounds__(kWsThreads, 1)
-attn128_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_qs,
+attn128_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_qs, const __grid_constant__ CUtensorMap tm_q1,
                   const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
                   const __grid_constant__ CUtensorMap tm_kx, const __grid_constant__ CUtensorMap tm_vx, const AttnParams p,
                   const int kv_box_rows) {
     // tm_q:  q with a box of (64 features, group heads, tile_tokens tokens): one 64-column slab of a tile
-    // tm_qs: the same with (64, short_group, short_box_tokens), for packed items
+    // tm_qs / tm_q1: the same with (64, short_group, short_tokens) and (64, short_group, 1), for packed items of several tokens and of one
     // tm_k / tm_v: (64 features, 8 keys, 2 halves, 8-key groups, (block, kv-head)), box (64, 8, 2, kv_box_rows / 8, 1): the keys of
     //        a page, or of a whole tile where pages are that large
     // tm_kx / tm_vx: (64 features, keys, 2 halves, kv-head, block), box (64, 8, 2, 1, 1): eight keys, the extent of the keys exact --
@@ -197,6 +197,7 @@ attn128_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
         prefetch_tmap(&tm_k);
         prefetch_tmap(&tm_v);
         prefetch_tmap(&tm_qs);
+        prefetch_tmap(&tm_q1);
     }
     __syncthreads();
     if (warp == 2) {
@@ -334,9 +335,11 @@ attn128_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                     // (tokens past the end of q read as zero; rows of a following request are never stored; tile rows the
                     // boxes do not cover keep whatever they held)
                     if (ok && packed) {
-                        mbar_arrive_expect_tx(bar_q_full, 2 * p.short_group * p.short_box_tokens * 128);
-                        tma_load_3d(sQ, &tm_qs, bar_q_full, 0, h0, u.q_row0);
-                        tma_load_3d(sQ + kSlabBytes, &tm_qs, bar_q_full, 64, h0, u.q_row0);
+                        const bool one = (u.rows & 0xffff) == 1;
+                        const CUtensorMap* tm = one ? &tm_q1 : &tm_qs;
+                        mbar_arrive_expect_tx(bar_q_full, 2 * p.short_group * (one ? 1 : p.short_tokens) * 128);
+                        tma_load_3d(sQ, tm, bar_q_full, 0, h0, u.q_row0);
+                        tma_load_3d(sQ + kSlabBytes, tm, bar_q_full, 64, h0, u.q_row0);
                     } else if (ok) {
                         mbar_arrive_expect_tx(bar_q_full, 4 * p.group * p.tile_tokens * 128);
 #pragma unroll

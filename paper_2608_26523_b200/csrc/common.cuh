@@ -80,7 +80,7 @@ struct AttnParams {
     int32_t total_q;
     // d = 128 kernel, how tile rows are packed: row r of a tile is q-head h0 + r % group of token r / group
     int32_t group, tile_tokens;               // items of two tiles
-    int32_t short_group, short_box_tokens;    // items of one tile (short units); tokens a copy of its Q tile brings
+    int32_t short_group, short_tokens;        // items of one tile (short units)
     // d = 128 kernel, K/V copies: (block b, kv-head g) is coordinate b * block_units + g * head_units of a cache's map
     int32_t k_block_units, k_head_units, k_end;   // (k_end: one past the last: reads as zero)
     int32_t v_block_units, v_head_units, v_end;
