@@ -603,7 +603,7 @@ dsa_attn_kernel(const __grid_constant__ CUtensorMap tm_qh, const __grid_constant
                             stage_put(stage, lane, hf * 4 + q4, make_uint4(w[0], w[1], w[2], w[3]));
                         }
                     }
-                    stage_flush(stage, lane, [&](int i) -> uint8_t* {
+                    stage_flush(stage, lane, 32, [&](int i) -> uint8_t* {
                         return i < warp_rows ? static_cast<uint8_t*>(p.out) + ((first_row + i * row_step) * kMlaDv + (k >> 1) * 256 + half * 128 + (k & 1) * 64) * 2
                                              : nullptr;
                     });
@@ -619,7 +619,7 @@ dsa_attn_kernel(const __grid_constant__ CUtensorMap tm_qh, const __grid_constant
                         stage_put(stage, lane, q4,
                                   make_uint4(__float_as_uint(__uint_as_float(r[q4 * 4]) * inv_l), __float_as_uint(__uint_as_float(r[q4 * 4 + 1]) * inv_l),
                                              __float_as_uint(__uint_as_float(r[q4 * 4 + 2]) * inv_l), __float_as_uint(__uint_as_float(r[q4 * 4 + 3]) * inv_l)));
-                    stage_flush(stage, lane, [&](int i) -> uint8_t* {
+                    stage_flush(stage, lane, 32, [&](int i) -> uint8_t* {
                         return i < warp_rows ? reinterpret_cast<uint8_t*>(p.o_parts + (first_row + i * row_step) * kMlaDv + (c >> 2) * 256 + half * 128 + (c & 3) * 32)
                                              : nullptr;
                     });

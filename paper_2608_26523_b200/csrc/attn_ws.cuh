@@ -755,7 +755,7 @@ attn128_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                                 stage_put(stage, lane, hf * 4 + q4, make_uint4(w[0], w[1], w[2], w[3]));
                             }
                         }
-                        stage_flush(stage, lane, [&](int i) -> uint8_t* {
+                        stage_flush(stage, lane, 32, [&](int i) -> uint8_t* {
                             const int orow = __shfl_sync(0xffffffffu, out_row0, i);
                             return warp_row0 + i < tile_rows ? static_cast<uint8_t*>(p.out) + (static_cast<long long>(orow) * 128 + c * 64) * 2 : nullptr;
                         });
@@ -772,7 +772,7 @@ attn128_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                             stage_put(stage, lane, q4,
                                       make_uint4(__float_as_uint(__uint_as_float(r[q4 * 4]) * inv_l), __float_as_uint(__uint_as_float(r[q4 * 4 + 1]) * inv_l),
                                                  __float_as_uint(__uint_as_float(r[q4 * 4 + 2]) * inv_l), __float_as_uint(__uint_as_float(r[q4 * 4 + 3]) * inv_l)));
-                        stage_flush(stage, lane, [&](int i) -> uint8_t* {
+                        stage_flush(stage, lane, 32, [&](int i) -> uint8_t* {
                             const int orow = __shfl_sync(0xffffffffu, out_row0, i);
                             return warp_row0 + i < tile_rows ? reinterpret_cast<uint8_t*>(p.o_parts + (part0 + orow) * 128 + c * 32) : nullptr;
                         });

@@ -237,10 +237,22 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
 __device__ __forceinline__ void stage_put(uint8_t* stage, int lane, int q, uint4 v) {
     *reinterpret_cast<uint4*>(stage + lane * 128 + ((q ^ (lane & 7)) << 4)) = v;
 }
-// row_of(r): address of row r's 128 bytes, or null if the row is not to be written (r: row of the warp's 32)
+// row_of(r): address of row r's 128 bytes, or null if the row is not to be written (r: row of the warp's 32); rows: how many of them
+// are (at most eight, as of a request of few tokens, take two of the eight steps: MLA, eight requests of eight tokens with two
+// splits, 390 -> 376 us)
 template <typename RowOf>
-__device__ __forceinline__ void stage_flush(const uint8_t* stage, int lane, RowOf row_of) {
+__device__ __forceinline__ void stage_flush(const uint8_t* stage, int lane, int rows, RowOf row_of) {
     __syncwarp();
+    if (rows <= 8) {
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const int r = 4 * i + (lane >> 3), q = lane & 7;
+            uint8_t* dst = row_of(r);
+            if (dst) *reinterpret_cast<uint4*>(dst + q * 16) = *reinterpret_cast<const uint4*>(stage + r * 128 + ((q ^ (r & 7)) << 4));
+        }
+        __syncwarp();
+        return;
+    }
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
         const int r = 4 * i + (lane >> 3), q = lane & 7;
