@@ -716,6 +716,9 @@ vpp_status run_chunk_attn(const vpp_chunk_attn_args* a, vpp_stream_t stream_, co
         const TileTimes t = tile_times(a, fam);
         pp.unit_us = static_cast<float>(t.unit_us);
         pp.short_us = static_cast<float>(t.short_us);
+        pp.short_per_unit = static_cast<float>(t.short_us / t.unit_us);
+        // (several requests, not all of them decode rows: the others have units of one kind, or of one length)
+        pp.lead_items = fam == Family::kGqa128 && a->num_reqs > 1 && a->total_q > a->num_reqs ? 4 * c.slots : 0;
         pp.min_len = kMinLen;
         pp.min_short_len = kMinShortLen;
         pp.lead = fam == Family::kMla576 ? kMlaLead : kLead;

@@ -215,12 +215,13 @@ attn128_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
     if (blockIdx.x == 0 && tid == 0 && p.status) *p.status = list.error;
     const int G = p.num_q_heads / p.num_kv_heads;
     // Items: the short units' (unit, group of q-heads), which run packed (their groups are larger where a kv-head's group
-    // does not fill a tile well), then those of the units of two tiles.  The short units come first because decode rows
-    // sit at the end of long contexts: one of them started last would run alone.
+    // does not fill a tile well), and those of the units of two tiles.  Whatever is long comes early, since such an item started
+    // last would run alone: the short ones, which sit at the end of long contexts, in a batch of few items behind the units that take longer than any of
+    // them (prep.cuh), then the rest.
     const int num_packed = list.num_short;
     const int num_normal = list.num_units - num_packed;
     const int normal_slots = p.num_q_heads / p.group, packed_slots = p.num_q_heads / p.short_group;
-    const int packed_items = num_packed * packed_slots, unit_block = list.unit_block;
+    const int packed_items = num_packed * packed_slots, unit_block = list.unit_block, lead_items = list.num_lead * normal_slots;
     const int total_items = packed_items + num_normal * normal_slots;
 
     if (warp < 4) {
@@ -304,13 +305,14 @@ attn128_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                 WorkUnit u{};
                 int h0 = 0;
                 bool packed = false;
-                if (have && item < packed_items) {
-                    u = p.units[num_normal + item / packed_slots];
-                    h0 = (item % packed_slots) * p.short_group;
-                    packed = true;
+                packed = have && static_cast<uint32_t>(item - lead_items) < static_cast<uint32_t>(packed_items);
+                if (packed) {
+                    const int k = item - lead_items;
+                    u = p.units[num_normal + k / packed_slots];
+                    h0 = (k % packed_slots) * p.short_group;
                 } else if (have) {
                     int ui, hs;
-                    decode_item(item - packed_items, num_normal, unit_block, normal_slots, G / p.group, ui, hs);
+                    decode_item(item < lead_items ? item : item - packed_items, num_normal, unit_block, normal_slots, G / p.group, ui, hs);
                     u = p.units[ui];
                     h0 = hs * p.group;
                 }

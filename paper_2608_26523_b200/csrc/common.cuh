@@ -37,24 +37,25 @@ struct __align__(16) WorkHeader {
     int32_t error;        // VPP_DEV_* (0 = ok) of the lengths
     int32_t counter;      // persistent-kernel work counter
     int32_t num_checkers; // blocks that checked a part of the block table
-    int32_t pad[2];
+    int32_t num_lead;     // units at the start of the list that are handed out before the short ones (d = 128 kernel)
+    int32_t pad;
     int32_t bad_table[kMaxCheckers];   // one word each: VPP_DEV_BAD_BLOCK if it found an entry out of range, else 0
 };
 static_assert(kMaxCheckers == 8, "read_header");
 
 // The head of the work list as the kernels after the decomposition see it: nothing to do when a check failed.
 struct WorkList {
-    int32_t num_units, num_short, unit_block, error;
+    int32_t num_units, num_short, unit_block, error, num_lead;
 };
 __device__ __forceinline__ WorkList read_header(const WorkHeader* h) {
     const int4* q = reinterpret_cast<const int4*>(h);
     const int4 a = q[0], b = q[1], c = q[2], d = q[3];   // (independent loads: one round trip)
     const int bad[8] = {c.x, c.y, c.z, c.w, d.x, d.y, d.z, d.w};
-    WorkList w{a.x, a.y, a.z, a.w};
+    WorkList w{a.x, a.y, a.z, a.w, b.z};
 #pragma unroll
     for (int i = 0; i < 8; ++i)
         if (w.error == 0 && i < b.y) w.error = bad[i];
-    if (w.error != 0) w.num_units = w.num_short = 0;
+    if (w.error != 0) w.num_units = w.num_short = w.num_lead = 0;
     return w;
 }
 

@@ -38,6 +38,8 @@ struct PrepParams {
     int32_t unit_items, short_items;      // work items of a unit and of a short unit
     int32_t ranges, short_ranges;         // into how many equal ranges a launch of one kind of units is cut
     float unit_us, short_us;              // time of a KV tile of an item
+    float short_per_unit;                 // short_us / unit_us
+    int32_t lead_items;                   // launches of fewer items put the long units of two tiles before the short ones (0: none)
     int32_t min_len, min_short_len;       // fewest KV tiles worth a work item
     int32_t lead, short_lead;             // what starting and ending a work item costs, in KV tiles
     int32_t partial;     // 1: key-range restricted launch whose results are partial (o fp32, lse) of "split 0"
@@ -131,11 +133,23 @@ __device__ __forceinline__ void check_block_table(const PrepParams& p, int check
     if (threadIdx.x == 0) p.header->bad_table[checker] = any ? 2 /* VPP_DEV_BAD_BLOCK */ : 0;
 }
 
+// In a batch of few items, the units of two tiles that take longer than the longest short one go before the short ones: those in front
+// of the bin of this length.  (64 tokens at 8000 keys and 30 decode rows at 4000 to 4400 of 64/8 heads: 212 us with all of them at
+// the end, 155 so.  Where there are several items to a slot the end is filled anyway: a mixed batch of 14 lost 0.5 %.)
+// (out of line: see block_scan2)
+__device__ __noinline__ void put_long_units_first(WorkHeader* header, const int* bins, int short_bin, float bin_scale, float short_per_unit,
+                                                  int lead, int short_lead) {
+    const int nthr = blockDim.x;
+    const float as_long = (2 * nthr - 1 - short_bin) * short_per_unit + (short_lead * short_per_unit - lead) * bin_scale;
+    if (threadIdx.x == 0) header->num_lead = bins[min(max(nthr - 1 - static_cast<int>(as_long), 0), nthr - 1)];
+    __syncthreads();
+}
+
 __global__ void __launch_bounds__(kPrepMaxThreads, 1) prep_kernel(const PrepParams p) {
     __shared__ int2 warp_sums[32];
     __shared__ int bins[2 * kPrepMaxThreads];   // blockDim.x bins of decreasing cost, then as many for the short units
     __shared__ int s_P[kPrepSmemReqs], s_C[kPrepSmemReqs], s_q[kPrepSmemReqs], s_t[kPrepSmemReqs + 1];
-    __shared__ int s_error, s_max, s_min;
+    __shared__ int s_error, s_max, s_min, s_normal, s_items, s_short_bin;
     const int tid = threadIdx.x, nthr = blockDim.x;
     pdl_launch_dependents();   // the attention kernel may set itself up (barriers, tensor memory) while this runs
     pdl_wait();                // the lengths may come from the kernel launched just before; the workspace may be in use by it
@@ -152,6 +166,7 @@ __global__ void __launch_bounds__(kPrepMaxThreads, 1) prep_kernel(const PrepPara
         s_error = 0;
         s_max = 1;
         s_min = 1 << 30;
+        s_short_bin = 2 * nthr;
         p.header->num_checkers = gridDim.x - 1;
     }
     bins[tid] = 0;
@@ -343,6 +358,7 @@ __global__ void __launch_bounds__(kPrepMaxThreads, 1) prep_kernel(const PrepPara
             const int4 sc = block_scan2(b0 + b1, 0, warp_sums);
             bins[2 * tid] = sc.x;
             bins[2 * tid + 1] = sc.x + b0;
+            if (p.lead_items > 0 && 2 * tid >= nthr && b0 + b1 > 0) atomicMin(&s_short_bin, b0 > 0 ? 2 * tid : 2 * tid + 1);   // the longest short unit's
             if (2 * tid == nthr) {   // the first of the short units' bins
                 const int n = sc.z < p.max_units ? sc.z : p.max_units;
                 p.header->num_units = n;
@@ -353,8 +369,13 @@ __global__ void __launch_bounds__(kPrepMaxThreads, 1) prep_kernel(const PrepPara
                 p.header->unit_block = p.balanced ? 1 : 4 * s_min >= 3 * s_max ? p.unit_block : p.ragged_unit_block;
                 p.header->counter = 0;
                 p.header->error = 0;
+                p.header->num_lead = 0;
+                s_normal = sc.x;
+                s_items = sc.x * p.unit_items + (sc.z - sc.x) * p.short_items;
             }
             __syncthreads();
+            if (p.lead_items > 0 && s_normal > 0 && s_short_bin < 2 * nthr && s_items < p.lead_items)
+                put_long_units_first(p.header, bins, s_short_bin, bin_scale, p.short_per_unit, p.lead, p.short_lead);
         }
     }
 }
