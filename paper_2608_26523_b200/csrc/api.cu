@@ -416,6 +416,7 @@ ItemCounts item_counts(const vpp_chunk_attn_args* a, Family fam) {
 // The start and end of a work item (query load, first K/V, epilogue) in KV tiles: ~4 us of ~2 us a tile; packed items
 // ~4.5 us of ~1.5 us; MLA items (144 KB of queries, 256 KB of partial results) ~9 us of ~1.9.
 constexpr int kLead = 2, kShortLead = 3, kMlaLead = 5;
+constexpr double kL2Keeps = 96e6;   // bytes of keys and values that stay in the 126 MB of L2 while a launch goes over them
 constexpr int kMinLen = 2, kMinShortLen = 4;   // fewest KV tiles worth a work item (start-up ~4 us, ~2 / ~1 us per tile)
 
 // Time of a KV tile of a work item, measured at full clock.  (Packed items have a producer warp for V of their own in decode
@@ -444,7 +445,27 @@ int ranges_of(int slots, int items) {
     return best;
 }
 
-// most: parts a unit of a balanced cut may get.
+// Equal splits of one request's chunk, and the time they take: waves of items, the last of them as idle as the items are equally long
+// (a chunk that is half the context or more has items of all lengths, which go longest first), and the partial results (whose
+// stores mostly hide behind the items).  Measured on 8192-token chunks at 64K-128K prefixes: 512 items (3.46 waves) gain 7-9 % from two splits, 256 items 1.5 % from
+// four, 128 and 1024 items are best unsplit.
+int chunk_splits(long long items, int slots, double tiles, double chunk_tiles, double unit_us, double parts_us, int most, double* us) {
+    const double mean = tiles - 0.5 * chunk_tiles, equal = chunk_tiles < 0.5 * tiles ? 1.0 - chunk_tiles / tiles : 0.0;
+    int best = 1;
+    for (int s = 1; s <= 8 && s <= most; ++s) {
+        if (s > 1 && tiles / s < 4.0) break;   // keep at least 4 KV tiles per split
+        const double w = static_cast<double>(items) * s / slots;
+        const double waves = std::fmax(w + (std::ceil(w) - w) * equal, 1.0);
+        const double t = std::fmax(waves * (mean / s + kLead), tiles / s + kLead) * unit_us * (1.0 + 0.01 * (s - 1)) + (s > 1 ? 8.0 + 0.4 * parts_us * s : 0.0);
+        if (s == 1 || t < 0.975 * *us) {
+            best = s;
+            *us = t;
+        }
+    }
+    return best;
+}
+
+// most: parts a unit of a launch of few items may get.
 SplitPlan plan_splits(const vpp_chunk_attn_args* a, Family fam, int most = vpp::kMergeMaxSplits) {
     if (a->num_kv_splits >= 1) return {a->num_kv_splits, false};
     if (a->total_q <= 0 || a->num_reqs <= 0) return {1, false};
@@ -459,6 +480,8 @@ SplitPlan plan_splits(const vpp_chunk_attn_args* a, Family fam, int most = vpp::
     //  least idle last wave, below; MLA's pairs of SMs take their items in a fixed order, so more items than pairs are left alone:
     //  110 decode rows 75 us uncut, 88 cut; mixed batches of d = 128: up to two items per slot)
     const bool few = mla ? items <= c.slots : decode || one_request ? items * 5 < c.slots * 4ll : items < 2ll * c.slots;
+    const double chunk_tiles = a->total_q / static_cast<double>(vpp::kTileN);
+    const double parts_us = 8.0 * a->total_q * a->num_q_heads * a->head_dim_v / 3e6;      // of one partial result per row, written and read
     if (few) {
         // Is it worth it?  Uncut, the longest unit takes tiles * us, or a ragged batch of more items than slots about half of that
         // after the mean ends.  Cut, everybody takes its share, plus the decomposition's and the merge's part and the partial
@@ -466,14 +489,23 @@ SplitPlan plan_splits(const vpp_chunk_attn_args* a, Family fam, int most = vpp::
         // are taken to end there, a batch's to be half as long.)  200 tokens of 64 heads at 2048 keys: 40 us uncut, 47 cut; 256 tokens of 4
         // heads at 1024 keys 24 uncut, 21 cut.
         const TileTimes t = tile_times(a, fam);
-        const double us = decode ? t.short_us : t.unit_us, mean = one_request ? (decode ? tiles : tiles - a->total_q / 256.0) : 0.5 * tiles;
+        const double us = decode ? t.short_us : t.unit_us, mean = one_request ? (decode ? tiles : tiles - 0.5 * chunk_tiles) : 0.5 * tiles;
         const int least = decode ? kMinShortLen : kMinLen;
         double share = mean * units / ranges_of(c.slots, per_unit);
         if (share < least) share = least;
         if (share < mean / most) share = mean / most;
         const double uncut_us = us * (items <= c.slots ? tiles : std::fmax(tiles, mean * items / c.slots + 0.5 * tiles));
-        const double parts_us = 8.0 * a->total_q * a->num_q_heads * a->head_dim_v / 3e6;      // of one partial result per row
-        const double cut_us = us * share + (decode && !mla ? 6.0 : 8.0) + parts_us * (mean / share > 1 ? mean / share : 1);
+        double cut_us = us * share + (decode && !mla ? 6.0 : 8.0) + parts_us * (mean / share > 1 ? mean / share : 1);
+        const double kv_bytes = 512.0 * a->max_seq_len * a->num_kv_heads;
+        if (one_request && !mla && units > 1 && kv_bytes > kL2Keeps) {
+            // The parts of a balanced cut read different keys at the same time, so that every unit fetches keys that L2 does not keep
+            // from memory for itself (4.1 TB/s); equal splits of all units go over them together.  400 tokens of 64/8 heads at 65536 keys
+            // 949 us balanced, 804 equal; 256 tokens of 64/4 heads at 131072 keys 1003, 944; 300 of 32/8 there 684, 600.
+            cut_us = std::fmax(cut_us, units * kv_bytes / 4.1e6 + 8.0);
+            double equal_us = 0;
+            const int equal = chunk_splits(items, c.slots, tiles, chunk_tiles, us, parts_us, most, &equal_us);
+            if (equal_us < cut_us) return {equal, false};
+        }
         if (cut_us >= uncut_us) return {1, false};
         // what a unit may need: its share of the slots when all are equally long; several times that when they are ragged (one
         // long context among short ones gets most of the slots)
@@ -533,13 +565,13 @@ vpp::WorkspaceLayout layout_of(const vpp_chunk_attn_args* a, Family fam, SplitPl
 
 // The layout of a launch whose workspace may hold `limit` bytes: where the library's own cut needs more, its units get fewer parts
 // (2048 tokens of 8/1 heads at 16369 keys: 32.3 MiB with four, 24.2 with three; 119 us, 137, and 229 uncut), and none if that does
-// not do.  A cut of all units into the same number is not made coarser: that number was chosen for how the items fill the SMs.
+// not do.  The equal splits of a launch that fills the SMs are not made fewer: their number is that of the best last wave.
 vpp::WorkspaceLayout layout_for(const vpp_chunk_attn_args* a, Family fam, size_t limit) {
     SplitPlan plan = plan_splits(a, fam);
     vpp::WorkspaceLayout L = layout_of(a, fam, plan);
     if (L.total <= limit || a->num_kv_splits != 0 || plan.splits == 1) return L;
     const vpp::WorkspaceLayout uncut = layout_of(a, fam, {1, false});
-    if (!plan.balanced || uncut.total > limit) return uncut;
+    if (uncut.total > limit) return uncut;
     const size_t part = (L.total - uncut.total) / (plan.splits - 1);     // bytes that one more part takes
     for (int most = 1 + static_cast<int>((limit - uncut.total) / part); most > 1; --most) {   // (the first or, by alignment, the second fits)
         plan = plan_splits(a, fam, most);

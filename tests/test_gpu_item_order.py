@@ -72,3 +72,13 @@ def test_chunks_of_longer_items_go_before_decode_rows(chunk, rows, hq, hkv, firs
     longer = [u for u in normal if us(u) > 1.05 * longest]                  # (bins of lengths: 1 / 128 of the longest)
     assert all(us(u) > 0.95 * longest for u in normal[:head["lead"]])
     assert head["lead"] >= len(longer) > 0 if first else head["lead"] == 0, (head, len(longer))
+
+
+@pytest.mark.parametrize("hq,hkv,chunk,seq", [(64, 8, 400, 65536), (32, 8, 300, 131072), (32, 16, 512, 32768)])
+def test_units_whose_keys_exceed_l2_are_cut_at_the_same_places(hq, hkv, chunk, seq):
+    """Equal splits of all units: units that run together go over the same keys."""
+    head, units = _launch([seq - chunk], [chunk], hq, hkv)
+    assert api.vpp_last_launch_count() == 3
+    for s in range(max(u["split"] for u in units) + 1):
+        part = [u for u in units if u["split"] == s]
+        assert max(u["begin"] for u in part) - min(u["begin"] for u in part) <= chunk // 128 + 1
