@@ -381,13 +381,26 @@ RowPacking row_packing(const vpp_chunk_attn_args* a) {
     const int G = a->num_q_heads / a->num_kv_heads;
     RowPacking r{};
     // the largest part of a kv-head's group that fills at least 125 of the 128 rows (1 always does)
+    auto fills = [&](int d) { return G % d == 0 && d * (vpp::kTileM / d) >= 125; };
     r.group = 1;
     for (int d = 1; d <= vpp::kTileM && d <= G; ++d)
-        if (G % d == 0 && d * (vpp::kTileM / d) >= 125) r.group = d;
-    r.tile_tokens = vpp::kTileM / r.group;
+        if (fills(d)) r.group = d;
     // a packed item streams its K/V for these rows alone: the whole group if it fits a tile, however well it fills it
     r.short_group = G <= vpp::kTileM ? G : r.group;
     r.short_tokens = vpp::kTileM / r.short_group;
+    if (a->num_reqs == 1 && (G & (G - 1)) != 0) {
+        // One chunk, of a known length, in groups that are no power of two (whose units divide one another): a smaller part of the group where the largest leaves a tail that goes over all the keys for a
+        // few tokens.  512 tokens of groups of three are six units of 84 and eight tokens over, or, head by head, two units of
+        // 256: 512 tokens of 24/8 heads at 16384 keys 143 us and 101, 768 tokens of 48/8 at 65536 1650 and 1050.
+        auto visits = [&](int d) {    // tile visits per KV tile and kv-head
+            const int unit = 2 * (vpp::kTileM / d), rest = a->total_q % unit;
+            return (a->total_q / unit + (rest > r.short_tokens ? 1 : 0)) * 2.0 * (G / d) + (rest > 0 && rest <= r.short_tokens ? 2.0 : 0.0);
+        };
+        const int largest = r.group;
+        for (int d = largest - 1; d >= 1; --d)
+            if (fills(d) && visits(d) < 0.95 * visits(largest) && visits(d) < visits(r.group)) r.group = d;
+    }
+    r.tile_tokens = vpp::kTileM / r.group;
     r.unit_rows = 2 * r.tile_tokens;
     return r;
 }

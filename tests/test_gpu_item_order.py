@@ -82,3 +82,10 @@ def test_units_whose_keys_exceed_l2_are_cut_at_the_same_places(hq, hkv, chunk, s
     for s in range(max(u["split"] for u in units) + 1):
         part = [u for u in units if u["split"] == s]
         assert max(u["begin"] for u in part) - min(u["begin"] for u in part) <= chunk // 128 + 1
+
+
+@pytest.mark.parametrize("hq,hkv,chunk,rows", [(24, 8, 512, 256), (24, 8, 504, 84), (15, 5, 256, 256), (48, 8, 768, 128), (64, 8, 268, 32)])
+def test_tiles_of_a_chunk_whose_tail_would_go_over_all_keys_again(hq, hkv, chunk, rows):
+    """A part of the group of q-heads that divides the chunk better is taken where the largest leaves a few tokens over."""
+    _, units = _launch([4096 - chunk], [chunk], hq, hkv, splits=1)
+    assert max(u["rows"] for u in units) == rows

@@ -27,3 +27,11 @@ def test_units_of_very_different_length_in_one_launch():
     prob = W.make_problem(9600, [0, 3000, 700, 0], [900, 64, 1, 300], 8, 4, 128, 128, block_size=64, std=0.8)
     out, lse, _ = run_gpu(prob.to("cuda"), 1)
     print(compare(out, lse, prob, oracle.all_rows(prob.chunk_len.numpy(), 8), "ragged units"))
+
+
+@pytest.mark.parametrize("group,chunk", [(3, 256), (3, 512), (5, 256), (6, 768), (7, 512), (3, 341)])
+def test_one_chunk_in_parts_of_its_groups(group, chunk):
+    prob = W.make_problem(9650 + group, [500], [chunk], 2 * group, 2, 128, 128, block_size=64, std=0.8)
+    for splits in (0, 2):
+        out, lse, _ = run_gpu(prob.to("cuda"), splits)
+        print(compare(out, lse, prob, oracle.all_rows(prob.chunk_len.numpy(), 2 * group), "group %d, %d tokens, S=%d" % (group, chunk, splits)))
