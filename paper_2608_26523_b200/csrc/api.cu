@@ -312,65 +312,6 @@ struct ItemCounts {
     int unit_rows, unit_items, short_items, slots;
 };
 
-int uniform_splits(const vpp_chunk_attn_args* a, int heads_per_item) {
-    const int group = a->num_q_heads / a->num_kv_heads;
-    if (heads_per_item == 2 && a->total_q > 0 && a->total_q <= a->num_reqs && group <= vpp::kTileM) {
-        // A decode batch of the d = 128 family: one packed item per (token, kv-head), all about max_seq_len long.  Equal
-        // items fill the SMs in whole waves, so the split count is the one with the least idle last wave, charged with
-        // what splitting costs (measured: partials + merge ~5 %, ~1 % per extra split, ~4 us of start-up per unit
-        // against ~1.5 us per KV tile).
-        const double items = static_cast<double>(a->total_q) * a->num_kv_heads;
-        const double slots = sm_count_or_default();
-        const double tiles = a->max_seq_len / static_cast<double>(vpp::kTileN);
-        int best = 1;
-        double best_cost = 0.0;
-        for (int s = 1; s <= 4; ++s) {
-            if (s > 1 && tiles / s < 4.0) break;   // keep at least 4 KV tiles per split
-            const double waves = items * s / slots;
-            double cost = std::ceil(waves) / waves;
-            if (s > 1) cost *= 1.05 + 0.01 * s;
-            cost *= 1.0 + (s - 1) * 4.0 / (tiles * 1.5 + 1.0);
-            if (s == 1 || cost < best_cost) {
-                best = s;
-                best_cost = cost;
-            }
-        }
-        return best;
-    }
-    if (heads_per_item == 2 && a->num_reqs == 1) {
-        // One request of the d = 128 family: the work items (256 rows each) are about equally long, so
-        // they fill the SMs in waves here too.  Measured on 8192-token chunks at 64K-128K prefixes: 512 items (3.46
-        // waves) gain 7-9 % from two splits, 256 items 1.5 % from four, 128 and 1024 items are best unsplit.
-        const double items = static_cast<double>((a->total_q + vpp::kTileM - 1) / vpp::kTileM) * (a->num_q_heads / 2);
-        const double slots = sm_count_or_default();
-        const double tiles = a->max_seq_len / static_cast<double>(vpp::kTileN);
-        int best = 1;
-        double best_cost = 0.0;
-        for (int s = 1; s <= 8 && items > 0; ++s) {
-            if (s > 1 && tiles / s < 4.0) break;   // keep at least 4 KV tiles per split
-            const double waves = items * s / slots;
-            double cost = std::ceil(waves) / waves;
-            if (s > 1) cost *= 1.045 + 0.01 * (s - 1);                 // partials + merge
-            cost *= 1.0 + (s - 1) * 4.0 / (tiles * 2.0 + 1.0);        // ~4 us of start-up per unit, ~2 us per KV tile
-            if (s == 1 || cost < best_cost) {
-                best = s;
-                best_cost = cost;
-            }
-        }
-        return best;
-    }
-    const long long tiles = (a->total_q + vpp::kTileM - 1) / vpp::kTileM + a->num_reqs;
-    const long long items = tiles * (a->num_q_heads / heads_per_item);
-    const int sms = sm_count_or_default();
-    if (items >= 2ll * sms || items == 0) return 1;
-    long long s = (2ll * sms + items - 1) / items;
-    const long long by_len = (a->max_seq_len / vpp::kTileN) / 4;  // keep at least 4 KV tiles per split
-    if (s > by_len) s = by_len;
-    if (s > 16) s = 16;
-    if (s < 1) s = 1;
-    return static_cast<int>(s);
-}
-
 // How the d = 128 kernel packs (token, q-head) pairs into the rows of a tile (attn_ws.cuh).
 struct RowPacking {
     int group, tile_tokens;         // items of two tiles: q-heads x tokens of a tile
@@ -407,14 +348,8 @@ RowPacking row_packing(const vpp_chunk_attn_args* a) {
 // Query rows of a work unit.
 int unit_rows_of(const vpp_chunk_attn_args* a, Family fam) { return fam == Family::kGqa128 ? row_packing(a).unit_rows : vpp::kTileM; }
 
-// (the split choice below counts work items of 256 rows: two 128-row tiles)
-bool even_groups(const vpp_chunk_attn_args* a) { return (a->num_q_heads / a->num_kv_heads) % 2 == 0; }
 // The absorbed-MLA kernel runs on pairs of SMs (2-CTA clusters).
 bool mla_kernel_available() { return sm_count_or_default() >= 2; }
-int heads_per_item(const vpp_chunk_attn_args* a, Family fam) {
-    if (fam == Family::kMla576) return 1;
-    return even_groups(a) ? 2 : 1;
-}
 
 ItemCounts item_counts(const vpp_chunk_attn_args* a, Family fam) {
     const int sms = sm_count_or_default();
@@ -458,10 +393,30 @@ int ranges_of(int slots, int items) {
     return best;
 }
 
+// Equal splits of a batch of decode rows that fills the SMs (80 % of them or more): as many as leave the least idle last wave,
+// charged with what splitting costs (measured: partials + merge ~5 %, ~1 % per extra split, ~4 us of start-up per unit against
+// ~1.5 us per KV tile when all SMs stream).
+int decode_splits(long long items, int slots, double tiles) {
+    int best = 1;
+    double best_cost = 0.0;
+    for (int s = 1; s <= 4; ++s) {
+        if (s > 1 && tiles / s < 4.0) break;   // keep at least 4 KV tiles per split
+        const double waves = static_cast<double>(items) * s / slots;
+        double cost = std::ceil(waves) / waves;
+        if (s > 1) cost *= 1.05 + 0.01 * s;
+        cost *= 1.0 + (s - 1) * 4.0 / (tiles * 1.5 + 1.0);
+        if (s == 1 || cost < best_cost) {
+            best = s;
+            best_cost = cost;
+        }
+    }
+    return best;
+}
+
 // Equal splits of one request's chunk, and the time they take: waves of items, the last of them as idle as the items are equally long
 // (a chunk that is half the context or more has items of all lengths, which go longest first), and the partial results (whose
 // stores mostly hide behind the items).  Measured on 8192-token chunks at 64K-128K prefixes: 512 items (3.46 waves) gain 7-9 % from two splits, 256 items 1.5 % from
-// four, 128 and 1024 items are best unsplit.
+// four, 128 and 1024 items are best unsplit; 4096 tokens of 32/32 heads without a prefix (512 items) 131 us unsplit, 215 in two.
 int chunk_splits(long long items, int slots, double tiles, double chunk_tiles, double unit_us, double parts_us, int most, double* us) {
     const double mean = tiles - 0.5 * chunk_tiles, equal = chunk_tiles < 0.5 * tiles ? 1.0 - chunk_tiles / tiles : 0.0;
     int best = 1;
@@ -527,8 +482,13 @@ SplitPlan plan_splits(const vpp_chunk_attn_args* a, Family fam, int most = vpp::
         if (s > most) s = most;
         return s < 2 ? SplitPlan{1, false} : SplitPlan{static_cast<int>(s), true};
     }
-    if (mla) return {1, false};
-    return {uniform_splits(a, heads_per_item(a, fam)), false};
+    if (mla || !(decode || one_request)) return {1, false};   // (others have two items a slot or more here, of different lengths)
+    if (decode) return {decode_splits(items, c.slots, a->max_seq_len / static_cast<double>(vpp::kTileN)), false};
+    // (a last unit whose rows fit one tile runs packed)
+    const int rest = a->total_q % c.unit_rows;
+    const long long tail = rest > 0 && rest <= row_packing(a).short_tokens ? c.short_items - c.unit_items : 0;
+    double equal_us = 0;
+    return {chunk_splits(items + tail, c.slots, tiles, chunk_tiles, tile_times(a, fam).unit_us, parts_us, most, &equal_us), false};
 }
 
 using MergeKernel = void (*)(const float*, const float*, int, long long, int, int, const int32_t*, const vpp::WorkHeader*, __nv_bfloat16*,

@@ -35,3 +35,21 @@ def test_cutting_is_chosen_where_it_pays(total_q, num_reqs, hq, hkv, seq, mla, c
         pytest.skip("the expectations are for 148 SMs")
     auto, uncut = (_workspace(total_q, num_reqs, hq, hkv, seq, s, mla) for s in (0, 1))
     assert (auto > uncut) == cut
+
+
+@pytest.mark.parametrize("total_q,hq,hkv,seq,cut", [
+    (1280, 32, 32, 32768, True), (1280, 32, 16, 32768, True),     # 160 items either way: twelve would run a second wave alone
+    (4096, 32, 32, 4096, False), (4096, 32, 16, 4096, False),     # items of all lengths: longest first fills the last wave
+    (8192, 16, 2, 73728, True), (8192, 64, 4, 73728, False)])     # 3.5 and 14 waves of equally long items
+def test_equal_splits_go_by_the_items_that_run(total_q, hq, hkv, seq, cut):
+    if torch.cuda.is_available() and torch.cuda.get_device_properties(0).multi_processor_count != 148:
+        pytest.skip("the expectations are for 148 SMs")
+    auto, uncut = (_workspace(total_q, 1, hq, hkv, seq, s) for s in (0, 1))
+    assert (auto > uncut) == cut
+
+
+@pytest.mark.parametrize("rows,heads", [(5, (32, 32)), (20, (24, 8)), (8, (40, 40))])
+def test_decode_rows_of_odd_groups_are_cut_like_those_of_even_ones(rows, heads):
+    hq, hkv = heads
+    one = lambda q: _workspace(rows, rows, q, hkv, 16384, 0) - _workspace(rows, rows, q, hkv, 16384, 1)
+    assert one(2 * hkv) / (2 * hkv) == pytest.approx(one(hq) / hq, rel=0.02)
