@@ -367,14 +367,19 @@ constexpr int kLead = 2, kShortLead = 3, kMlaLead = 5;
 constexpr double kL2Keeps = 96e6;   // bytes of keys and values that stay in the 126 MB of L2 while a launch goes over them
 constexpr int kMinLen = 2, kMinShortLen = 4;   // fewest KV tiles worth a work item (start-up ~4 us, ~2 / ~1 us per tile)
 
-// Time of a KV tile of a work item, measured at full clock.  (Packed items have a producer warp for V of their own in decode
-// batches only.)
+// Does the d = 128 kernel run with a second producer warp, for the V tiles?  Where most of the work is packed items, which are bound by the
+// arrival of K/V: batches of requests of 64 tokens or fewer on average.  64/8 heads, without it and with it: 30 decode rows at 4000 to
+// 4400 keys and 64 tokens at 8000 155 and 130 us, 200 rows and 1000 tokens 1046 and 916, 32 requests of 4 tokens 165 and 144; the
+// other way round 60 rows and 4000 tokens 1351 and 1384, a chunk by itself 1 to 2 %.
+bool v_producer(const vpp_chunk_attn_args* a) { return a->total_q <= (a->num_reqs > 1 ? 64ll * a->num_reqs : 1); }
+
+// Time of a KV tile of a work item, measured at full clock.
 struct TileTimes {
     double unit_us, short_us;
 };
 TileTimes tile_times(const vpp_chunk_attn_args* a, Family fam) {
     if (fam == Family::kMla576) return {1.6, 1.6};
-    return {1.75, a->total_q <= a->num_reqs ? 0.85 : 1.3};
+    return {1.75, v_producer(a) ? 0.85 : 1.3};
 }
 
 // Ranges of a balanced cut when every unit has `items` work items: as many as fill the slots in one round, or in up to four where
@@ -798,8 +803,7 @@ vpp_status run_chunk_attn(const vpp_chunk_attn_args* a, vpp_stream_t stream_, co
     } else {
         // a second producer warp for launches bound by the arrival of K/V: batches of decode rows.  (Prefill loses 1 to 2 % with it,
         // over pages of any size: 2048 tokens of 64 heads at prefix 16385 1003 us with it, 989 without.)
-        const bool v_warp = a->total_q <= a->num_reqs;
-        auto kern = v_warp ? vpp::attn128_ws_kernel<true> : vpp::attn128_ws_kernel<false>;
+        auto kern = v_producer(a) ? vpp::attn128_ws_kernel<true> : vpp::attn128_ws_kernel<false>;
         ce = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, vpp::kWsSmemBytes);
         if (ce == cudaSuccess)
             ce = launch(kern, static_cast<unsigned>(sms), vpp::kWsThreads, vpp::kWsSmemBytes, stream, tm_q, tm_qs, tm_q1, tm_k, tm_v, tm_kx,
