@@ -330,3 +330,13 @@ def test_cost_curve_fit_and_balance_identity_of_the_benchmark():
     assert bench.fit_cost_curve([0, 100], [1.0, 2.0]) is None
     rec = bench.read_traffic_record("attn128_ws_cfg2_traffic.txt")
     assert rec["prefix"] == "131072" and float(rec["dram_bytes_read"]) > 0 and rec["kernel"] == "attn128_ws_kernel"
+
+
+def test_the_current_stream_without_torchs_private_names(monkeypatch):
+    """torch's raw stream handle is not part of its public interface: where it is missing, the public call is used."""
+    class Stream:
+        cuda_stream = 0x5150
+
+    monkeypatch.setattr(api, "_raw_stream", None)
+    monkeypatch.setattr(torch.cuda, "current_stream", Stream)
+    assert api._current_stream() == 0x5150
