@@ -206,8 +206,8 @@ vpp_status vpp_chunk_attn_partial_fwd(const vpp_chunk_attn_args *args, int32_t k
  *    with VPP_ERR_WORKSPACE and nothing is enqueued; vpp_static_last_error() says how much was needed.
  *    (Split-KV partials dominate: 4 * num_kv_splits * total_q * num_q_heads * (head_dim_v + 1) bytes.)
  *  - All calls on a device share the one array, and it keeps whatever the previous call left there.
- *    Nothing in it has to start at zero -- the work-decomposition kernel rewrites the header, the work
- *    list and the per-row split counts of each launch before they are read -- but two calls that
+ *    Nothing in it has to start at zero -- the work-decomposition kernel rewrites the header and the work
+ *    list of each launch, the attention kernel the per-row split counts, before they are read -- but two calls that
  *    overlap on the GPU (different streams, or graphs replayed concurrently) race on it.  Serialise them.
  *  - Other errors and the meaning of *status are those of vpp_chunk_attn_fwd.
  */
@@ -343,8 +343,9 @@ const char *vpp_host_last_error(void);
  * total_q, max_seq_len, softmax_scale: as in vpp_chunk_attn_args.
  * out          bf16 [total_q, num_q_heads, 512]; lse float [total_q, num_q_heads] or NULL.
  * workspace    device memory of vpp_sparse_attn_workspace_size(total_q) bytes, 16-byte aligned; owned by the
- *              caller, contents irrelevant on entry.  With few tokens it holds partial results too (their lists are cut into parts, merged by a third kernel); a workspace that holds
- *              256 + 8 total_q bytes only is accepted and the launch runs uncut.
+ *              caller, contents irrelevant on entry.  With few tokens it holds partial results too (their lists
+ *              are cut into parts, merged by a third kernel); a workspace that holds 256 + 8 total_q bytes only
+ *              is accepted and the launch runs uncut.
  * status       optional device int32, zeroed by the call; VPP_DEV_BAD_LENGTHS (nothing is written),
  *              VPP_DEV_BAD_BLOCK (a needed block_table entry outside [0, num_blocks): results undefined but no
  *              access leaves the cache) or VPP_DEV_TIMEOUT as in vpp_chunk_attn_fwd.

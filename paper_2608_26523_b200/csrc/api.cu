@@ -110,7 +110,7 @@ EncodeFn get_encode() {
 }
 
 // Encoded tensor maps are cached: a serving loop calls with the same buffers and shapes again and again, and seven
-// to nine driver encodes per call are a visible part of a short launch.  A map depends only on (base address, rank,
+// (d = 128) or four (MLA) driver encodes per call are a visible part of a short launch.  A map depends only on (base address, rank,
 // extents, strides, box), so an entry never goes stale; the cache is a small 4-way set-associative table (least recently
 // used way replaced) guarded by a mutex.
 struct TmapKey {
@@ -124,7 +124,7 @@ using RawEncodeFn = bool (*)(CUtensorMap*, const TmapKey&);
 
 class TmapCache {
 public:
-    static constexpr int kSets = 64, kWays = 4;   // a call uses up to nine maps; 256 entries serve a few dozen distinct launches
+    static constexpr int kSets = 64, kWays = 4;   // a call uses up to seven maps; 256 entries serve a few dozen distinct launches
     bool get(const TmapKey& key, RawEncodeFn encode, CUtensorMap* out) {
         const uint64_t h = hash(key);
         Slot* set = slots_ + (h % kSets) * kWays;
@@ -801,8 +801,6 @@ vpp_status run_chunk_attn(const vpp_chunk_attn_args* a, vpp_stream_t stream_, co
             ce = launch(kern, static_cast<unsigned>((sms / 2) * 2), vpp::kMla2Threads, vpp::kMla2SmemBytes, stream, tm_q9, tm_qh9, tm_k93,
                         tm_k92, ap, box_rows);
     } else {
-        // a second producer warp for launches bound by the arrival of K/V: batches of decode rows.  (Prefill loses 1 to 2 % with it,
-        // over pages of any size: 2048 tokens of 64 heads at prefix 16385 1003 us with it, 989 without.)
         auto kern = v_producer(a) ? vpp::attn128_ws_kernel<true> : vpp::attn128_ws_kernel<false>;
         ce = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, vpp::kWsSmemBytes);
         if (ce == cudaSuccess)

@@ -56,7 +56,7 @@ constexpr int kMla2SmemBytes = kMla2QBytes + kMla2KBytes + kMla2VBytes + kMla2PB
 // K and V in shared memory.  Pages of 64 tokens and more: slabs of 64 features, 8 KB apart.  Smaller pages (kSmallPages): 8-key
 // groups, in each the slabs of the hand-back group (K: three) or chunk (V: two) side by side, 1 KB of eight keys apiece -- the keys of
 // a page are consecutive then, so a group's or chunk's share of a page is ONE copy instead of one per slab (512 tokens at prefix
-// 8195, 128 heads: pages of 16 1176 -> 991 us, of 32 965 -> 918).  Pages of 64 keep the slabs: one copy either way, and the
+// 8195, 128 heads: pages of 16 1176 -> 943 us, of 32 965 -> 907).  Pages of 64 keep the slabs: one copy either way, and the
 // MMAs read K groups of 3 KB 9 % slower (887 against 977 us).
 template <bool kSmallPages>
 struct MlaLayout {

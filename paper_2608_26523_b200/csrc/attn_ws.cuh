@@ -450,7 +450,7 @@ attn128_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                 if (!wait1(bar_q_full, q_it & 1, 302)) break;
                 ++q_it;
                 if (packed) {
-                    // Packed single-token item: both tiles hold the same Q (the heads of one kv-head) and share the KV
+                    // Packed item (a short unit): both tiles use the same Q (the unit's tokens x the heads of one kv-head) and share the KV
                     // range -- tile t takes the KV tiles kv_begin + t, + t + 2, ... as an independent online softmax
                     // (its own S_t, O_t); the two partial results are merged by softmax group 0 at the end.
                     // Ring index of K(jj) is base + 2 jj, of V(jj) base + 2 jj + 1.
@@ -587,7 +587,7 @@ attn128_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
             if (!valid) break;
             // the first part and head of a unit says how many partial results its rows have
             if (p.row_splits && u.split <= 0 && ring_h0 == 0 && row < tile_rows && row % grp == 0 && !(packed && t == 1)) p.row_splits[u.q_row0 + tok] = n_splits;
-            // One item's softmax work.  The packed variant (single-token items) is compiled separately so that the
+            // One item's softmax work.  The packed variant (short units) is compiled separately so that the
             // prefill path keeps the registers and the instruction count it had without it.
             auto run_item = [&](auto packed_tag) -> bool {
             constexpr bool kPacked = decltype(packed_tag)::value;

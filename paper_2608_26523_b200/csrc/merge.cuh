@@ -119,7 +119,7 @@ lse_merge_kernel(const float* __restrict__ o_parts, const float* __restrict__ ls
     }
 }
 
-// The same merge for at most kSMax (<= 8) partials, the case every launch of this library produces: one thread per
+// The same merge for at most kSMax (<= 8) partials: one thread per
 // 16-byte piece of an output row (consecutive threads take consecutive pieces, so a warp reads whole 512-byte runs of
 // every partial), kPieces pieces per trip.  Each thread reads the few log-sum-exp values of its row itself (the lanes
 // of a warp mostly share a row: one broadcast transaction) and forms the weights in registers -- no shuffles, no
