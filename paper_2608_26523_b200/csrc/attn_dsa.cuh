@@ -13,7 +13,7 @@
 // unevenly (setmaxnreg) to make room for them.  2048 tokens with lists of
 // 2048 at prefix 65536: 10 producer warps of 24 and 32 lanes 1458 us, these 1362 us.
 // A launch of few tokens (a decode batch) would leave most pairs idle for the 16 tiles of a 2048-entry list: then a token's
-// list is cut into `splits` parts, an item each, whose partial results lse_merge_small_kernel joins (16 tokens: 62.6 -> 38.2 us for the step).
+// list is cut into `splits` parts, an item each, whose partial results lse_merge_small_kernel joins (16 tokens: 62.6 -> 38.2 us for the step, 36.8 -> 35.4 with a shorter store of the partial results).
 // Entries that do not take part are pointed at the token's own cache row (always present and finite) and masked out
 // of the softmax through a 128-bit validity mask that warp 0 publishes per tile.  The cost per token does not depend on
 // the prefix length: the flat latency curve the paper says weakens its linear-growth assumption.
@@ -288,11 +288,12 @@ dsa_attn_kernel(const __grid_constant__ CUtensorMap tm_qh, const __grid_constant
         for (int item = pair; item < num_items && ok; item += num_pairs) {
             int t, j0, j1;
             part_of(item, t, j0, j1);
+            int e_next[4];
+            if (kParts) load_entries(t, j0, key0, e_next);   // (beside the token's look-up; longer items have time for it after: 2048 tokens are 2 % slower so)
             const int2 tk = __ldg(p.tok + t);
             if (tk.x < 0) continue;
             const int self_row = row_of(tk.x, tk.y);
-            int e_next[4];
-            load_entries(t, j0, key0, e_next);
+            if (!kParts) load_entries(t, j0, key0, e_next);
             if (kw == kDsaKWarps - 1 && lane == 0) {
                 // This warp loads Q too: it may be replaced once the scores of the previous item's last tile are done, which is
                 // what the last group waits for.  (A warp that runs further ahead, as the one of the masks does, must not wait
@@ -336,11 +337,12 @@ dsa_attn_kernel(const __grid_constant__ CUtensorMap tm_qh, const __grid_constant
         for (int item = pair; item < num_items && ok; item += num_pairs) {
             int t, j0, j1;
             part_of(item, t, j0, j1);
+            int e_next[4];
+            if (kParts) load_entries(t, j0, key0, e_next);   // (beside the token's look-up; longer items have time for it after: 2048 tokens are 2 % slower so)
             const int2 tk = __ldg(p.tok + t);
             if (tk.x < 0) continue;
             const int self_row = row_of(tk.x, tk.y);
-            int e_next[4];
-            load_entries(t, j0, key0, e_next);
+            if (!kParts) load_entries(t, j0, key0, e_next);
             for (int j = j0; j < j1 && ok; ++j) {
                 int e[4], r[4];
 #pragma unroll
@@ -502,11 +504,12 @@ dsa_attn_kernel(const __grid_constant__ CUtensorMap tm_qh, const __grid_constant
                 }
                 float mx[8];
 #pragma unroll
-                for (int k = 0; k < 8; ++k) mx[k] = __uint_as_float(s[k]);
+                for (int i = 0; i < 64; i += 16)
 #pragma unroll
-                for (int i = 8; i < 64; i += 8)
-#pragma unroll
-                    for (int k = 0; k < 8; ++k) mx[k] = fmaxf(mx[k], __uint_as_float(s[i + k]));
+                    for (int k = 0; k < 8; ++k) {
+                        const float v0 = __uint_as_float(s[i + k]), v1 = __uint_as_float(s[i + 8 + k]);
+                        mx[k] = i == 0 ? fmaxf(v0, v1) : fmax3(mx[k], v0, v1);
+                    }
                 const float mxa = fmaxf(fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])),
                                         fmaxf(fmaxf(mx[4], mx[5]), fmaxf(mx[6], mx[7])));
                 float mxb;
@@ -540,11 +543,14 @@ dsa_attn_kernel(const __grid_constant__ CUtensorMap tm_qh, const __grid_constant
                 }
                 const float m_use = (m_ref == -INFINITY) ? 0.f : m_ref;
                 uint32_t pk[32];
+                // (packed fma and three-input maxima: the softmax shares its issue slots with 17 warps of producers; 2048 tokens 1353 -> 1340 us)
+                const uint64_t sc2 = pack_f32x2(sc, sc), neg_m2 = pack_f32x2(-m_use, -m_use);
                 float sum0 = 0.f, sum1 = 0.f;
 #pragma unroll
                 for (int i = 0; i < 64; i += 2) {
-                    const float p0 = ex2(fmaf(__uint_as_float(s[i]), sc, -m_use));
-                    const float p1 = ex2(fmaf(__uint_as_float(s[i + 1]), sc, -m_use));
+                    float x0, x1;
+                    unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(s[i]), __uint_as_float(s[i + 1])), sc2, neg_m2), x0, x1);
+                    const float p0 = ex2(x0), p1 = ex2(x1);
                     sum0 += p0;
                     sum1 += p1;
                     pk[i >> 1] = pack_bf16x2(p0, p1);
@@ -581,8 +587,7 @@ dsa_attn_kernel(const __grid_constant__ CUtensorMap tm_qh, const __grid_constant
             const bool live = h < p.num_q_heads;
             // row of out / lse, or of the partials (part, token, q-head)
             const long long out_row = (kParts ? static_cast<long long>(item - t * p.splits) * p.total_q + t : t) * p.num_q_heads + h;
-            constexpr int row_step = 1;                           // the warp's 32 rows: consecutive q-heads
-            const int warp_rows = p.num_q_heads - (h - lane);
+            const int warp_rows = p.num_q_heads - (h - lane);     // the warp's 32 rows: consecutive q-heads
             const long long first_row = out_row - lane;
             // (P V of the last tile is done, so the warp's own rows of P serve as the stage of its stores)
             uint8_t* const stage = p_row - lane * 128;
@@ -604,25 +609,27 @@ dsa_attn_kernel(const __grid_constant__ CUtensorMap tm_qh, const __grid_constant
                         }
                     }
                     stage_flush(stage, lane, 32, [&](int i) -> uint8_t* {
-                        return i < warp_rows ? static_cast<uint8_t*>(p.out) + ((first_row + i * row_step) * kMlaDv + (k >> 1) * 256 + half * 128 + (k & 1) * 64) * 2
+                        return i < warp_rows ? static_cast<uint8_t*>(p.out) + ((first_row + i) * kMlaDv + (k >> 1) * 256 + half * 128 + (k & 1) * 64) * 2
                                              : nullptr;
                     });
                 }
             } else {
+                // (the next columns come from tensor memory while the stage is emptied)
+                const StageRows to = stage_rows(lane, [&](int i) -> uint8_t* {
+                    return i < warp_rows ? reinterpret_cast<uint8_t*>(p.o_parts + (first_row + i) * kMlaDv + half * 128) : nullptr;
+                });
+                uint32_t r[32];
+                tmem_ld32(tO0, r);
 #pragma unroll 1
                 for (int c = 0; c < 8; ++c) {     // 32 fp32 columns of 32 rows
-                    uint32_t r[32];
-                    tmem_ld32((c < 4 ? tO0 : tO1) + (c & 3) * 32, r);
                     tc_wait_ld();
 #pragma unroll
                     for (int q4 = 0; q4 < 8; ++q4)
                         stage_put(stage, lane, q4,
                                   make_uint4(__float_as_uint(__uint_as_float(r[q4 * 4]) * inv_l), __float_as_uint(__uint_as_float(r[q4 * 4 + 1]) * inv_l),
                                              __float_as_uint(__uint_as_float(r[q4 * 4 + 2]) * inv_l), __float_as_uint(__uint_as_float(r[q4 * 4 + 3]) * inv_l)));
-                    stage_flush(stage, lane, 32, [&](int i) -> uint8_t* {
-                        return i < warp_rows ? reinterpret_cast<uint8_t*>(p.o_parts + (first_row + i * row_step) * kMlaDv + (c >> 2) * 256 + half * 128 + (c & 3) * 32)
-                                             : nullptr;
-                    });
+                    if (c < 7) tmem_ld32((c < 3 ? tO0 : tO1) + ((c + 1) & 3) * 32, r);
+                    stage_flush(stage, lane, to, (c >> 2) * 1024 + (c & 3) * 128);
                 }
             }
             if (live && half == 0) {
