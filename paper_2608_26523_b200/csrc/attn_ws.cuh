@@ -48,6 +48,9 @@ static_assert(kWsStages <= 4, "V-tail barrier slots");
 constexpr int kWsStageBytes = 8 * 32 * 128;   // 4 KB per softmax warp for the epilogue's stores
 constexpr int kWsSmemBytes = 2 * kTileBytes + kWsStages * kTileBytes + 1024 /*align*/ + 2048 /*barriers, ring, merge exchange*/ + kWsStageBytes;
 static_assert(kWsSmemBytes <= 232448, "shared memory of one CTA");
+// (bytes from the first barrier)
+constexpr int kWsBarS = 48, kWsBarP = 64, kWsBarO = 80, kWsBarJoin = 104, kWsBarX1 = 128 + 16 * kWsStages, kWsBarX0 = kWsBarX1 + 8, kWsBarPart = 208;
+constexpr int kWsAbort = 512, kWsXm = 1024, kWsStage = 2048;
 constexpr float kRescaleThreshold = 8.f;      // log2 units
 // Early hand-overs of P: bit c set = the key columns up to 32 (c + 1) are handed to the MMA thread as soon as they are in
 // tensor memory, so that O += P V starts on them while the rest of the exponentials are computed (0: P is handed over whole).
@@ -119,6 +122,174 @@ __device__ __noinline__ void ws_packed_merge(void* out, float* lse_out, float* o
     }
 }
 
+// Whole items of one token and up to kQuarterHeads q-heads (decode rows that are not cut): the item's rows stand in Q four times, once in the 32 lanes of
+// each softmax warp, and the warps share out the 128 keys of a tile -- 32 each, an online softmax of its own, the P of the others' keys
+// zero -- where one warp would take them all and the others idle.  Tile t's O is then the sum of four over the lanes, and an item's
+// result the sum of eight, joined by group 0: every warp weighs its two and leaves them in the stage, all sum.
+// A tile's softmax is a third as long, so that what ends an item hides behind the copies of the next: 256 decode rows of 64/8 heads, contexts to
+// 8192 tokens, 578 -> 567 us.  What bounds it is the memory (6 TB/s while tiles stream).
+constexpr int kQuarterHeads = 16;             // rows of 512 bytes in a warp's 8 KB of the stage
+static_assert(4 * kQuarterHeads * 512 <= kWsStageBytes, "the stage of both groups");
+// dst: row of the item's first head; lse: its log-sum-exp, or null; area: the CTA's barriers, xm and stage
+__device__ __forceinline__ bool ws_quarter_join(uint8_t* dst, float* lse, bool second, uint8_t* area, uint32_t bar, uint32_t tO,
+                                                int heads, float m_ref, float l_run) {
+    volatile int* const s_abort = reinterpret_cast<volatile int*>(area + kWsAbort);
+    float* const xm = reinterpret_cast<float*>(area + kWsXm);
+    uint8_t* const stage = area + kWsStage;
+    const int row = threadIdx.x & 127, w = row >> 5, lane = row & 31;
+    const float m1 = xm[row], l1 = xm[128 + row];
+    const float m = fmaxf(m_ref, m1);
+    const float a0 = m_ref == -INFINITY ? 0.f : ex2(m_ref - m), a1 = m1 == -INFINITY ? 0.f : ex2(m1 - m);
+    xm[row] = m;              // (read by this thread alone so far)
+    xm[128 + row] = a0 * l_run + a1 * l1;
+    __syncwarp();
+    if (lane == 0) mbar_arrive(bar);
+    if (!mbar_wait(bar, 0, s_abort, 406)) return false;      // (two phases an item: the same parities every time)
+    float M = -INFINITY, L = 0.f;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) M = fmaxf(M, xm[k * 32 + lane]);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const float mk = xm[k * 32 + lane];
+        if (mk != -INFINITY) L = fmaf(ex2(mk - M), xm[128 + k * 32 + lane], L);
+    }
+    const float f = m == -INFINITY ? 0.f : ex2(m - M) / L;
+    const float s0 = a0 * f, s1 = a1 * f;
+    uint8_t* const mine = stage + w * (kQuarterHeads * 512) + lane * 512;
+#pragma unroll 1
+    for (int c = 0; c < 8; ++c) {     // 16 output columns at a time (registers)
+        uint32_t r[16], r1[16];
+        tmem_ld16(tO + c * 16, r);
+        if (second) tmem_ld16(tO + 128 + c * 16, r1);
+        tc_wait_ld();
+        if (lane < heads) {
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+                float v = __uint_as_float(r[i]) * s0;
+                if (second) v = fmaf(__uint_as_float(r1[i]), s1, v);
+                r[i] = __float_as_uint(v);
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                *reinterpret_cast<uint4*>(mine + (((c * 4 + q) ^ (lane & 7)) << 4)) = make_uint4(r[4 * q], r[4 * q + 1], r[4 * q + 2], r[4 * q + 3]);
+        }
+    }
+    if (lane < heads && w == 0 && lse) lse[lane] = (M + log2f(L)) * 0.6931471805599453f;
+    __syncwarp();
+    if (lane == 0) mbar_arrive(bar);
+    if (!mbar_wait(bar, 1, s_abort, 407)) return false;
+    for (int i = row; i < heads * 16; i += 128) {     // eight columns of a row
+        const int h = i >> 4, c8 = i & 15;
+        float acc[8] = {};
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const uint8_t* const from = stage + k * (kQuarterHeads * 512) + h * 512;
+            const float4 x = *reinterpret_cast<const float4*>(from + (((2 * c8) ^ (h & 7)) << 4));
+            const float4 y = *reinterpret_cast<const float4*>(from + (((2 * c8 + 1) ^ (h & 7)) << 4));
+            acc[0] += x.x; acc[1] += x.y; acc[2] += x.z; acc[3] += x.w;
+            acc[4] += y.x; acc[5] += y.y; acc[6] += y.z; acc[7] += y.w;
+        }
+        *reinterpret_cast<uint4*>(dst + (h * 128 + c8 * 8) * 2) =
+            make_uint4(pack_bf16x2(acc[0], acc[1]), pack_bf16x2(acc[2], acc[3]), pack_bf16x2(acc[4], acc[5]), pack_bf16x2(acc[6], acc[7]));
+    }
+    return true;
+}
+
+// Softmax of one item of quarters, by a warp of group t: 32 of the keys of every second tile, then the join.
+// (out of line, like the join of packed items: the prefill path keeps its registers)
+__device__ __noinline__ bool ws_run_quarters(uint8_t* dst, float* lse, int kv_end, int pos, int heads, float sc, uint32_t sBar,
+                                             uint8_t* area, uint32_t tmem_base, uint32_t s_it, uint32_t o_it, uint32_t x_it) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, t = (warp - 4) >> 2, wq = warp & 3, row = threadIdx.x & 127;
+    const uint32_t lane_off = static_cast<uint32_t>(wq * 32) << 16, tS = tmem_base + t * 128 + lane_off, tO = tmem_base + 256 + t * 128 + lane_off;
+    volatile int* const s_abort = reinterpret_cast<volatile int*>(area + kWsAbort);
+    float* const xm = reinterpret_cast<float*>(area + kWsXm);
+    float m_ref = -INFINITY, l_run = 0.f;
+    const int first = t;                      // (a whole row begins at its first tile)
+#pragma unroll 1
+    for (int j = first; j < kv_end; j += 2) {
+        if (!mbar_wait(sBar + kWsBarS + 8 * t, s_it & 1, s_abort, 402)) return false;
+        ++s_it;
+        tc_fence_after();
+        uint32_t s[32];
+        tmem_ld32(tS + 32 * wq, s);
+        tc_wait_ld();
+        const int lim = pos - j * kTileN - 32 * wq;      // columns <= lim are visible
+        if (lim < 31) {
+#pragma unroll
+            for (int i = 0; i < 32; ++i)
+                if (i > lim) s[i] = 0xff800000u;  // -inf
+        }
+        float mx[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) mx[k] = fmaxf(__uint_as_float(s[k]), __uint_as_float(s[4 + k]));
+#pragma unroll
+        for (int i = 8; i < 32; i += 8)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) mx[k] = fmax3(mx[k], __uint_as_float(s[i + k]), __uint_as_float(s[i + 4 + k]));
+        const float m_new = fmaxf(fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * sc, m_ref);
+        // (lanes beyond the heads hold leftovers: they never ask for a rescale)
+        const bool grow = lane < heads && ((m_new - m_ref > kRescaleThreshold) || (m_ref == -INFINITY && m_new != -INFINITY));
+        if (__any_sync(0xffffffffu, grow)) {
+            const float alpha = grow ? ex2(m_ref - m_new) : 1.f;  // m_ref = -inf gives 0
+            if (grow) m_ref = m_new;
+            l_run *= alpha;
+            if (j > first) {   // O of this tile already holds something
+                uint32_t o[16];
+#pragma unroll 1
+                for (int c = 0; c < 8; ++c) {
+                    tmem_ld16(tO + c * 16, o);
+                    tc_wait_ld();
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * alpha);
+                    tmem_st16(tO + c * 16, o);
+                }
+            }
+        }
+        const float m_use = (m_ref == -INFINITY) ? 0.f : m_ref;
+        float sum0 = 0.f, sum1 = 0.f;
+        uint32_t pk[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) pk[i] = 0;
+#pragma unroll
+        for (int k = 1; k < 4; ++k) tmem_st16(tS + ((wq + k) & 3) * 16, pk);
+#pragma unroll
+        for (int i = 0; i < 32; i += 2) {
+            const float p0 = ex2(fmaf(__uint_as_float(s[i]), sc, -m_use)), p1 = ex2(fmaf(__uint_as_float(s[i + 1]), sc, -m_use));
+            sum0 += p0;
+            sum1 += p1;
+            pk[i >> 1] = pack_bf16x2(p0, p1);
+        }
+        tmem_st16(tS + wq * 16, pk);
+        l_run += sum0 + sum1;
+        tc_wait_st();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) {
+#pragma unroll
+            for (int c = 0; c < 3; ++c)
+                if ((kPartMask >> c) & 1) mbar_arrive(sBar + kWsBarPart + 16 * c + 8 * t);
+            mbar_arrive(sBar + kWsBarP + 8 * t);
+        }
+    }
+    if (first < kv_end && !mbar_wait(sBar + kWsBarO + 8 * t, o_it & 1, s_abort, 403)) return false;   // (tile 1 of a one-tile item has none)
+    tc_fence_after();
+    if (t == 1) {
+        xm[row] = m_ref;
+        xm[128 + row] = l_run;
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(sBar + kWsBarX1);
+        return mbar_wait(sBar + kWsBarX0, x_it & 1, s_abort, 404);
+    }
+    if (!mbar_wait(sBar + kWsBarX1, x_it & 1, s_abort, 405)) return false;
+    tc_fence_after();
+    if (!ws_quarter_join(dst, lse, 1 < kv_end, area, sBar + kWsBarJoin, tO, heads, m_ref, l_run)) return false;
+    tc_fence_before();
+    __syncwarp();
+    if (lane == 0) mbar_arrive(sBar + kWsBarX0);
+    return true;
+}
+
 // K / V tile in shared memory: 8-key groups of 2 KB, features 0-63 then 64-127 of the eight keys, 128-byte swizzle.  Keys of a
 // page are consecutive in it, so a page of any size is ONE copy (issuing a copy costs a producer lane over 100 clk; with the
 // two 64-feature slabs 16 KB apart a page under 128 tokens took two).  256 decode rows over pages of 16
@@ -126,7 +297,9 @@ __device__ __noinline__ void ws_packed_merge(void* out, float* lse_out, float* o
 constexpr int kGroupBytes = 2048, kHalfBytes = 1024;
 constexpr int kExactRows = 8;                 // keys per copy of the exact map
 
-template <bool kVWarp>
+// kQuarters: for launches that are not cut, of up to kQuarterHeads q-heads a kv-head (an instantiation of its own: cut launches of decode rows
+// lose 1 % to the registers and the size of the code)
+template <bool kVWarp, bool kQuarters>
 __global__ void __launch_bounds__(kWsThreads, 1)
 attn128_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_qs, const __grid_constant__ CUtensorMap tm_q1,
                   const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
@@ -149,24 +322,24 @@ attn128_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
     const uint32_t bar_item_empty = sBar + 16;   // [2]
     const uint32_t bar_q_full = sBar + 32;
     const uint32_t bar_q_empty = sBar + 40;
-    const uint32_t bar_s_full = sBar + 48;       // [2]
-    const uint32_t bar_p_full = sBar + 64;       // [2]
-    const uint32_t bar_o_full = sBar + 80;       // [2]
+    const uint32_t bar_s_full = sBar + kWsBarS;       // [2]
+    const uint32_t bar_p_full = sBar + kWsBarP;       // [2]
+    const uint32_t bar_o_full = sBar + kWsBarO;       // [2]
     // Two slots used alternately: the producer can fix up the V tile of the next short item before the MMA thread has
     // looked at the barrier for this one (slot k & 1 for the k-th such tile, 24 bytes apart).
-    const uint32_t bar_vfix = sBar + 96;
+    const uint32_t bar_vfix = sBar + 96;         // (and + 120; kWsBarJoin is between)
     // [3][2] early hand-overs of P: part c (the key columns up to 32 (c + 1)) of tile t is in place.  One barrier per part:
     // the MMA thread may look at part 0 only after part 1 has arrived too, which a shared barrier could not tell apart.
-    const uint32_t bar_p_part = sBar + 208;
+    const uint32_t bar_p_part = sBar + kWsBarPart;
     const uint32_t bar_kv_full = sBar + 128;     // [kWsStages]
     const uint32_t bar_kv_empty = sBar + 128 + 8 * kWsStages;
-    const uint32_t bar_x1 = sBar + 128 + 16 * kWsStages;       // packed item: group 1 has published its (m, l) per row
-    const uint32_t bar_x0 = sBar + 128 + 16 * kWsStages + 8;   // packed item: group 0 has merged, tile 1 may be reused
+    const uint32_t bar_x1 = sBar + kWsBarX1;       // packed item: group 1 has published its (m, l) per row
+    const uint32_t bar_x0 = sBar + kWsBarX0;       // packed item: group 0 has merged, tile 1 may be reused
     uint8_t* gen_bar = gen_base + (2 + kWsStages) * kTileBytes;
-    volatile int* s_abort = reinterpret_cast<volatile int*>(gen_bar + 512);
+    volatile int* s_abort = reinterpret_cast<volatile int*>(gen_bar + kWsAbort);
     volatile uint32_t* s_tmem = reinterpret_cast<volatile uint32_t*>(gen_bar + 516);
     WsItem* ring = reinterpret_cast<WsItem*>(gen_bar + 576);  // 2 x 48 bytes
-    float* xm = reinterpret_cast<float*>(gen_bar + 1024);     // [2][128]: running maximum and row sum of tile 1 (packed items)
+    float* xm = reinterpret_cast<float*>(gen_bar + kWsXm);     // [2][128]: running maximum and row sum of tile 1 (packed items)
 
     const int tid = threadIdx.x;
     const int warp = tid >> 5;
@@ -186,6 +359,7 @@ attn128_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
         mbar_init(bar_vfix, 1);
         mbar_init(bar_vfix + 24, 1);
         mbar_init(bar_x1, 4);
+        mbar_init(sBar + kWsBarJoin, 4);
         mbar_init(bar_x0, 4);
         for (int i = 0; i < kWsStages; ++i) {
             mbar_init(bar_kv_full + 8 * i, 1);
@@ -339,9 +513,13 @@ attn128_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                     if (ok && packed) {
                         const bool one = (u.rows & 0xffff) == 1;
                         const CUtensorMap* tm = one ? &tm_q1 : &tm_qs;
-                        mbar_arrive_expect_tx(bar_q_full, 2 * p.short_group * (one ? 1 : p.short_tokens) * 128);
-                        tma_load_3d(sQ, tm, bar_q_full, 0, h0, u.q_row0);
-                        tma_load_3d(sQ + kSlabBytes, tm, bar_q_full, 64, h0, u.q_row0);
+                        const int copies = kQuarters && one ? 4 : 1;     // (one for the lanes of each softmax warp)
+                        mbar_arrive_expect_tx(bar_q_full, copies * 2 * p.short_group * (one ? 1 : p.short_tokens) * 128);
+#pragma unroll 1
+                        for (int i = 0; i < copies; ++i) {
+                            tma_load_3d(sQ + i * 4096, tm, bar_q_full, 0, h0, u.q_row0);
+                            tma_load_3d(sQ + i * 4096 + kSlabBytes, tm, bar_q_full, 64, h0, u.q_row0);
+                        }
                     } else if (ok) {
                         mbar_arrive_expect_tx(bar_q_full, 4 * p.group * p.tile_tokens * 128);
 #pragma unroll
@@ -741,7 +919,7 @@ attn128_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                 const float inv_l = 1.f / l_run;
                 const bool live = row < tile_rows;
                 // whole runs of 128 bytes: 64 bf16 or 32 fp32 columns of the warp's 32 rows at a time
-                uint8_t* const stage = gen_bar + 2048 + (warp - 4) * 4096;
+                uint8_t* const stage = gen_bar + kWsStage + (warp - 4) * 4096;
                 const int warp_row0 = (warp & 3) * 32;
                 if (u.split < 0) {
 #pragma unroll 1
@@ -796,6 +974,17 @@ attn128_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
             tc_fence_before();
             return true;
             };
+            if (kQuarters && packed && u.rows == 1) {
+                const long long row0 = static_cast<long long>(u.q_row0) * p.num_q_heads + ring_h0;
+                if (!ws_run_quarters(static_cast<uint8_t*>(p.out) + row0 * 256, p.lse ? p.lse + row0 : nullptr, u.kv_end, u.pos0, grp, sc, sBar, gen_bar, tmem_base,
+                                     s_it, o_it, x_it))
+                    break;
+                const int n = (u.kv_end + 1 - t) >> 1;      // tiles of this group
+                s_it += n;
+                o_it += n > 0 ? 1 : 0;
+                ++x_it;
+                continue;
+            }
             if (!(packed ? run_item(std::true_type{}) : run_item(std::false_type{}))) break;
         }
     }
