@@ -128,6 +128,7 @@ __device__ __noinline__ void ws_packed_merge(void* out, float* lse_out, float* o
 // result the sum of eight, joined by group 0: every warp weighs its two and leaves them in the stage, all sum.
 // A tile's softmax is a third as long, so that what ends an item hides behind the copies of the next: 256 decode rows of 64/8 heads, contexts to
 // 8192 tokens, 578 -> 567 us.  What bounds it is the memory (6 TB/s while tiles stream).
+// (Against 64 bits, 40 to 200 rows: results 2.16 - 2.21e-3 off before, 2.06 - 2.13e-3 now, log-sum-exps 3.5e-7 and 3.6e-7.)
 constexpr int kQuarterHeads = 16;             // rows of 512 bytes in a warp's 8 KB of the stage
 static_assert(4 * kQuarterHeads * 512 <= kWsStageBytes, "the stage of both groups");
 // dst: row of the item's first head; lse: its log-sum-exp, or null; area: the CTA's barriers, xm and stage
