@@ -123,8 +123,9 @@ __device__ __noinline__ void ws_packed_merge(void* out, float* lse_out, float* o
 }
 
 // Whole items of one token and up to kQuarterHeads q-heads (decode rows that are not cut): the item's rows stand in Q four times, once in the 32 lanes of
-// each softmax warp, and the warps share out the 128 keys of a tile -- 32 each, an online softmax of its own, the P of the others' keys
-// zero -- where one warp would take them all and the others idle.  Tile t's O is then the sum of four over the lanes, and an item's
+// each softmax warp, and the warps share out the 128 keys of a tile -- 32 each, an online softmax of its own -- where one warp would take
+// them all and the others idle.  The MMAs of a warp's keys write that warp's lanes of O only (zero weights for the others' would do as well
+// but for infinite values, 0 * inf).  Tile t's O is then the sum of four over the lanes, and an item's
 // result the sum of eight, joined by group 0: every warp weighs its two and leaves them in the stage, all sum.
 // A tile's softmax is a third as long, so that what ends an item hides behind the copies of the next: 256 decode rows of 64/8 heads, contexts to
 // 8192 tokens, 578 -> 567 us.  What bounds it is the memory (6 TB/s while tiles stream).
@@ -248,11 +249,7 @@ __device__ __noinline__ bool ws_run_quarters(uint8_t* dst, float* lse, int kv_en
         }
         const float m_use = (m_ref == -INFINITY) ? 0.f : m_ref;
         float sum0 = 0.f, sum1 = 0.f;
-        uint32_t pk[16];
-#pragma unroll
-        for (int i = 0; i < 16; ++i) pk[i] = 0;
-#pragma unroll
-        for (int k = 1; k < 4; ++k) tmem_st16(tS + ((wq + k) & 3) * 16, pk);
+        uint32_t pk[16];     // (the columns of the other warps' keys stay as they are: the MMAs of those keys leave these lanes of O alone)
 #pragma unroll
         for (int i = 0; i < 32; i += 2) {
             const float p0 = ex2(fmaf(__uint_as_float(s[i]), sc, -m_use)), p1 = ex2(fmaf(__uint_as_float(s[i + 1]), sc, -m_use));
@@ -590,29 +587,38 @@ attn128_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                     mma_ss_lhh(tS, q_lo + qoff, kHiQ, k_lo + koff, kHiKV, kIdescQK, k > 0);
                 }
             };
-            auto issue_pv = [&](uint32_t tO, uint32_t tP, uint32_t v_stage, bool first, int k0, int k1) {
+            // (quarter: the 16 keys of a step go to the lanes of the warp whose keys they are, and to no others)
+            auto issue_pv = [&](uint32_t tO, uint32_t tP, uint32_t v_stage, bool first, int k0, int k1, bool quarter) {
                 const uint32_t v_lo = desc_lo_sw128(v_stage, kHalfBytes);
 #pragma unroll
                 for (int k = k0; k < k1; ++k) {
-                    mma_ts_lh(tO, tP + k * 8, v_lo + k * (2 * kGroupBytes >> 4), kHiKV, kIdescPV, (!first || k > 0) ? 1u : 0u);
+                    const uint32_t a = tP + k * 8, b_lo = v_lo + k * (2 * kGroupBytes >> 4);
+                    if constexpr (kQuarters) {
+                        const uint32_t off = quarter ? 0xffffffffu : 0u;
+                        const int w = k >> 1;
+                        mma_ts_lh_lanes(tO, a, b_lo, kHiKV, kIdescPV, (!first || (quarter ? (k & 1) : k) > 0) ? 1u : 0u,
+                                        w == 0 ? 0u : off, w == 1 ? 0u : off, w == 2 ? 0u : off, w == 3 ? 0u : off);
+                    } else {
+                        mma_ts_lh(tO, a, b_lo, kHiKV, kIdescPV, (!first || k > 0) ? 1u : 0u);
+                    }
                 }
             };
             // O_t += P_t V for one KV tile, following the hand-overs: every early part as soon as it is there, the rest after
             // the whole of P.  pit = hand-overs of P_t seen so far (tile visits).
-            auto pv_tile = [&](int t, uint32_t tO, uint32_t tS, uint32_t v_stage, bool first, uint32_t pit, int where) -> bool {
+            auto pv_tile = [&](int t, uint32_t tO, uint32_t tS, uint32_t v_stage, bool first, uint32_t pit, int where, bool quarter) -> bool {
                 int k0 = 0;
 #pragma unroll
                 for (int c = 0; c < 3; ++c) {
                     if ((kPartMask >> c) & 1) {
                         if (!wait1(bar_p_part + 16 * c + 8 * t, pit & 1, where)) return false;
                         tc_fence_after();
-                        issue_pv(tO, tS, v_stage, first, k0, 2 * (c + 1));
+                        issue_pv(tO, tS, v_stage, first, k0, 2 * (c + 1), quarter);
                         k0 = 2 * (c + 1);
                     }
                 }
                 if (!wait1(bar_p_full + 8 * t, pit & 1, where + 1)) return false;
                 tc_fence_after();
-                issue_pv(tO, tS, v_stage, first, k0, 8);
+                issue_pv(tO, tS, v_stage, first, k0, 8, quarter);
                 return true;
             };
             while (true) {
@@ -660,7 +666,7 @@ attn128_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                             ++vfix_it;
                         }
                         const uint32_t tO = t ? tO1 : tO0, tS = t ? tS1 : tS0;
-                        ok = pv_tile(t, tO, tS, sKV + st * kTileBytes, jj < 2, pit, 324);
+                        ok = pv_tile(t, tO, tS, sKV + st * kTileBytes, jj < 2, pit, 324, kQuarters && u.rows == 1);
                         if (!ok) break;
                         tc_commit(bar_kv_empty + 8 * st);
                         if (t) ++p_it1; else ++p_it;
@@ -699,7 +705,7 @@ attn128_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                     const bool has_next = jj + 1 < n;
                     stK = kv_it % kWsStages;
                     // ---- tile 0 ----
-                    ok = pv_tile(0, tO0, tS0, sKV + stV * kTileBytes, jj == 0, p_it, 308);
+                    ok = pv_tile(0, tO0, tS0, sKV + stV * kTileBytes, jj == 0, p_it, 308, false);
                     if (!ok) break;
                     if (has_next) {
                         ok = wait1(bar_kv_full + 8 * stK, (kv_it / kWsStages) & 1, 307);
@@ -713,7 +719,7 @@ attn128_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                         tc_commit(bar_o_full);
                     }
                     // ---- tile 1 ----
-                    ok = pv_tile(1, tO1, tS1, sKV + stV * kTileBytes, jj == 0, p_it1, 312);
+                    ok = pv_tile(1, tO1, tS1, sKV + stV * kTileBytes, jj == 0, p_it1, 312, false);
                     if (!ok) break;
                     if (lane == 0) {
                         tc_commit(bar_kv_empty + 8 * stV);

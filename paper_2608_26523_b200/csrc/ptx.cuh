@@ -162,6 +162,18 @@ __device__ __forceinline__ void mma_ts_lh(uint32_t d_tmem, uint32_t a_tmem, uint
         : "memory");
 }
 
+// the same for the warps whose word of `off` is 0 only (word w: lanes 32 w .. 32 w + 31 of D; a set bit keeps the lane as it is)
+__device__ __forceinline__ void mma_ts_lh_lanes(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t hi, uint32_t idesc,
+                                                uint32_t accumulate, uint32_t off0, uint32_t off1, uint32_t off2, uint32_t off3) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .b64 db;\n\t"
+        "setp.ne.b32 p, %5, 0;\n\t"
+        "mov.b64 db, {%2, %3};\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], db, %4, {%6, %7, %8, %9}, p;\n\t}" ::"r"(d_tmem),
+        "r"(a_tmem), "r"(b_lo), "r"(hi), "r"(idesc), "r"(accumulate), "r"(off0), "r"(off1), "r"(off2), "r"(off3)
+        : "memory");
+}
+
 // TMEM <-> registers, shape 32x32b: thread t of warp w touches lane 32*(w%4)+t, 32 consecutive columns.
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
     asm volatile(
