@@ -152,10 +152,10 @@ __device__ __forceinline__ bool ws_quarter_join(uint8_t* dst, float* lse, bool s
     for (int k = 0; k < 4; ++k) M = fmaxf(M, xm[k * 32 + lane]);
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-        const float mk = xm[k * 32 + lane];
-        if (mk != -INFINITY) L = fmaf(ex2(mk - M), xm[128 + k * 32 + lane], L);
+        const float mk = xm[k * 32 + lane];     // (-inf: no key of its own, or scores of NaN, whose sum is NaN and must stay so)
+        L = fmaf(mk == -INFINITY ? 0.f : ex2(mk - M), xm[128 + k * 32 + lane], L);
     }
-    const float f = m == -INFINITY ? 0.f : ex2(m - M) / L;
+    const float f = (m == -INFINITY ? 0.f : ex2(m - M)) / L;     // (all scores -inf: 0 / 0, as the definition has it)
     const float s0 = a0 * f, s1 = a1 * f;
     uint8_t* const mine = stage + w * (kQuarterHeads * 512) + lane * 512;
 #pragma unroll 1

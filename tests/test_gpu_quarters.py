@@ -1,5 +1,5 @@
 """Decode rows whose heads' softmax is shared out over the warps by keys, 32 of a tile each: contexts on both sides of those edges,
-one tile, two and several, group sizes up to the limit and beyond it, parts of rows, references that grow in one warp alone, and infinite values."""
+one tile, two and several, group sizes up to the limit and beyond it, parts of rows, references that grow in one warp alone, values and scores that are not finite."""
 import numpy as np
 import pytest
 
@@ -55,3 +55,27 @@ def test_infinite_values(heads):
     np.testing.assert_array_equal(got_o[~fin], ref_o[~fin])
     assert np.abs(got_o[fin] - ref_o[fin]).max() <= ABS_TOL      # (values of N(0, 1): averages stay below 4)
     assert (np.abs(got_l - ref_l) / np.maximum(1.0, np.abs(ref_l))).max() <= LSE_TOL
+
+
+@pytest.mark.parametrize("ctx", [20, 100, 128, 250, 600])
+def test_scores_that_are_no_numbers(ctx):
+    """A row with a key of NaN has no result, wherever the key is and however many of its neighbours are NaN too; nor has a row
+    whose scores are all -inf.  Rows beside them keep theirs."""
+    nan, ninf = float("nan"), float("-inf")
+    spans = [(0, ctx), (0, 1), (ctx - 1, ctx), (0, min(32, ctx)), (ctx // 2, ctx), (ctx // 128 * 128, ctx // 128 * 128 + min(ctx % 128, 32))]
+    prob = _edge_problem([ctx] * (len(spans) + 2), 8, 1)
+    bad = [r for r, (a, b) in enumerate(spans) if b > a]
+    for r in bad:
+        for pos in range(*spans[r]):
+            prob.k_cache[_slot(prob, r, pos)] = nan
+    no_scores = len(spans)
+    prob.q[no_scores, :, 5] = 1.0
+    for pos in range(ctx):
+        prob.k_cache[_slot(prob, no_scores, pos) + (0, 5)] = ninf
+    out, lse, _ = run_gpu(prob.to("cuda"), 1)
+    out, lse = out.cpu(), lse.cpu()
+    assert out[bad].isnan().all() and lse[bad].isnan().all()
+    assert out[no_scores].isnan().all() and (lse[no_scores] == ninf).all()
+    rows = oracle.all_rows(prob.chunk_len.numpy(), 8)
+    rest = [r for r in range(len(spans) + 2) if r not in bad and r != no_scores]
+    print(compare(out, lse, prob, rows[np.isin(rows[:, 0], rest)], "rows beside them"))
