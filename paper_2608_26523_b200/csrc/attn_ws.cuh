@@ -198,9 +198,10 @@ __device__ __forceinline__ bool ws_quarter_join(uint8_t* dst, float* lse, bool s
 }
 
 // Softmax of one item of quarters, by a warp of group t: 32 of the keys of every second tile, then the join.
-// (out of line, like the join of packed items: the prefill path keeps its registers)
-__device__ __noinline__ bool ws_run_quarters(uint8_t* dst, float* lse, int kv_end, int pos, int heads, float sc, uint32_t sBar,
-                                             uint8_t* area, uint32_t tmem_base, uint32_t s_it, uint32_t o_it, uint32_t x_it) {
+// (in line: out of line, the twelve arguments and what lives across the call cost a stack frame and 52 bytes of spills; the other
+// instantiations of the kernel do not have it)
+__device__ __forceinline__ bool ws_run_quarters(uint8_t* dst, float* lse, int kv_end, int pos, int heads, float sc, uint32_t sBar,
+                                                uint8_t* area, uint32_t tmem_base, uint32_t s_it, uint32_t o_it, uint32_t x_it) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, t = (warp - 4) >> 2, wq = warp & 3, row = threadIdx.x & 127;
     const uint32_t lane_off = static_cast<uint32_t>(wq * 32) << 16, tS = tmem_base + t * 128 + lane_off, tO = tmem_base + 256 + t * 128 + lane_off;
     volatile int* const s_abort = reinterpret_cast<volatile int*>(area + kWsAbort);
