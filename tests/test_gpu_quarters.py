@@ -1,7 +1,11 @@
 """Decode rows whose heads' softmax is shared out over the warps by keys, 32 of a tile each: contexts on both sides of those edges,
-one tile, two and several, group sizes up to the limit and beyond it, parts of rows, references that grow in one warp alone, values and scores that are not finite."""
+one tile, two and several, group sizes up to the limit and beyond it, parts of rows, references that grow in one warp alone, many items
+on an SM and items of other kinds between them, values and scores that are not finite."""
+import math
+
 import numpy as np
 import pytest
+import torch
 
 import oracle
 from paper_2608_26523_b200 import workloads as W
@@ -20,7 +24,8 @@ def test_contexts_around_the_edges_of_quarters(heads, splits):
 
 
 def test_a_reference_that_grows_late_in_one_quarter():
-    """Rescales of O in one warp while the others' references stand: keys whose scores rise by far, in different quarters and tiles."""
+    """References that rise by far, so that each outweighs all before it: the weights at the join.  (What was summed before they grow
+    does not show in this result: test_what_was_summed_before_a_reference_grows.)"""
     prob = W.make_problem(8990, [639], [1], 8, 1, 128, 128, block_size=64, std=0.1)
     for i, pos in enumerate((5, 200, 330, 470, 601, 639)):
         prob.k_cache[int(prob.block_table[0, pos // 64]), pos % 64, 0] = prob.q[0, 0] * (40.0 * (i + 1))
@@ -79,3 +84,64 @@ def test_scores_that_are_no_numbers(ctx):
     rows = oracle.all_rows(prob.chunk_len.numpy(), 8)
     rest = [r for r in range(len(spans) + 2) if r not in bad and r != no_scores]
     print(compare(out, lse, prob, rows[np.isin(rows[:, 0], rest)], "rows beside them"))
+
+
+@pytest.mark.parametrize("heads,rows", [((64, 8), 200), ((8, 1), 400), ((16, 1), 400), ((32, 32), 40)])
+def test_many_items_of_a_cta(heads, rows):
+    """Several items to an SM one after the other, of one tile, two, three and several, odd and even numbers, in the order of their
+    lengths and the ends of long and of one-tile items next to each other: every element."""
+    rng = np.random.default_rng(rows + heads[0])
+    ctx = rng.choice([1, 7, 31, 32, 33, 64, 100, 127, 128, 129, 200, 256, 257, 300, 384, 385, 400, 530], size=rows)
+    # (std 0.5: a result of few keys is off by half an ulp of its own and 2^-9 of the largest value, whose weight is rounded: below 2 that
+    # is 3.9e-3 + 4.5e-3 at most, under the tolerance of 1e-2; values of N(0, 1) reach 4.5, and 1.05e-2)
+    prob = W.make_problem(9040 + heads[0], [int(c) - 1 for c in ctx], [1] * rows, heads[0], heads[1], 128, 128, block_size=16, std=0.5)
+    out, lse, _ = run_gpu(prob.to("cuda"), 1)
+    print(compare(out, lse, prob, oracle.all_rows(prob.chunk_len.numpy(), heads[0]), "many items"))
+
+
+@pytest.mark.parametrize("heads", [(64, 8), (16, 1), (32, 32)])
+def test_items_of_every_kind_on_a_cta(heads):
+    """More requests than tokens: rows of one token between units of a few tokens and of several hundred, which share barriers, the
+    stage and the exchange area with them."""
+    rng = np.random.default_rng(heads[0])
+    chunk = [0] * 900 + [1] * 150 + [2, 3, 5, 8, 16] * 4 + [300, 130]
+    if heads[0] == heads[1]:
+        chunk = [0] * 700 + [1] * 40 + [2, 100, 128, 300]
+    assert sum(chunk) <= len(chunk)
+    order = rng.permutation(len(chunk))
+    chunk = [chunk[i] for i in order]
+    prefix = [int(rng.choice([0, 1, 30, 100, 127, 128, 250, 400])) if c else 0 for c in chunk]
+    # (std 0.5: see above)
+    prob = W.make_problem(9060 + heads[0], prefix, chunk, heads[0], heads[1], 128, 128, block_size=16, std=0.5)
+    out, lse, _ = run_gpu(prob.to("cuda"), 1)
+    print(compare(out, lse, prob, oracle.all_rows(prob.chunk_len.numpy(), heads[0]), "mixed kinds"))
+
+
+def growing_problem(levels):
+    """Scores by design: head h sees every key at log2 weight 0 but for one key of the last tiles, in the tile parity and quarter
+    of h, which is `levels[h]` above.  The earlier keys of each quarter and parity, as many as 2^9 together, have values of their
+    own about 1, so that what a warp held before its reference grew is a tenth of the result."""
+    n_heads, tiles = len(levels), 32
+    prob = W.make_problem(9080, [tiles * 128 - 1], [1], n_heads, 1, 128, 128, block_size=128, std=0.1)
+    gen = torch.Generator().manual_seed(9081)
+    base = torch.randn((2, 4, 128), generator=gen)
+    pos = torch.arange(tiles * 128)
+    part = base[pos // 128 % 2, pos // 32 % 4]
+    k = torch.zeros((tiles * 128, 128))
+    v = part + 0.1 * torch.randn((tiles * 128, 128), generator=gen)
+    prob.q.zero_()
+    for h, level in enumerate(levels):
+        prob.q[0, h, h] = 8.0
+        late = (tiles - 2 + (h >> 2 & 1)) * 128 + (h & 3) * 32 + 5 + h
+        k[late, h] = level * math.log(2.0) / (8.0 * prob.scale)
+    table = prob.block_table[0].long()
+    prob.k_cache[table, :, 0] = k.view(tiles, 128, 128).to(torch.bfloat16)
+    prob.v_cache[table, :, 0] = v.view(tiles, 128, 128).to(torch.bfloat16)
+    return prob
+
+
+def test_what_was_summed_before_a_reference_grows():
+    """Rescales of a warp's O and sum that the result shows: in every quarter of both tile parities, by different factors."""
+    prob = growing_problem([8.5, 9.0, 9.5, 10.0, 8.6, 9.2, 9.8, 10.4, 9.4, 8.8, 10.2, 9.6, 9.1, 9.9, 8.7, 9.3])
+    out, lse, _ = run_gpu(prob.to("cuda"), 1)
+    print(compare(out, lse, prob, oracle.all_rows(prob.chunk_len.numpy(), 16), "rescaled"))
