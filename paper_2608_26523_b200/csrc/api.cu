@@ -373,6 +373,20 @@ constexpr int kMinLen = 2, kMinShortLen = 4;   // fewest KV tiles worth a work i
 // other way round 60 rows and 4000 tokens 1351 and 1384, a chunk by itself 1 to 2 %.
 bool v_producer(const vpp_chunk_attn_args* a) { return a->total_q <= (a->num_reqs > 1 ? 64ll * a->num_reqs : 1); }
 
+// Does the d = 128 kernel share out the keys of a decode row's tiles over the softmax warps (attn_ws.cuh)?  Its items end later (the join of
+// eight results) and hand the SM to the next one earlier, so it pays where an SM runs several, one after the other, and not where
+// each has one; groups of more heads have a longer join.  Uncut rows of the same batch packed and shared out, us, contexts to 8192 / to 512 / of 128
+// tokens: 8 rows of 64/8 heads (64 items) 75.3 and 76.8 / 17.5 and 17.9 / 12.7 both; 24 of 32/8 (192) 83.7 and 84.5 / 19.9 and 20.1 / 17.9
+// and 17.1; 40 of 32/8 (320) 134.6 and 134.2 / 27.6 and 27.4 / 23.9 and 22.7; 300 of 64/8 to 512 126.7 and 117.8; 256 to 8192 765 and 748.  Groups of
+// 16: 64 rows of 64/4 (256) 106.2 and 106.6 / 23.8 and 24.5 / 24.4 and 24.3; 96 (384) 150.6 both / 30.8 and 31.2 / 26.5 and 25.4;
+// 149 (596) 216.9 and 214.9 / 41.8 and 40.8 / 31.6 and 31.0.
+// (Which of more requests than tokens are decode rows only the device knows: a chunk of 1500 tokens among 2000 empty requests takes 70.8 us so, 69.2
+// otherwise; 256 rows among 768 empty ones 219 and 231.)
+bool shares_out_keys(const vpp_chunk_attn_args* a, int short_group) {
+    const long long items = static_cast<long long>(a->total_q) * (a->num_q_heads / short_group);
+    return a->total_q <= a->num_reqs && short_group <= vpp::kQuarterHeads && items >= (short_group <= 8 ? 2ll : 3ll) * sm_count_or_default();
+}
+
 // Time of a KV tile of a work item, measured at full clock.
 struct TileTimes {
     double unit_us, short_us;
@@ -801,9 +815,7 @@ vpp_status run_chunk_attn(const vpp_chunk_attn_args* a, vpp_stream_t stream_, co
             ce = launch(kern, static_cast<unsigned>((sms / 2) * 2), vpp::kMla2Threads, vpp::kMla2SmemBytes, stream, tm_q9, tm_qh9, tm_k93,
                         tm_k92, ap, box_rows);
     } else {
-        // Batches of decode rows that are not cut: their softmax is shared out over the warps (attn_ws.cuh).  256 rows of 64/8 heads 578 -> 567 us;
-        // rows that are cut lose 1 % to the longer join (8 rows 43.3 -> 43.8), and items of several tokens registers.
-        const bool quarters = a->total_q <= a->num_reqs && L.splits == 1 && !range && rp.short_group <= vpp::kQuarterHeads;
+        const bool quarters = L.splits == 1 && !range && shares_out_keys(a, rp.short_group);
         auto kern = !v_producer(a) ? vpp::attn128_ws_kernel<false, false> : quarters ? vpp::attn128_ws_kernel<true, true> : vpp::attn128_ws_kernel<true, false>;
         ce = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, vpp::kWsSmemBytes);
         if (ce == cudaSuccess)
