@@ -614,9 +614,10 @@ dsa_attn_kernel(const __grid_constant__ CUtensorMap tm_qh, const __grid_constant
                     });
                 }
             } else {
-                // Two steps of 32 columns a turn: the second's columns come from tensor memory while the stage is emptied of the first's.  Each load
-                // is waited for in straight line and with its registers: nothing may copy them before, as the back edge of a loop could.
-                // (16 tokens with lists of 2048: 35.4 us a step, 35.2 with the load carried round the loop, 35.6 unrolled whole)
+                // Four steps of 32 columns a turn: while the stage is emptied of one, the next one's columns come from tensor memory.  Each load is
+                // waited for in straight line and with its registers: nothing may copy them before, as the back edge of a loop could.
+                // (16 tokens with lists of 2048: 35.2 us a step; 35.0 with a load carried round the loop, 35.3 with no load under a flush or
+                // two steps a turn, 35.5 unrolled whole: the code of an epilogue comes from far away)
                 const StageRows to = stage_rows(lane, [&](int i) -> uint8_t* {
                     return i < warp_rows ? reinterpret_cast<uint8_t*>(p.o_parts + (first_row + i) * kMlaDv + half * 128) : nullptr;
                 });
@@ -628,18 +629,17 @@ dsa_attn_kernel(const __grid_constant__ CUtensorMap tm_qh, const __grid_constant
                                              __float_as_uint(__uint_as_float(v[q4 * 4 + 2]) * inv_l), __float_as_uint(__uint_as_float(v[q4 * 4 + 3]) * inv_l)));
                 };
 #pragma unroll 1
-                for (int c = 0; c < 8; c += 2) {     // 32 fp32 columns of 32 rows at a time
-                    const uint32_t tO = (c < 4 ? tO0 : tO1) + (c & 3) * 32;
-                    const int bytes = (c >> 2) * 1024 + (c & 3) * 128;
-                    uint32_t r[32], r1[32];
-                    tmem_ld32(tO, r);
-                    tc_wait_ld(r);
-                    put(r);
-                    tmem_ld32(tO + 32, r1);
-                    stage_flush(stage, lane, to, bytes);
-                    tc_wait_ld(r1);
-                    put(r1);
-                    stage_flush(stage, lane, to, bytes + 128);
+                for (int c = 0; c < 2; ++c) {     // 128 fp32 columns, 32 at a time, of 32 rows
+                    const uint32_t tO = c == 0 ? tO0 : tO1;
+                    uint32_t r[4][32];
+                    tmem_ld32(tO, r[0]);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        tc_wait_ld(r[i]);
+                        put(r[i]);
+                        if (i < 3) tmem_ld32(tO + 32 * (i + 1), r[i + 1]);
+                        stage_flush(stage, lane, to, c * 1024 + i * 128);
+                    }
                 }
             }
             if (live && half == 0) {
