@@ -7,13 +7,14 @@
 // MMA, softmax and barrier structure is taken.  What differs is the producer side: a KV tile is 128 listed rows that
 // lie anywhere in the cache, fetched with the gather form of the tensor copy (cp.async.bulk.tensor ... tile::gather4:
 // four rows of 64 columns per instruction, 128-byte swizzle applied on the way in).  What bounds the kernel is the rate at
-// which these copies are issued: a warp issues them one lane after the other at ~180 clk apiece, warps issue independently,
-// an SM sustains one per ~10 clk.  A tile and CTA takes 272 (K: 64 keys x 9 slabs, V: 128 keys x 4 slabs, four rows each),
+// which these copies are issued: a warp issues them one lane after the other, 113 clk apiece (up to 180 when all warps issue), warps issue
+// independently, and an SM sustains one per 10 to 16 clk alone, one per 19 beside the MMAs.  A tile and CTA takes 272 (K: 64 keys x 9 slabs, V: 128 keys x 4 slabs, four rows each),
 // so they are spread over 17 producer warps of 16 lanes, one slab of 64 keys each, and the register file is split
 // unevenly (setmaxnreg) to make room for them.  2048 tokens with lists of
 // 2048 at prefix 65536: 10 producer warps of 24 and 32 lanes 1458 us, these 1362 us.
 // A launch of few tokens (a decode batch) would leave most pairs idle for the 16 tiles of a 2048-entry list: then a token's
-// list is cut into `splits` parts, an item each, whose partial results lse_merge_small_kernel joins (16 tokens: 62.6 -> 38.2 us for the step, 36.8 -> 35.4 with a shorter store of the partial results).
+// list is cut into `splits` parts, an item each, whose partial results lse_merge_small_kernel joins (16 tokens: 62.6 -> 38.2 us for the step;
+// 36.7 -> 35.2 since partial results are stored with less waiting).
 // Entries that do not take part are pointed at the token's own cache row (always present and finite) and masked out
 // of the softmax through a 128-bit validity mask that warp 0 publishes per tile.  The cost per token does not depend on
 // the prefix length: the flat latency curve the paper says weakens its linear-growth assumption.
@@ -289,7 +290,8 @@ dsa_attn_kernel(const __grid_constant__ CUtensorMap tm_qh, const __grid_constant
             int t, j0, j1;
             part_of(item, t, j0, j1);
             int e_next[4];
-            if (kParts) load_entries(t, j0, key0, e_next);   // (beside the token's look-up; longer items have time for it after: 2048 tokens are 2 % slower so)
+            // (beside the token's look-up: 0.1 us of 35 for 16 tokens; longer items have time for it after, 2048 tokens are 2 % slower so)
+            if (kParts) load_entries(t, j0, key0, e_next);
             const int2 tk = __ldg(p.tok + t);
             if (tk.x < 0) continue;
             const int self_row = row_of(tk.x, tk.y);
@@ -338,7 +340,7 @@ dsa_attn_kernel(const __grid_constant__ CUtensorMap tm_qh, const __grid_constant
             int t, j0, j1;
             part_of(item, t, j0, j1);
             int e_next[4];
-            if (kParts) load_entries(t, j0, key0, e_next);   // (beside the token's look-up; longer items have time for it after: 2048 tokens are 2 % slower so)
+            if (kParts) load_entries(t, j0, key0, e_next);   // (as the key producers)
             const int2 tk = __ldg(p.tok + t);
             if (tk.x < 0) continue;
             const int self_row = row_of(tk.x, tk.y);
@@ -543,7 +545,7 @@ dsa_attn_kernel(const __grid_constant__ CUtensorMap tm_qh, const __grid_constant
                 }
                 const float m_use = (m_ref == -INFINITY) ? 0.f : m_ref;
                 uint32_t pk[32];
-                // (packed fma and three-input maxima: the softmax shares its issue slots with 17 warps of producers; 2048 tokens 1353 -> 1340 us)
+                // (packed fma and three-input maxima: the softmax shares its issue slots with 17 warps of producers; 2048 tokens 1298 -> 1284 us)
                 const uint64_t sc2 = pack_f32x2(sc, sc), neg_m2 = pack_f32x2(-m_use, -m_use);
                 float sum0 = 0.f, sum1 = 0.f;
 #pragma unroll
@@ -616,8 +618,8 @@ dsa_attn_kernel(const __grid_constant__ CUtensorMap tm_qh, const __grid_constant
             } else {
                 // Four steps of 32 columns a turn: while the stage is emptied of one, the next one's columns come from tensor memory.  Each load is
                 // waited for in straight line and with its registers: nothing may copy them before, as the back edge of a loop could.
-                // (16 tokens with lists of 2048: 35.2 us a step; 35.0 with a load carried round the loop, 35.3 with no load under a flush or
-                // two steps a turn, 35.5 unrolled whole: the code of an epilogue comes from far away)
+                // (16 tokens with lists of 2048: 35.16 us a step; 35.24 two steps a turn, 35.33 with no load under a flush, 35.5 unrolled whole -- the
+                // code of an epilogue comes from far away -- and 35.01 with a load carried round the loop)
                 const StageRows to = stage_rows(lane, [&](int i) -> uint8_t* {
                     return i < warp_rows ? reinterpret_cast<uint8_t*>(p.o_parts + (first_row + i) * kMlaDv + half * 128) : nullptr;
                 });

@@ -738,7 +738,7 @@ attn_mla2_kernel(const __grid_constant__ CUtensorMap tm_q1, const __grid_constan
                 const float m_use = (m_ref == -INFINITY) ? 0.f : m_ref;
                 uint32_t pk[32];
                 // (packed fma here, three-input maxima above: fewer instructions beside the MMAs, which the power limit turns into clocks;
-                //  2048 tokens of 128 heads at 32768 keys 15.66 -> 15.42 ms)
+                //  2048 tokens of 128 heads at 32768 keys 15.04 -> 14.87 ms, means of eight runs each in turn that differ by 1.5 % among themselves)
                 const uint64_t sc2 = pack_f32x2(sc, sc), neg_m2 = pack_f32x2(-m_use, -m_use);
                 float sum0 = 0.f, sum1 = 0.f;
 #pragma unroll

@@ -10,6 +10,7 @@
 //   warps 4-7   softmax group for tile 0: one query row per thread, fp32 online softmax on S_0 read
 //               from tensor memory, P_0 written back to tensor memory as bf16 over S_0.
 //   warps 8-11  the same for tile 1.
+// (Shared-out items, below, differ in that: there a row stands in a lane of each warp of a group.)
 // While one group works on its S tile the tensor core runs the other tile's MMAs.
 //
 // The rows of a tile are (token, q-head) pairs: `group` q-heads of one kv-head over `tile_tokens` consecutive tokens,
@@ -21,6 +22,8 @@
 // run "packed": both tiles of its item use that one Q tile and split the KV tiles between
 // them (even ones to tile 0, odd ones to tile 1) as two independent online softmaxes whose results softmax group 0
 // merges at the end -- one softmax chain per KV tile would leave the memory system idle most of the time.
+// In large batches of decode rows (kQuarters) a packed item of one token is "shared out" as well: each warp of a group has the item's rows
+// in its lanes and takes 32 of a tile's 128 keys, and group 0 joins eight results instead of two (ws_run_quarters).
 // Tensor memory: S_0 | S_1 | O_0 | O_1, 128 fp32 columns each (all 512 columns).
 //
 // The math per row is the paper's Eq. 1 with the causal rule, evaluated KV tile by KV tile with a
@@ -45,7 +48,7 @@ constexpr int kTileBytes = 2 * kSlabBytes;    // one 128 x 128 bf16 tile
 // (the two alternating slots of the V-tail barrier cover a producer that runs at most two V tiles ahead of the MMA thread:
 //  a ring of more than four stages would need more slots -- five stages failed parity on short items)
 static_assert(kWsStages <= 4, "V-tail barrier slots");
-constexpr int kWsStageBytes = 8 * 32 * 128;   // 4 KB per softmax warp for the epilogue's stores
+constexpr int kWsStageBytes = 8 * 32 * 128;   // 4 KB per softmax warp for the epilogue's stores (the join of shared-out items: 8 KB per warp of group 0)
 constexpr int kWsSmemBytes = 2 * kTileBytes + kWsStages * kTileBytes + 1024 /*align*/ + 2048 /*barriers, ring, merge exchange*/ + kWsStageBytes;
 static_assert(kWsSmemBytes <= 232448, "shared memory of one CTA");
 // (bytes from the first barrier)
@@ -127,8 +130,9 @@ __device__ __noinline__ void ws_packed_merge(void* out, float* lse_out, float* o
 // them all and the others idle.  The MMAs of a warp's keys write that warp's lanes of O only (zero weights for the others' would do as well
 // but for infinite values, 0 * inf).  Tile t's O is then the sum of four over the lanes, and an item's
 // result the sum of eight, joined by group 0: every warp weighs its two and leaves them in the stage, all sum.
-// A tile's softmax is a third as long, so that what ends an item hides behind the copies of the next: 256 decode rows of 64/8 heads, contexts to
-// 8192 tokens, 578 -> 567 us.  What bounds it is the memory (6 TB/s while tiles stream).
+// A warp has 32 exponentials a tile instead of 128, so that what ends an item hides behind the copies of the next: 256 decode rows of 64/8
+// heads, contexts to 8192 tokens, 802 us packed and 771 so (6.3 TB/s); all of 8192 tokens 1361 and 1322 us, which is 6.5 TB/s, the copy rate.  Where
+// contexts differ, the rest is the start of the launch and the SMs' unequal ends; what share each has is not measured.
 // (Against 64 bits, 40 to 200 rows: results 2.16 - 2.21e-3 off before, 2.06 - 2.13e-3 now, log-sum-exps 3.5e-7 and 3.6e-7.)
 constexpr int kQuarterHeads = 16;             // rows of 512 bytes in a warp's 8 KB of the stage
 static_assert(4 * kQuarterHeads * 512 <= kWsStageBytes, "the stage of both groups");
@@ -332,13 +336,15 @@ attn128_ws_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
     const uint32_t bar_p_part = sBar + kWsBarPart;
     const uint32_t bar_kv_full = sBar + 128;     // [kWsStages]
     const uint32_t bar_kv_empty = sBar + 128 + 8 * kWsStages;
-    const uint32_t bar_x1 = sBar + kWsBarX1;       // packed item: group 1 has published its (m, l) per row
-    const uint32_t bar_x0 = sBar + kWsBarX0;       // packed item: group 0 has merged, tile 1 may be reused
+    const uint32_t bar_x1 = sBar + kWsBarX1;       // packed item: group 1 has published its (m, l) per row (shared out: per lane)
+    const uint32_t bar_x0 = sBar + kWsBarX0;       // packed item: group 0 has merged, tile 1, xm and group 1's stage may be reused
+    // (kWsBarJoin, shared-out items: the warps of group 0 have published their own (m, l), then their weighed results: two phases an item)
     uint8_t* gen_bar = gen_base + (2 + kWsStages) * kTileBytes;
     volatile int* s_abort = reinterpret_cast<volatile int*>(gen_bar + kWsAbort);
     volatile uint32_t* s_tmem = reinterpret_cast<volatile uint32_t*>(gen_bar + 516);
     WsItem* ring = reinterpret_cast<WsItem*>(gen_bar + 576);  // 2 x 48 bytes
-    float* xm = reinterpret_cast<float*>(gen_bar + kWsXm);     // [2][128]: running maximum and row sum of tile 1 (packed items)
+    // [2][128]: running maximum and row sum of tile 1 (packed items); shared out, of each lane of tile 1, then of both tiles together
+    float* xm = reinterpret_cast<float*>(gen_bar + kWsXm);
 
     const int tid = threadIdx.x;
     const int warp = tid >> 5;
