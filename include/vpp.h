@@ -72,9 +72,10 @@ typedef void *vpp_stream_t; /* a cudaStream_t */
  *              the chunk's own K/V are written before this call.  Slots past that point inside a
  *              request's last block may hold anything (NaN included) and blocks the block table
  *              does not name are never read.
- *              A row that sees a key whose value is infinite or NaN gets what the definition gives.  Rows of the
- *              same chunk up to 255 positions before that key may get NaN in its features too (a masked
- *              key has weight 0, and 0 * inf is NaN); decode rows see every key, so none of theirs do.
+ *              A row that sees a key whose value is infinite or NaN gets what the definition gives, a weight
+ *              below 2^-126 of the largest counting as 0.  Rows of the same chunk up to 255 positions before
+ *              that key may get NaN in its features too (a masked key has weight 0, and 0 * inf is NaN);
+ *              decode rows see every key, so none of theirs do.
  * block_table  int32 [num_reqs, max_blocks_per_req]: physical block of logical block j of request r.
  *              NULL means contiguous: request r is "block" r and block_size is ignored (slot = token).
  *              Then EVERY request's region must really hold max_seq_len slots (the kernels fetch whole
